@@ -93,19 +93,22 @@ typedef struct rts_peel_config {
                            n_chan <= 960, else RTS_EINVAL), RTS_BLOCK_TCGEN05 (tcgen05.mma
                            with TMEM accumulators, TF32 with split operands; n_chan <= 768,
                            else RTS_EINVAL).  All give FP32-level accuracy. */
-  int32_t solve_kernel;  /* blocked peel only: RTS_SOLVE_AUTO (0: the corrected averages,
-                           ALS sweeps and model matrices of a whole block in one
-                           cooperative launch whose CTAs meet at grid-wide barriers, when
-                           the device supports cooperative launches and the rows of
-                           ceil(n_ant / n_SM) antennas fit in shared memory, about
-                           n_ant <= 900 on GB300; otherwise as RTS_SOLVE_LAUNCHES),
+  int32_t solve_kernel;  /* blocked peel only: RTS_SOLVE_AUTO (0: for n_ant <= 256 the
+                           chain of eight sources at a time in one thread-block cluster
+                           whose CTAs exchange iterates through distributed shared
+                           memory; above that the corrected averages, ALS sweeps and
+                           model matrices of a whole block in one cooperative launch
+                           whose CTAs meet at grid-wide barriers, when the device supports
+                           cooperative launches and the rows of ceil(n_ant / n_SM)
+                           antennas fit in shared memory, about n_ant <= 900 on GB300;
+                           otherwise as RTS_SOLVE_LAUNCHES),
                            RTS_SOLVE_LAUNCHES (1: one launch per ALS sweep, per
-                           correction and per model step).  The cooperative launch
-                           solves the 2x2 systems of the sweeps before the last in
-                           FP32 and the last in FP64, the per-step launches every
-                           sweep in FP64; both accumulate the normal equations'
-                           cross-thread sums in FP64, and their results agree to
-                           FP32 rounding (statuses outside a band around 1e-6). */
+                           correction and per model step).  The cluster and the
+                           cooperative launch solve the 2x2 systems of the sweeps before
+                           the last in FP32 and the last in FP64 (from float-float or
+                           FP64 sums), the per-step launches every sweep in FP64; their
+                           results agree to FP32 rounding (statuses outside a band
+                           around 1e-6). */
   int32_t grad_kernel;   /* RTS_PREC_MIXED adjoint (rts_peel_grad, rts_peel_offsets):
                            RTS_GRAD_AUTO (0: phasors factorised per 16-channel group into
                            two shared-memory tables, T1[q] T2[r], when the tables of all

@@ -12,4 +12,28 @@ __device__ inline void kahan_add(float& sum, float& comp, float x) {
   sum = t;
 }
 
+// An unevaluated sum hi + lo of two floats.  Adding two of them costs 8 FP32
+// instructions and keeps about 47 bits; an FP64 addition occupies a
+// sub-partition's FP64 pipe for 64 cycles a warp.
+struct FF { float hi, lo; };
+__device__ __forceinline__ FF ff_two_sum(float a, float b) {
+  FF r;
+  r.hi = __fadd_rn(a, b);
+  const float bb = __fsub_rn(r.hi, a);
+  r.lo = __fadd_rn(__fsub_rn(a, __fsub_rn(r.hi, bb)), __fsub_rn(b, bb));
+  return r;
+}
+__device__ __forceinline__ FF ff_add(FF a, FF b) {
+  FF r = ff_two_sum(a.hi, b.hi);
+  r.lo = __fadd_rn(r.lo, __fadd_rn(a.lo, b.lo));
+  return r;
+}
+// s + a b, the product exact
+__device__ __forceinline__ FF ff_fma(float a, float b, FF s) {
+  const float p = __fmul_rn(a, b), e = fmaf(a, b, -p);
+  FF r = ff_two_sum(s.hi, p);
+  r.lo = __fadd_rn(r.lo, __fadd_rn(s.lo, e));
+  return r;
+}
+
 }  // namespace rts

@@ -14,6 +14,7 @@
 #include "block_kernels.cuh"
 #include "block_tc05_kernels.cuh"
 #include "block_tc_kernels.cuh"
+#include "cluster_solve_kernels.cuh"
 #include "common.cuh"
 #include "grad_kernels.cuh"
 #include "offset_kernels.cuh"
@@ -85,6 +86,11 @@ struct rts_peel_t {
   bool bs_ok = false;              // set up and fits (shared memory, cooperative launch)
   int bs_grid = 0, bs_apc = 0;
   size_t bs_smem = 0;
+  // solve of small arrays by one cluster per group of sources (k_cluster_solve)
+  int cl_size = 0, cl_apc = 0;     // CTAs (0: not used), antenna slots of each
+  size_t cl_smem = 0;
+  float4* cl_V = nullptr;          // [kClGroup][n_ant][2][n_ant] a group's corrected averages
+  float2* cl_D = nullptr;          // [kClPairs][n_ant][n_ant] its own D_jq
   unsigned* b_sync = nullptr;      // [2] barrier counter, abort flag
   double* b_part = nullptr;        // [BK][n_ant][4] per-antenna convergence sums of the last sweep
   cudaStream_t b_main = nullptr;   // high-priority stream for passes, corrections and solves
@@ -364,8 +370,12 @@ int ensure_block_workspace(rts_peel_t* h) {
 // small arrays), the rows of ceil(n_ant / G) antennas per CTA in shared memory.
 // Leaves bs_ok false (the per-sweep launches are used) when the device has no
 // cooperative launch or the rows do not fit.
+int setup_cluster_solve(rts_peel_t* h);
+
 int setup_block_solve(rts_peel_t* h) {
   if (h->solve_kernel != RTS_SOLVE_AUTO) return RTS_OK;
+  int rcc = setup_cluster_solve(h);
+  if (rcc || h->cl_size) return rcc;
   int coop = 0, n_sm = 0, smem_max = 0;
   RTS_CUDA(h, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
   RTS_CUDA(h, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device));
@@ -395,6 +405,88 @@ int setup_block_solve(rts_peel_t* h) {
   h->bs_smem = smem;
   h->bs_ok = true;
   return RTS_OK;
+}
+
+cudaLaunchConfig_t cluster_config(const rts_peel_t* h, cudaLaunchAttribute* attr, cudaStream_t s) {
+  cudaLaunchConfig_t c;
+  std::memset(&c, 0, sizeof(c));
+  c.gridDim = dim3(h->cl_size);
+  c.blockDim = dim3(32 * h->cl_apc);
+  c.dynamicSmemBytes = h->cl_smem;
+  c.stream = s;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = h->cl_size;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  c.attrs = attr;
+  c.numAttrs = 1;
+  return c;
+}
+
+// geometry of the cluster solve: about kClSlots antennas a CTA, at most kClMaxCta CTAs.
+// Leaves cl_size 0 (k_block_solve is used) when the rows do not fit or the device
+// has no room for such a cluster.
+int setup_cluster_solve(rts_peel_t* h) {
+  if (h->per_pass > kCorrMaxJ) return RTS_OK;
+  int smem_max = 0;
+  RTS_CUDA(h, cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
+  cudaFuncAttributes fa;
+  RTS_CUDA(h, cudaFuncGetAttributes(&fa, k_cluster_solve));
+  int cs = 1;
+  while (cs < kClMaxCta && (h->n_ant + cs - 1) / cs > kClSlots) cs *= 2;
+  const int apc = (h->n_ant + cs - 1) / cs;
+  if (apc > kClMaxSlots) return RTS_OK;
+  const size_t smem = cluster_solve_smem(h->n_ant, apc);
+  if (smem + fa.sharedSizeBytes + 1024 > (size_t)smem_max) return RTS_OK;
+  RTS_CUDA(h, cudaFuncSetAttribute(k_cluster_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max - (int)fa.sharedSizeBytes));
+  if (cs > 8 && cudaFuncSetAttribute(k_cluster_solve, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return RTS_OK;
+  }
+  h->cl_apc = apc;
+  h->cl_smem = smem;
+  h->cl_size = cs;
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t c = cluster_config(h, &attr, nullptr);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, k_cluster_solve, &c) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    h->cl_size = 0;
+    return RTS_OK;
+  }
+  RTS_CUDA(h, cudaMalloc((void**)&h->b_part, (size_t)h->per_pass * h->n_ant * 4 * sizeof(double)));
+  const size_t nn = (size_t)h->n_ant * h->n_ant;
+  RTS_CUDA(h, cudaMalloc((void**)&h->cl_V, kClGroup * 2 * nn * sizeof(float4)));
+  RTS_CUDA(h, cudaMalloc((void**)&h->cl_D, kClPairs * nn * sizeof(float2)));
+  return RTS_OK;
+}
+
+// the solve chain of sources s0 .. s0 + nblk - 1 by groups of kClGroup sources:
+// the terms of the block's earlier sources by the whole GPU, then the group's
+// chain in one cluster
+int launch_cluster_solve(rts_peel_t* h, int s0, int nblk, const float2* Dt, void* d_jones, cudaStream_t s) {
+  ClusterSolveArgs a;
+  a.V = h->cl_V; a.D = h->cl_D; a.src = h->d_src; a.s0 = s0;
+  a.n_ant = h->n_ant; a.n_bl = h->n_bl; a.n_iter = h->n_iter;
+  a.apc = h->cl_apc;
+  a.M = h->b_model; a.part = h->b_part; a.status = h->d_status; a.rel = h->d_rel;
+  a.jones = static_cast<float2*>(d_jones);
+  for (int q0 = 0; q0 < nblk; q0 += kClGroup) {
+    a.q0 = q0;
+    a.n_grp = std::min(kClGroup, nblk - q0);
+    {
+      Span span(h, RTS_K_BLOCK_FIX, s);
+      k_cluster_prep<<<(unsigned)((h->n_bl * 4 + 127) / 128), 128, 0, s>>>(h->b_avg, q0, a.n_grp, h->b_model, Dt,
+                                                                          h->d_bl_ant, h->n_ant, h->n_bl, h->cl_V,
+                                                                          h->cl_D);
+      span.end(1);
+    }
+    Span span(h, RTS_K_SOLVE, s);
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t c = cluster_config(h, &attr, s);
+    RTS_CUDA(h, cudaLaunchKernelEx(&c, k_cluster_solve, a));
+    span.end(1);
+  }
+  return check_launch(h, "cluster solve launch");
 }
 
 // the solve chain of sources s0 .. s0 + nblk - 1 (corrected averages, ALS,
@@ -520,11 +612,13 @@ int blocked_block(rts_peel_t* h) {
   const unsigned bl_grid = (unsigned)((h->n_bl + 255) / 256);
   const float2* Dt = h->b_dir[b % R];
   int rc;
-  if (h->bs_ok) {
-    rc = launch_block_solve(h, s0, nblk, Dt, br.jones, s);
+  const bool whole = h->cl_size || h->bs_ok;      // the block's chain as a whole
+  if (whole) {
+    rc = h->cl_size ? launch_cluster_solve(h, s0, nblk, Dt, br.jones, s)
+                    : launch_block_solve(h, s0, nblk, Dt, br.jones, s);
     if (rc) return rc;
   }
-  for (int q = 0; q < nblk && !h->bs_ok; ++q) {
+  for (int q = 0; q < nblk && !whole; ++q) {
     const int k = s0 + q;
     {
       Span span(h, RTS_K_BLOCK_FIX, s);
@@ -538,7 +632,7 @@ int blocked_block(rts_peel_t* h) {
     rc = launch_als(h, h->d_avg, h_src[3 * k + 2], static_cast<char*>(br.jones) + k * jstride, k, s);
     if (rc) return rc;
   }
-  if (!h->bs_ok) {
+  if (!whole) {
     Span span(h, RTS_K_BLOCK_FIX, s);
     k_block_model<<<bl_grid, 256, 0, s>>>(als_solution(h), h_src[3 * (s0 + nblk - 1) + 2], h->d_bl_ant,
                                            h->n_bl, h->b_model + (size_t)(nblk - 1) * h->n_bl * 4);
@@ -1445,7 +1539,7 @@ int rts_peel_kernels(const rts_peel_t* h, int32_t* block_kernel, int32_t* solve_
   if (block_kernel)
     *block_kernel = h->per_pass == 1 ? 0 : (h->block_tc05 ? RTS_BLOCK_TCGEN05 : (h->block_tc ? RTS_BLOCK_TENSOR : RTS_BLOCK_FMA));
   if (solve_kernel)
-    *solve_kernel = h->b_avg ? (h->bs_ok ? RTS_SOLVE_AUTO : RTS_SOLVE_LAUNCHES) : h->solve_kernel;
+    *solve_kernel = h->b_avg ? (h->cl_size || h->bs_ok ? RTS_SOLVE_AUTO : RTS_SOLVE_LAUNCHES) : h->solve_kernel;
   return RTS_OK;
 }
 
@@ -1487,7 +1581,7 @@ void rts_peel_destroy(rts_peel_t* h) {
   if (cudaGetDevice(&prev) == cudaSuccess && prev != h->device) cudaSetDevice(h->device);
   void* ptrs[] = {h->d_uvw, h->d_bl_ant, h->d_freq_c, h->d_avg, h->d_J[0], h->d_J[1], h->d_Jf[0],
                   h->d_Jf[1], h->d_norms, h->d_flag, h->d_status, h->d_rel, h->d_src, h->d_jones_stage,
-                  h->b_avg, h->b_aph, h->b_model, h->b_sync, h->b_part, h->d_perr, h->t_mom, h->t_X[0],
+                  h->b_avg, h->b_aph, h->b_model, h->b_sync, h->b_part, h->cl_V, h->cl_D, h->d_perr, h->t_mom, h->t_X[0],
                   h->t_X[1], h->t_Xf[0], h->t_Xf[1], h->t_rot_part, h->t_rot_count, h->t_rot_step};
   for (void* p : ptrs)
     if (p) cudaFree(p);
