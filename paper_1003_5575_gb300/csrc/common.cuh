@@ -137,4 +137,22 @@ __device__ inline double2 phasor_d(double x) {
   return make_double2(c, s);
 }
 
+// Reduce 8 doubles over the 32 lanes of a warp (a fixed shuffle tree: three
+// levels exchange half of the remaining values, two add the last one); lane L
+// ends with the warp total of value (L >> 2) & 7.
+__device__ __forceinline__ double warp_reduce_scatter8d(double (&v)[8], int lane) {
+  #pragma unroll
+  for (int o = 16, n = 8; o >= 4; o >>= 1, n >>= 1) {
+    const bool upper = (lane & o) != 0;
+    #pragma unroll
+    for (int i = 0; i < n / 2; ++i) {
+      const double send = upper ? v[i] : v[i + n / 2];
+      const double keep = upper ? v[i + n / 2] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double r = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 2);
+  return r + __shfl_xor_sync(0xffffffffu, r, 1);
+}
+
 }  // namespace rts

@@ -43,6 +43,10 @@ struct rts_peel_t {
   int2* d_bl_ant = nullptr;        // [n_bl]
   double* d_freq_c = nullptr;      // [n_chan] nu_c / c
   void* d_avg = nullptr;           // [n_bl][4] cube precision
+  // FP64 handles with exactly uniform channels: phasor tables of the subtracted and
+  // the averaged source, [n_time][n_ant][Q + R] each (k_fp64_ant_tables)
+  double2* d_tab64[2] = {nullptr, nullptr};
+  int tab64_q = 0, tab64_r = 0, tab64_at = 0;      // tab64_at: the last average's
   double2* d_J[2] = {nullptr, nullptr};
   float2* d_Jf[2] = {nullptr, nullptr};
   double* d_norms = nullptr;       // [n_ant][2]
@@ -206,9 +210,40 @@ StreamArgs stream_args(rts_peel_t* h, const void* src, void* dst, void* avg) {
   return a;
 }
 
-// one streaming pass: sub (subtract source) and/or acc (average for source)
-int launch_stream(rts_peel_t* h, bool sub, bool acc, const StreamArgs& a, cudaStream_t s) {
+template <bool TAB>
+void launch_stream_fp64(bool sub, bool acc, const StreamArgs& a, const Fp64Tables& tb, size_t smem, cudaStream_t s) {
+  const dim3 grid((unsigned)a.n_bl), block(kStreamThreads);
+  if (sub && acc) k_stream_fp64<true, true, TAB><<<grid, block, smem, s>>>(a, tb);
+  else if (sub) k_stream_fp64<true, false, TAB><<<grid, block, smem, s>>>(a, tb);
+  else k_stream_fp64<false, true, TAB><<<grid, block, smem, s>>>(a, tb);
+}
+
+// one streaming pass: sub (subtract source) and/or acc (average for source).
+// in_peel: the passes of a cadence, which own the handle's workspace (the FP64
+// phasor tables among it); rts_peel_rotate_average may run beside one
+int launch_stream(rts_peel_t* h, bool sub, bool acc, bool in_peel, const StreamArgs& a, cudaStream_t s) {
   const dim3 grid((unsigned)h->n_bl), block(kStreamThreads);
+  if (in_peel && h->precision == RTS_PREC_FP64 && h->d_tab64[0]) {
+    // the averaged source's antenna tables into the slot that the pass before the
+    // last one read; the subtracted source's are the last average's
+    Span span(h, sub && acc ? RTS_K_SUB_AVERAGE : (sub ? RTS_K_SUBTRACT : RTS_K_AVERAGE), s);
+    Fp64Tables tb;
+    tb.R = h->tab64_r; tb.Q = h->tab64_q;
+    tb.lr = 0;
+    while ((1 << tb.lr) < tb.R) ++tb.lr;
+    const size_t per_t = (size_t)2 * (tb.Q + tb.R) * sizeof(double2);
+    tb.n_t = (int)std::max<size_t>(1, std::min<size_t>(h->n_time, kFp64TableBytes / per_t));
+    tb.sub = h->d_tab64[h->tab64_at];
+    if (acc) {
+      h->tab64_at ^= 1;
+      k_fp64_ant_tables<<<2 * (unsigned)h->n_sm, 256, 0, s>>>(h->d_uvw, a.acc, h->n_ant, h->n_time, tb.Q, tb.R,
+                                                             a.nu0_c, a.dnu_c, h->d_tab64[h->tab64_at]);
+    }
+    tb.acc = h->d_tab64[h->tab64_at];
+    launch_stream_fp64<true>(sub, acc, a, tb, tb.n_t * per_t, s);
+    span.end(acc ? 2 : 1);
+    return check_launch(h, "streaming kernel launch");
+  }
   Span span(h, sub && acc ? RTS_K_SUB_AVERAGE : (sub ? RTS_K_SUBTRACT : RTS_K_AVERAGE), s);
   if (h->precision == RTS_PREC_MIXED) {
     const size_t smem = (size_t)h->n_time * 4 * sizeof(unsigned long long);
@@ -216,10 +251,7 @@ int launch_stream(rts_peel_t* h, bool sub, bool acc, const StreamArgs& a, cudaSt
     else if (sub) k_stream_mixed<true, false><<<grid, block, smem, s>>>(a);
     else k_stream_mixed<false, true><<<grid, block, smem, s>>>(a);
   } else {
-    const size_t smem = (size_t)h->n_time * 2 * sizeof(double);
-    if (sub && acc) k_stream_fp64<true, true><<<grid, block, smem, s>>>(a);
-    else if (sub) k_stream_fp64<true, false><<<grid, block, smem, s>>>(a);
-    else k_stream_fp64<false, true><<<grid, block, smem, s>>>(a);
+    launch_stream_fp64<false>(sub, acc, a, Fp64Tables(), (size_t)h->n_time * 2 * sizeof(double), s);
   }
   span.end(1);
   return check_launch(h, "streaming kernel launch");
@@ -702,7 +734,7 @@ int peel_device(rts_peel_t* h, const void* d_vis, void* d_resid, int32_t n_src,
   const size_t jstride = (size_t)h->n_ant * 4 * h->elem;
   StreamArgs a = stream_args(h, d_vis, d_resid, h->d_avg);
   a.acc = make_dir(h_src[0], h_src[1], h_src[2]);
-  int rc = launch_stream(h, false, true, a, s);
+  int rc = launch_stream(h, false, true, true, a, s);
   if (rc) return rc;
   for (int k = 0; k < n_src; ++k) {
     rc = launch_als(h, h->d_avg, h_src[3 * k + 2], static_cast<char*>(d_jones) + k * jstride, k, s);
@@ -712,7 +744,7 @@ int peel_device(rts_peel_t* h, const void* d_vis, void* d_resid, int32_t n_src,
     b.Jsub = als_solution(h);
     const bool more = k + 1 < n_src;
     if (more) b.acc = make_dir(h_src[3 * (k + 1)], h_src[3 * (k + 1) + 1], h_src[3 * (k + 1) + 2]);
-    rc = launch_stream(h, true, more, b, s);
+    rc = launch_stream(h, true, more, true, b, s);
     if (rc) return rc;
   }
   if (h_status) return read_status(h, n_src, h_status, s);
@@ -1119,6 +1151,20 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
   if ((e = cudaMemset(h->d_flag, 0, sizeof(int))) != cudaSuccess) return bail(e, "clear flag");
   if ((e = cudaMemset(h->d_status, 0, (size_t)h->max_sources * sizeof(int))) != cudaSuccess)
     return bail(e, "clear status");
+  if (h->precision == RTS_PREC_FP64) {
+    // phasor tables where nu_0 + c dnu is every channel to FP64 rounding (a phase of
+    // 1e3 turns then moves by less than the FP64 phase itself is rounded) and they
+    // stay small beside the cube (256 MB: past that a sincospi a sample)
+    bool uniform = true;
+    for (int c = 0; c < h->n_chan && uniform; ++c) uniform = std::fabs(f[c] - (nu0 + c * dnu)) <= 4.5e-16 * f[c];
+    const int R = fp64_table_r(h->n_chan), Q = (h->n_chan + R - 1) / R;
+    const size_t bytes = (size_t)h->n_time * h->n_ant * (Q + R) * sizeof(double2);
+    if (uniform && bytes <= ((size_t)128 << 20)) {
+      for (int k = 0; k < 2; ++k)
+        if ((e = cudaMalloc((void**)&h->d_tab64[k], bytes)) != cudaSuccess) return bail(e, "cudaMalloc(phasor tables)");
+      h->tab64_q = Q; h->tab64_r = R;
+    }
+  }
   // the blocked schedule's tables, streams and solve set-up, and the Taylor
   // cadence's moments and iterates, are allocated here too (the paper's Section 5
   // advice), so a cadence allocates nothing
@@ -1385,7 +1431,7 @@ int rts_peel_rotate_average(rts_peel_t* h, const void* d_vis, double l, double m
     return fail(h, RTS_EINVAL, "direction must be finite with l^2 + m^2 < 1");
   StreamArgs a = stream_args(h, d_vis, nullptr, d_avg);
   a.acc = make_dir(l, m, 1.0);
-  return launch_stream(h, false, true, a, as_stream(stream));
+  return launch_stream(h, false, true, false, a, as_stream(stream));
 }
 
 int rts_peel_solve(rts_peel_t* h, const void* d_avg, double S, void* d_jones, int32_t* h_status,
@@ -1581,7 +1627,7 @@ void rts_peel_destroy(rts_peel_t* h) {
   if (cudaGetDevice(&prev) == cudaSuccess && prev != h->device) cudaSetDevice(h->device);
   void* ptrs[] = {h->d_uvw, h->d_bl_ant, h->d_freq_c, h->d_avg, h->d_J[0], h->d_J[1], h->d_Jf[0],
                   h->d_Jf[1], h->d_norms, h->d_flag, h->d_status, h->d_rel, h->d_src, h->d_jones_stage,
-                  h->b_avg, h->b_aph, h->b_model, h->b_sync, h->b_part, h->cl_V, h->cl_D, h->d_perr, h->t_mom, h->t_X[0],
+                  h->b_avg, h->b_aph, h->b_model, h->b_sync, h->b_part, h->cl_V, h->cl_D, h->d_perr, h->d_tab64[0], h->d_tab64[1], h->t_mom, h->t_X[0],
                   h->t_X[1], h->t_Xf[0], h->t_Xf[1], h->t_rot_part, h->t_rot_count, h->t_rot_step};
   for (void* p : ptrs)
     if (p) cudaFree(p);

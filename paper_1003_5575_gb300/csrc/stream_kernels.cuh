@@ -56,28 +56,6 @@ __device__ inline void block_sum_f32_to_f64(float (&v)[N], double* s_red /* [32]
   }
 }
 
-template <int N>
-__device__ inline void block_sum_f64(double (&v)[N], double* s_red, double (&out)[N]) {
-  #pragma unroll
-  for (int k = 0; k < N; ++k)
-    #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0)
-    #pragma unroll
-    for (int k = 0; k < N; ++k) s_red[warp * N + k] = v[k];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = blockDim.x >> 5;
-    #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      double s = 0.0;
-      for (int w = 0; w < nw; ++w) s += s_red[w * N + k];
-      out[k] = s;
-    }
-  }
-}
-
 // (t, c) walk of one thread: s = t*n_chan + c advanced by kStreamThreads
 struct TCWalk {
   int t, c, dt, dc, n_chan;
@@ -207,26 +185,74 @@ __global__ void __launch_bounds__(kStreamThreads, 3) k_stream_mixed(StreamArgs a
 }
 
 // ---------------------------------------------------------------------------
-// plain FP64: complex128 cube, per-sample FP64 phase tau * nu_c / c, FP64 sincospi
+// plain FP64: complex128 cube, FP64 sincospi, FP64 arithmetic
+//
+// GB300 retires about 1.7 FP64 fused multiply-adds a cycle and SM (19 cycles a
+// warp instruction), so the pass is bound by how many it issues: 32 a sample
+// are the two roles' four complex multiply-adds each, written as fused chains;
+// two sincospi a sample would be about 80 more.  Where the channels are uniform
+// to FP64 rounding the phasor is therefore a product of table entries instead
+// (4 more a role): channel c = R q + r has e^{2 pi i tau nu_c / c} = T1[q] T2[r]
+// with T1[q] = e^{2 pi i tau (nu_0 + R q dnu) / c}, T2[r] = e^{2 pi i tau r dnu / c},
+// and, because tau_ij = tau_i - tau_j, each table of a baseline is the product
+// T_i conj(T_j) of its antennas' tables, which k_fp64_ant_tables forms once per
+// source ([n_time][n_ant][Q + R]).  At 128 antennas x 128 channels x 8 times x 50
+// sources the whole cadence, solves included, went from 111 to 48.6 ms.  Other
+// frequency lists (uniform to 1e-9 only) keep one sincospi per sample and role
+// (TAB = false).
 
-template <bool SUB, bool ACC>
-__global__ void __launch_bounds__(kStreamThreads) k_stream_fp64(StreamArgs a) {
-  extern __shared__ double s_tau[];   // [n_time][2]: tau_sub, tau_acc
+constexpr size_t kFp64TableBytes = 32 * 1024;    // a CTA's baseline tables, at most (but one time's)
+
+// R of the tables: about sqrt(n_chan), a power of two
+__host__ inline int fp64_table_r(int n_chan) {
+  int r = 1;
+  while (r * r < n_chan) r *= 2;
+  return r;
+}
+
+// [n_time][n_ant][Q + R]: T1 then T2 of one source direction
+__global__ void __launch_bounds__(256) k_fp64_ant_tables(const double* __restrict__ uvw, SrcDir d, int n_ant,
+                                                        int n_time, int Q, int R, double nu0_c, double dnu_c,
+                                                        double2* __restrict__ tab) {
+  const int n_e = Q + R;
+  const int64_t n = (int64_t)n_time * n_ant * n_e;
+  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t ta = x / n_e;
+    const int e = (int)(x - ta * n_e);
+    const double* u = uvw + ta * 3;
+    const double tau = u[0] * d.l + u[1] * d.m + u[2] * d.nm1;
+    tab[x] = phasor_d(tau * (e < Q ? nu0_c + (double)(R * e) * dnu_c : (double)(e - Q) * dnu_c));
+  }
+}
+
+struct Fp64Tables {
+  const double2* sub;       // [n_time][n_ant][Q + R] of the subtracted source
+  const double2* acc;       // of the averaged source
+  int Q, R, lr;             // R = 1 << lr
+  int n_t;                  // times whose baseline tables a CTA holds at once
+};
+
+template <bool SUB, bool ACC, bool TAB>
+__global__ void __launch_bounds__(kStreamThreads) k_stream_fp64(StreamArgs a, Fp64Tables tb) {
+  extern __shared__ __align__(16) unsigned char s_f64[];
+  // TAB: [n_t][sub, acc][Q + R] double2; else [n_time][2] double: tau_sub, tau_acc
+  double2* s_tab = reinterpret_cast<double2*>(s_f64);
+  double* s_tau = reinterpret_cast<double*>(s_f64);
   __shared__ double2 s_M[4];
-  __shared__ double s_red[(kStreamThreads / 32) * 8];
+  __shared__ double s_red[kStreamThreads / 32][8];
   const int64_t bl = blockIdx.x;
   const int2 ij = a.bl_ant[bl];
-  for (int t = threadIdx.x; t < a.n_time; t += blockDim.x) {
-    if (SUB) s_tau[2 * t] = delay_m(a.uvw, a.n_ant, t, ij.x, ij.y, a.sub);
-    if (ACC) s_tau[2 * t + 1] = delay_m(a.uvw, a.n_ant, t, ij.x, ij.y, a.acc);
-  }
-  if (SUB && threadIdx.x == 0) {
-    M22<double2> Ji, Jj;
-    #pragma unroll
-    for (int e = 0; e < 4; ++e) { Ji.e[e] = a.Jsub[(size_t)ij.x * 4 + e]; Jj.e[e] = a.Jsub[(size_t)ij.y * 4 + e]; }
-    M22<double2> P = mmul_h(Ji, Jj);
-    #pragma unroll
-    for (int e = 0; e < 4; ++e) s_M[e] = make_double2(a.sub.S * P.e[e].x, a.sub.S * P.e[e].y);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (!TAB)
+    for (int t = tid; t < a.n_time; t += kStreamThreads) {
+      if (SUB) s_tau[2 * t] = delay_m(a.uvw, a.n_ant, t, ij.x, ij.y, a.sub);
+      if (ACC) s_tau[2 * t + 1] = delay_m(a.uvw, a.n_ant, t, ij.x, ij.y, a.acc);
+    }
+  if (SUB && tid < 4) {                      // -S J_i J_j^H, one entry a thread
+    const int r = tid >> 1, c = tid & 1;
+    const double2 *Ji = a.Jsub + (size_t)ij.x * 4 + 2 * r, *Jj = a.Jsub + (size_t)ij.y * 4 + 2 * c;
+    const double2 m = cadd(cmulc(Ji[0], Jj[0]), cmulc(Ji[1], Jj[1]));
+    s_M[tid] = make_double2(-a.sub.S * m.x, -a.sub.S * m.y);
   }
   __syncthreads();
   double2 M[4];
@@ -239,35 +265,64 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream_fp64(StreamArgs a) {
   for (int k = 0; k < 8; ++k) acc[k] = 0.0;
   const double2* src = static_cast<const double2*>(a.src);
   double2* dst = static_cast<double2*>(a.dst);
-  const int n_s = a.n_time * a.n_chan;
-  TCWalk w;
-  w.init(threadIdx.x, a.n_chan);
-  for (int s = threadIdx.x; s < n_s; s += kStreamThreads, w.next()) {
-    const size_t idx = (((size_t)w.t * a.n_bl + bl) * a.n_chan + w.c) * 4;
-    double2 x[4];
-    #pragma unroll
-    for (int e = 0; e < 4; ++e) x[e] = src[idx + e];
-    if (SUB) {
-      double2 ph = phasor_d(s_tau[2 * w.t] * a.freq_c[w.c]);     // exp(+2 pi i phi)
-      #pragma unroll
-      for (int e = 0; e < 4; ++e) { x[e] = csub(x[e], cmulc(M[e], ph)); dst[idx + e] = x[e]; }
+  const int n_e = tb.Q + tb.R;
+  const int t_step = TAB ? tb.n_t : a.n_time;
+  for (int t0 = 0; t0 < a.n_time; t0 += t_step) {
+    const int nt = min(t_step, a.n_time - t0);
+    if (TAB) {
+      if (t0) __syncthreads();               // the previous times' tables are read
+      for (int x = tid; x < nt * 2 * n_e; x += kStreamThreads) {
+        const int row = x / n_e, e = x - row * n_e;
+        if ((row & 1) ? !ACC : !SUB) continue;
+        const double2* g = (row & 1) ? tb.acc : tb.sub;
+        const size_t at = (size_t)(t0 + (row >> 1)) * a.n_ant;
+        s_tab[x] = cmulc(g[(at + ij.x) * n_e + e], g[(at + ij.y) * n_e + e]);
+      }
+      __syncthreads();
     }
-    if (ACC) {
-      double2 ph = phasor_d(s_tau[2 * w.t + 1] * a.freq_c[w.c]);
+    const int n_s = nt * a.n_chan;
+    TCWalk w;
+    w.init(tid, a.n_chan);
+    for (int s = tid; s < n_s; s += kStreamThreads, w.next()) {
+      const size_t idx = (((size_t)(t0 + w.t) * a.n_bl + bl) * a.n_chan + w.c) * 4;
+      double2 x[4];
       #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        double2 r = cmul(x[e], ph);
-        acc[2 * e] += r.x; acc[2 * e + 1] += r.y;
+      for (int e = 0; e < 4; ++e) x[e] = src[idx + e];
+      auto phasor = [&](int role) {           // exp(+2 pi i phi)
+        if (!TAB) return phasor_d(s_tau[2 * w.t + role] * a.freq_c[w.c]);
+        const double2* T = s_tab + (size_t)(2 * w.t + role) * n_e;
+        return cmul(T[w.c >> tb.lr], T[tb.Q + (w.c & (tb.R - 1))]);
+      };
+      if (SUB) {
+        const double2 ph = phasor(0);
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) {         // x += (-M) conj(ph)
+          x[e].x = fma(M[e].x, ph.x, fma(M[e].y, ph.y, x[e].x));
+          x[e].y = fma(M[e].y, ph.x, fma(-M[e].x, ph.y, x[e].y));
+          dst[idx + e] = x[e];
+        }
+      }
+      if (ACC) {
+        const double2 ph = phasor(1);
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          acc[2 * e] = fma(x[e].x, ph.x, fma(-x[e].y, ph.y, acc[2 * e]));
+          acc[2 * e + 1] = fma(x[e].x, ph.y, fma(x[e].y, ph.x, acc[2 * e + 1]));
+        }
       }
     }
   }
   if (ACC) {
-    double tot[8];
-    block_sum_f64<8>(acc, s_red, tot);
-    if (threadIdx.x == 0) {
-      double2* out = static_cast<double2*>(a.avg) + bl * 4;
+    // warp totals by halving exchanges (9 additions a lane for the 8 sums), then
+    // one thread a sum adds the warps' in warp order
+    const double v = warp_reduce_scatter8d(acc, lane);
+    if ((lane & 3) == 0) s_red[warp][lane >> 2] = v;
+    __syncthreads();
+    if (tid < 8) {
+      double t = 0.0;
       #pragma unroll
-      for (int e = 0; e < 4; ++e) out[e] = make_double2(tot[2 * e] * a.inv_n, tot[2 * e + 1] * a.inv_n);
+      for (int w2 = 0; w2 < kStreamThreads / 32; ++w2) t += s_red[w2][tid];
+      static_cast<double*>(a.avg)[bl * 8 + tid] = t * a.inv_n;
     }
   }
 }
