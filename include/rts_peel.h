@@ -86,9 +86,11 @@ typedef struct rts_peel_config {
                            one pass per block of that many sources, the averages inside a
                            block corrected in closed form (same results); 0 = library
                            default (RTS_BLOCK) */
-  int32_t block_kernel;  /* blocked peel only: RTS_BLOCK_AUTO (0: the tcgen05 pass when
-                           n_chan <= 768, else the mma.sync pass when n_chan <= 960, else
-                           the FP32 pass), RTS_BLOCK_FMA (the FP32 FMA pass),
+  int32_t block_kernel;  /* blocked peel only: RTS_BLOCK_AUTO (0: the FP32 pass when
+                           n_chan <= 256, else the tcgen05 pass when n_chan <= 768, else
+                           the mma.sync pass when n_chan <= 960, else the FP32 pass),
+                           RTS_BLOCK_FMA (the FP32 FMA pass; a warp per baseline and time
+                           while n_chan <= 256),
                            RTS_BLOCK_TENSOR (TF32 mma.sync with split operands;
                            n_chan <= 960, else RTS_EINVAL), RTS_BLOCK_TCGEN05 (tcgen05.mma
                            with TMEM accumulators, TF32 with split operands; n_chan <= 768,

@@ -22,6 +22,7 @@
 #include "predict_kernels.cuh"
 #include "solve_kernels.cuh"
 #include "stream_kernels.cuh"
+#include "strip_kernels.cuh"
 #include "taylor_kernels.cuh"
 #include "taylor_block_kernels.cuh"
 
@@ -32,6 +33,8 @@ struct rts_peel_t {
   int per_pass = 1;                // sources per streaming pass (1 or RTS_BLOCK)
   bool block_tc = false;           // blocked passes as TF32 mma.sync (k_block_pass_tc)
   bool block_tc05 = false;           // blocked passes as tcgen05 MMAs (k_block_pass_tc05)
+  bool tay_tc05 = false;             // and the Taylor cadence's
+  int strip_qh = 0;                  // FP32 passes by k_block_pass_strip<strip_qh> (0: k_block_pass)
   int* d_perr = nullptr;           // [1] set by a tcgen05 pass whose mbarrier wait ran out
   int64_t n_bl = 0;
   double nu0 = 0, dnu = 0;
@@ -336,6 +339,17 @@ int set_block_smem(rts_peel_t* h, int smem) {
   return RTS_OK;
 }
 
+// handles of other sizes share the kernels: the attribute is the most they may take
+constexpr int kStripMaxSmem = 227 * 1024;
+
+template <int QH>
+int set_strip_smem(rts_peel_t* h) {
+  RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_strip<QH, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripMaxSmem));
+  RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_strip<QH, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripMaxSmem));
+  RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_strip<QH, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripMaxSmem));
+  return RTS_OK;
+}
+
 int setup_block_solve(rts_peel_t* h);
 
 // the tcgen05 pass holds all 512 TMEM columns: at least 116 KB of shared memory
@@ -376,12 +390,14 @@ int ensure_block_workspace(rts_peel_t* h) {
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
+  }
+  if (h->tay_tc05) {
     const int tay = (int)tc05_tay_launch_smem(h);
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
-    return RTS_OK;
   }
+  if (h->block_tc05) return RTS_OK;
   if (h->block_tc) {
     const int tsm = (int)tc_pass_smem(h->n_chan);
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
@@ -389,6 +405,7 @@ int ensure_block_workspace(rts_peel_t* h) {
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
     return RTS_OK;
   }
+  if (h->strip_qh) return h->strip_qh == 2 ? set_strip_smem<2>(h) : h->strip_qh == 4 ? set_strip_smem<4>(h) : set_strip_smem<8>(h);
   const int smem = (int)block_pass_smem(h);
   switch (BK) {
     case 8: return set_block_smem<8>(h, smem);
@@ -543,6 +560,16 @@ int launch_block_solve(rts_peel_t* h, int s0, int nblk, const float2* Dt, void* 
   return check_launch(h, "block solve launch");
 }
 
+template <int QH>
+void strip_pass_t(const rts_peel_t* h, bool sub, bool acc, const BlockPassArgs& a, cudaStream_t s) {
+  const StripGrid g = strip_grid(h->n_time);
+  const size_t smem = strip_pass_smem<QH>(g, h->n_time);
+  const unsigned grid = (unsigned)((h->n_bl + g.bpc - 1) / g.bpc), nthr = 32u * g.wpb * g.bpc;
+  if (sub && acc) k_block_pass_strip<QH, true, true><<<grid, nthr, smem, s>>>(a, h->per_pass, g);
+  else if (sub) k_block_pass_strip<QH, true, false><<<grid, nthr, smem, s>>>(a, h->per_pass, g);
+  else k_block_pass_strip<QH, false, true><<<grid, nthr, smem, s>>>(a, h->per_pass, g);
+}
+
 template <int BK>
 void block_pass_t(bool sub, bool acc, const BlockPassArgs& a, unsigned grid, size_t smem, cudaStream_t s) {
   if (sub && acc) k_block_pass<BK, true, true><<<grid, kBlkThreads, smem, s>>>(a);
@@ -569,6 +596,15 @@ int launch_block_pass(rts_peel_t* h, bool sub, bool acc, const BlockPassArgs& a,
     if (sub && acc) k_block_pass_tc<true, true><<<grid, kTcThreads, tsm, s>>>(a, h->per_pass);
     else if (sub) k_block_pass_tc<true, false><<<grid, kTcThreads, tsm, s>>>(a, h->per_pass);
     else k_block_pass_tc<false, true><<<grid, kTcThreads, tsm, s>>>(a, h->per_pass);
+    span.end(1);
+    return check_launch(h, "block pass launch");
+  }
+  if (h->strip_qh) {
+    switch (h->strip_qh) {
+      case 2: strip_pass_t<2>(h, sub, acc, a, s); break;
+      case 4: strip_pass_t<4>(h, sub, acc, a, s); break;
+      default: strip_pass_t<8>(h, sub, acc, a, s); break;
+    }
     span.end(1);
     return check_launch(h, "block pass launch");
   }
@@ -873,7 +909,7 @@ int peel_taylor(rts_peel_t* h, const void* d_vis, void* d_resid, int32_t n_src, 
 // tcgen05 blocked workspace of 64-source blocks (its tables hold a Taylor
 // block: phases of 21 <= 32 sources, 210 x 5 <= 2016 D terms, 63 slots)
 bool taylor_blocked(const rts_peel_t* h) {
-  return h->block_tc05 && h->per_pass == kTc5Src && h->n_band == h->n_chan;
+  return h->tay_tc05 && h->per_pass == kTc5Src && h->n_band == h->n_chan;
 }
 
 // mu_j = mean_c x_c^j, x_c = (c - (N - 1)/2) / N, in FP64 (odd j: zero by symmetry)
@@ -1095,10 +1131,14 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
   h->grad_direct = cfg->grad_kernel == RTS_GRAD_DIRECT;
   {
     int bk = cfg->block_kernel;
+    h->tay_tc05 = per_pass > 1 && (bk == RTS_BLOCK_TCGEN05 || (bk == RTS_BLOCK_AUTO && cfg->n_chan <= kTc5MaxChan));
+    if (bk == RTS_BLOCK_AUTO && cfg->n_chan <= kStAutoChan) bk = RTS_BLOCK_FMA;
     if (bk == RTS_BLOCK_AUTO)
       bk = cfg->n_chan <= kTc5MaxChan ? RTS_BLOCK_TCGEN05 : (cfg->n_chan <= kTcMaxChan ? RTS_BLOCK_TENSOR : RTS_BLOCK_FMA);
     h->block_tc05 = per_pass > 1 && bk == RTS_BLOCK_TCGEN05;
     h->block_tc = per_pass > 1 && bk == RTS_BLOCK_TENSOR;
+    if (per_pass > 1 && bk == RTS_BLOCK_FMA && cfg->n_chan <= 32 * kStMaxQh)
+      h->strip_qh = cfg->n_chan <= 64 ? 2 : cfg->n_chan <= 128 ? 4 : 8;
   }
   h->n_ant = cfg->n_ant; h->n_chan = cfg->n_chan; h->n_time = cfg->n_time;
   h->n_iter = cfg->n_iter; h->precision = cfg->precision; h->max_sources = cfg->max_sources;

@@ -1,0 +1,53 @@
+"""The FP32 kernels that work on strips (strip_kernels.cuh) at the edges of their
+tiles: the blocked pass, the prediction and the adjoint, against the oracle.
+Strips hold 64, 128 or 256 channels in tiles of 16, sources go 32 or 64 at a
+time, a CTA's warps take 8 (pass, prediction) or 12 (adjoint) strips.
+
+Tolerances as test_gpu_parity.py.  The pass's cases are well conditioned: the
+FP64 oracle moves by at most 1.5e-7 (Jones) and 7e-8 x rms (residual) under an
+input perturbation of 1e-7 x rms."""
+import numpy as np
+import pytest
+
+import oracle
+from synth import Cadence
+
+torch = pytest.importorskip("torch")
+from _parity import TOL, check_status, jones_rel, make_peeler, oracle_case, rms_of, to_dev  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_5575_gb300 import build
+    build.build()
+
+
+PASS_CASES = [
+    ("17-channels", Cadence(40, 17, 8, 2, freq0_hz=167e6, seed=216), 64),
+    ("64-channels-one-time", Cadence(20, 64, 1, 3, freq0_hz=167e6, seed=211), 64),      # eight baselines a CTA
+    ("65-channels-9-times", Cadence(20, 65, 9, 33, freq0_hz=167e6, seed=212), 64),      # a warp's second time; 33 sources
+    ("65-channels-blocks-of-16", Cadence(20, 65, 9, 33, freq0_hz=167e6, seed=212), 16),
+    ("128-channels", Cadence(24, 128, 3, 6, freq0_hz=167e6, seed=213), 64),             # two baselines a CTA, odd count
+    ("129-channels", Cadence(24, 129, 5, 8, freq0_hz=167e6, seed=214), 8),
+    ("256-channels-17-times", Cadence(30, 256, 17, 35, freq0_hz=167e6, seed=215), 64),
+]
+
+
+@pytest.mark.parametrize("name,cad,per_pass", PASS_CASES, ids=[c[0] for c in PASS_CASES])
+def test_strip_pass_matches_oracle(name, cad, per_pass):
+    V, R_ref, J_ref, st_ref, rel_ref = oracle_case(cad)
+    p = make_peeler(cad, "mixed", per_pass=per_pass, block_kernel=1)
+    vis = to_dev(V, "mixed")
+    resid, jones, st = p.cadence(vis, cad.sources())
+    work = vis.clone()
+    r2, j2, _ = p.cadence(work, cad.sources(), resid=work)                   # in place: the same bits
+    torch.cuda.synchronize()
+    assert np.abs(resid.cpu().numpy() - R_ref).max() / rms_of(V) <= TOL["mixed"]
+    assert jones_rel(jones.cpu().numpy(), J_ref) <= TOL["mixed"]
+    check_status(name, st, st_ref, p.rel(cad.n_src), rel_ref)
+    assert torch.equal(r2, resid) and torch.equal(j2, jones)
+    p.close()
