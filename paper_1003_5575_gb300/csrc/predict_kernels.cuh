@@ -5,6 +5,7 @@
 #pragma once
 #include "stream_kernels.cuh"
 #include "kahan.cuh"
+#include "strip_kernels.cuh"
 
 namespace rts {
 
@@ -91,6 +92,109 @@ __global__ void __launch_bounds__(kStreamThreads) k_predict_mixed(PredictArgs a)
     }
     vis[idx] = make_float4(sum[0], sum[1], sum[2], sum[3]);
     vis[idx + 1] = make_float4(sum[4], sum[5], sum[6], sum[7]);
+  }
+}
+
+// The FP32 prediction on strips (strip_kernels.cuh): a warp accumulates one
+// (baseline, time, 32 QH channels) strip in registers, a launch takes up to
+// kPredictStripSrc sources in two groups.  Against one hardware sin/cos and a
+// compensated sum per (source, channel), about 60 instructions, it issues about
+// 15: phasors as products of table entries, packed multiply-adds, each group
+// of 32 sources summed in FP32 and the two groups and the cube added exactly
+// and rounded once.  Model matrices by float-float products (as their FP64
+// evaluation, rounded to FP32); phases as differences of the antennas' Q0.64
+// phases (k_block_ant_phases).  Bound by instruction issue and the FP32 pipe: 20
+// multiply-adds per source and channel, two an instruction.  100 sources into
+// 128 antennas x 256 channels x 8 times: 1.88 ms, k_predict_mixed 4.01 ms; error
+// against 64 bits 1.8e-7 and 2.0e-7.  Strips of 128 channels (QH = 4): 64 registers
+// hold a group's sum and the one before it.
+constexpr int kPredictStripSrc = 2 * kStGrp;
+// Antenna phases a handle keeps for predictions, at most: 1 KB per antenna and time,
+// 4 MB for 512 antennas and 8 times.  Longer cubes (more than 131 072 antenna-times),
+// and handles whose device has no room for them, take k_predict_mixed, which needs none.
+constexpr size_t kPredictAphBytes = (size_t)128 << 20;
+
+template <int QH> size_t predict_strip_smem(const StripGrid& g) {
+  return 256 * sizeof(float2) + (size_t)g.bpc * kPredictStripSrc * kStMRow * sizeof(float4) +
+         (size_t)g.wpb * g.bpc * sizeof(StripTables<QH>);
+}
+
+// a.n_src <= kPredictStripSrc; aph [n_time][n_ant][kPredictStripSrc]; n_tile tiles of 32 QH channels
+template <int QH>
+__global__ void __launch_bounds__(kStWarps * 32, 2) k_predict_strip(PredictArgs a, const PhaseAB* __restrict__ aph,
+                                                                   StripGrid g, int n_tile) {
+  extern __shared__ __align__(16) unsigned char ps_smem[];
+  float2* lut = reinterpret_cast<float2*>(ps_smem);
+  float4* Mt = reinterpret_cast<float4*>(lut + 256);                     // [bpc][kPredictStripSrc][kStMRow]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthr = blockDim.x;
+  StripTables<QH>& tb =
+      reinterpret_cast<StripTables<QH>*>(Mt + (size_t)g.bpc * kPredictStripSrc * kStMRow)[warp];
+  const int lb = warp / g.wpb, w = warp - lb * g.wpb;
+  const int64_t bl0 = (int64_t)blockIdx.x * g.bpc, bl = bl0 + lb;
+  lut_fill(lut, tid, nthr);
+  for (int i = tid; i < g.bpc * a.n_src * 4; i += nthr) {
+    const int e = i & 3, k = (i >> 2) % a.n_src, b = (i >> 2) / a.n_src;
+    if (bl0 + b >= a.n_bl) continue;
+    const int2 ij = a.bl_ant[bl0 + b];
+    const size_t at = (size_t)k * a.n_ant;
+    const double S = a.src[3 * k + 2];
+    const float Sh = (float)S, Sl = (float)(S - (double)Sh);
+    const float2 m = model_entry_ff(jones_row(a.jones, 2 * (at + ij.x) + (e >> 1)),
+                                    jones_row(a.jones, 2 * (at + ij.y) + (e & 1)), Sh, Sl);
+    strip_pack_model(Mt + ((size_t)b * kPredictStripSrc + k) * kStMRow, e, make_float2(-m.x, -m.y));
+  }
+  __syncthreads();
+  if (bl >= a.n_bl) return;
+  const int2 ij = a.bl_ant[bl];
+  const int n_strip = a.n_time * n_tile;
+  for (int s = w; s < n_strip; s += g.wpb) {
+    const int t = s / n_tile, c0 = (s - t * n_tile) * 32 * QH, nc = min(32 * QH, a.n_chan - c0);
+    const int np = (((nc + 15) >> 4) + 1) >> 1;
+    Strip<QH> R, R0;
+    #pragma unroll
+    for (int e = 0; e < 4; ++e)
+      #pragma unroll
+      for (int v = 0; v < QH / 2; ++v) R.re[e][v] = R.im[e][v] = R0.re[e][v] = R0.im[e][v] = make_float2(0.f, 0.f);
+    for (int k0 = 0; k0 < a.n_src; k0 += kStGrp) {
+      PhaseAB p;
+      p.a = 0; p.b = 0;
+      if (k0 + lane < a.n_src) {
+        const PhaseAB pi = aph[((size_t)t * a.n_ant + ij.x) * kPredictStripSrc + k0 + lane];
+        const PhaseAB pj = aph[((size_t)t * a.n_ant + ij.y) * kPredictStripSrc + k0 + lane];
+        p.b = pi.b - pj.b;
+        p.a = pi.a - pj.a + (unsigned long long)c0 * p.b;
+      }
+      if (k0) R0 = R;
+      if (k0)
+        #pragma unroll
+        for (int e = 0; e < 4; ++e)
+          #pragma unroll
+          for (int v = 0; v < QH / 2; ++v) R.re[e][v] = R.im[e][v] = make_float2(0.f, 0.f);
+      __syncwarp();
+      strip_tables<QH>(tb, p, lane, np, lut);
+      __syncwarp();
+      strip_subtract<QH>(R, tb, Mt + ((size_t)lb * kPredictStripSrc + k0) * kStMRow, min(kStGrp, a.n_src - k0), lane);
+    }
+    float4* vis = static_cast<float4*>(a.vis) + (((size_t)t * a.n_bl + bl) * a.n_chan + c0) * 2;
+    const int cl = 16 * (lane >> 4) * QH + (lane & 15);
+    #pragma unroll
+    for (int u = 0; u < QH; ++u) {
+      const int c = cl + 16 * u;
+      if (c >= nc) continue;
+      float re[4], im[4], re0[4], im0[4];
+      strip_channel(R, u, re, im);
+      strip_channel(R0, u, re0, im0);
+      float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
+      if (a.accumulate) { x0 = __ldcs(vis + 2 * c); x1 = __ldcs(vis + 2 * c + 1); }
+      auto sum = [](float x, float p, float q) {           // x + p + q, rounded once
+        const FF s = ff_two_sum(p, q), o = ff_two_sum(x, s.hi);
+        return o.hi + (o.lo + s.lo);
+      };
+      __stcs(vis + 2 * c, make_float4(sum(x0.x, re0[0], re[0]), sum(x0.y, im0[0], im[0]), sum(x0.z, re0[1], re[1]),
+                                     sum(x0.w, im0[1], im[1])));
+      __stcs(vis + 2 * c + 1, make_float4(sum(x1.x, re0[2], re[2]), sum(x1.y, im0[2], im[2]),
+                                         sum(x1.z, re0[3], re[3]), sum(x1.w, im0[3], im[3])));
+    }
   }
 }
 

@@ -57,6 +57,7 @@ struct rts_peel_t {
   int* d_status = nullptr;         // [max_sources]
   double* d_rel = nullptr;         // [max_sources]
   double* d_src = nullptr;         // [max_sources][3]
+  PhaseAB* d_aph = nullptr;        // [n_time][n_ant][kPredictStripSrc] antenna phases of a prediction's sources
   void* d_jones_stage = nullptr;   // [max_sources][n_ant][4] cube precision (host-buffer calls)
   GradWorkspace grad;
   // gains Taylor-expanded in frequency (allocated on the first Taylor cadence)
@@ -134,6 +135,8 @@ struct rts_peel_t {
 namespace {
 
 thread_local std::string g_init_err;
+
+int predict_setup(rts_peel_t* h);
 
 int fail(rts_peel_t* h, int code, const std::string& msg) {
   if (h) h->err = msg; else g_init_err = msg;
@@ -1211,6 +1214,7 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
   int rc = RTS_OK;
   if (h->per_pass > 1) rc = ensure_block_workspace(h);
   if (rc == RTS_OK && h->precision == RTS_PREC_MIXED) rc = taylor_setup(h);
+  if (rc == RTS_OK && h->precision == RTS_PREC_MIXED) rc = predict_setup(h);
   if (rc != RTS_OK) {
     const std::string m = h->err;
     rts_peel_destroy(h);
@@ -1424,6 +1428,34 @@ int rts_peel_pipeline_wait(rts_peel_t* h) {
   return worst;
 }
 
+}  // extern "C"
+
+namespace {
+template <int QH>
+StripGrid predict_grid(const rts_peel_t* h) {
+  return strip_grid((int)std::min<int64_t>(kStWarps, (int64_t)h->n_time * ((h->n_chan + 32 * QH - 1) / (32 * QH))));
+}
+template <int QH>
+void launch_predict_strip(rts_peel_t* h, const PredictArgs& a, cudaStream_t s) {
+  const StripGrid g = predict_grid<QH>(h);
+  k_predict_strip<QH><<<(unsigned)((h->n_bl + g.bpc - 1) / g.bpc), 32u * g.wpb * g.bpc, predict_strip_smem<QH>(g), s>>>(
+      a, h->d_aph, g, (h->n_chan + 32 * QH - 1) / (32 * QH));
+}
+int predict_setup(rts_peel_t* h) {
+  const size_t bytes = (size_t)h->n_time * h->n_ant * kPredictStripSrc * sizeof(PhaseAB);
+  if (bytes > kPredictAphBytes) return RTS_OK;
+  RTS_CUDA(h, cudaFuncSetAttribute(k_predict_strip<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripMaxSmem));
+  RTS_CUDA(h, cudaFuncSetAttribute(k_predict_strip<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripMaxSmem));
+  if (cudaMalloc((void**)&h->d_aph, bytes) != cudaSuccess) {     // then by k_predict_mixed
+    cudaGetLastError();
+    h->d_aph = nullptr;
+  }
+  return RTS_OK;
+}
+}  // namespace
+
+extern "C" {
+
 int rts_peel_predict(rts_peel_t* h, void* d_vis, int32_t n_src, const double* h_src,
                      const void* d_jones, int32_t accumulate, void* stream) {
   if (!h) return fail(nullptr, RTS_EINVAL, "handle is NULL");
@@ -1440,6 +1472,27 @@ int rts_peel_predict(rts_peel_t* h, void* d_vis, int32_t n_src, const double* h_
   }
   RTS_CUDA(h, cudaMemcpyAsync(h->d_src, h_src, sizeof(double) * 3 * n_src, cudaMemcpyHostToDevice, s));
   const size_t per_src = (size_t)h->n_time * (h->precision == RTS_PREC_MIXED ? 16 : 8);
+  if (h->d_aph) {
+    for (int k0 = 0; k0 < n_src; k0 += kPredictStripSrc) {
+      PredictArgs a;
+      a.vis = d_vis; a.uvw = h->d_uvw; a.bl_ant = h->d_bl_ant; a.freq_c = h->d_freq_c;
+      a.src = h->d_src + 3 * k0;
+      a.jones = static_cast<const float2*>(d_jones) + (size_t)k0 * h->n_ant * 4;
+      a.n_src = std::min(kPredictStripSrc, n_src - k0);
+      a.n_ant = h->n_ant; a.n_chan = h->n_chan; a.n_time = h->n_time; a.n_bl = h->n_bl;
+      a.nu0_c = h->nu0 / kCLight; a.dnu_c = h->dnu / kCLight;
+      a.accumulate = (k0 > 0 || accumulate) ? 1 : 0;
+      Span span(h, RTS_K_PREDICT, s);
+      k_block_ant_phases<kPredictStripSrc><<<4 * (unsigned)h->n_sm, 256, 0, s>>>(
+          a.src, a.n_src, h->d_uvw, h->n_ant, h->n_time, a.nu0_c, a.dnu_c, h->d_aph);
+      if (h->n_chan <= 64) launch_predict_strip<2>(h, a, s);
+      else launch_predict_strip<4>(h, a, s);
+      span.end(2);
+      rc = check_launch(h, "predict kernel launch");
+      if (rc) return rc;
+    }
+    return RTS_OK;
+  }
   int chunk = (int)std::min<size_t>(kPredictChunk, std::max<size_t>(1, 40960 / per_src));
   for (int k0 = 0; k0 < n_src; k0 += chunk) {
     PredictArgs a;
@@ -1667,7 +1720,7 @@ void rts_peel_destroy(rts_peel_t* h) {
   if (cudaGetDevice(&prev) == cudaSuccess && prev != h->device) cudaSetDevice(h->device);
   void* ptrs[] = {h->d_uvw, h->d_bl_ant, h->d_freq_c, h->d_avg, h->d_J[0], h->d_J[1], h->d_Jf[0],
                   h->d_Jf[1], h->d_norms, h->d_flag, h->d_status, h->d_rel, h->d_src, h->d_jones_stage,
-                  h->b_avg, h->b_aph, h->b_model, h->b_sync, h->b_part, h->cl_V, h->cl_D, h->d_perr, h->d_tab64[0], h->d_tab64[1], h->t_mom, h->t_X[0],
+                  h->b_avg, h->b_aph, h->b_model, h->b_sync, h->b_part, h->cl_V, h->cl_D, h->d_perr, h->d_aph, h->d_tab64[0], h->d_tab64[1], h->t_mom, h->t_X[0],
                   h->t_X[1], h->t_Xf[0], h->t_Xf[1], h->t_rot_part, h->t_rot_count, h->t_rot_step};
   for (void* p : ptrs)
     if (p) cudaFree(p);

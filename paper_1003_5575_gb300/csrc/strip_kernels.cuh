@@ -94,6 +94,24 @@ __device__ __forceinline__ void strip_pack_model(float4* Mt, int e, float2 m) {
   Mt[e] = make_float4(-m.x, -m.x, -m.y, -m.y);
 }
 
+// row x of Jones matrices in a caller's array, aligned to its elements only
+__device__ __forceinline__ float4 jones_row(const void* jones, size_t x) {
+  const float2* J = static_cast<const float2*>(jones) + 2 * x;
+  const float2 a = J[0], b = J[1];
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+// S J_i J_j^H, entry (r, c), rounded to FP32; rows of J as float4
+__device__ __forceinline__ float2 model_entry_ff(float4 a, float4 b, float Sh, float Sl) {
+  const FF zero = {0.f, 0.f};
+  const FF re = ff_fma(a.w, b.w, ff_fma(a.z, b.z, ff_fma(a.y, b.y, ff_fma(a.x, b.x, zero))));
+  const FF im = ff_fma(-a.z, b.w, ff_fma(a.w, b.z, ff_fma(-a.x, b.y, ff_fma(a.y, b.x, zero))));
+  auto scale = [&](FF v) {
+    const float p = __fmul_rn(v.hi, Sh);
+    return p + fmaf(v.hi, Sl, fmaf(v.lo, Sh, fmaf(v.hi, Sh, -p)));
+  };
+  return make_float2(scale(re), scale(im));
+}
+
 // R -= sum_{k < n} M_k conj(P_k), M packed [n][kStMRow]
 template <int QH>
 __device__ __forceinline__ void strip_subtract(Strip<QH>& R, const StripTables<QH>& tb, const float4* __restrict__ Mt,

@@ -51,3 +51,36 @@ def test_strip_pass_matches_oracle(name, cad, per_pass):
     check_status(name, st, st_ref, p.rel(cad.n_src), rel_ref)
     assert torch.equal(r2, resid) and torch.equal(j2, jones)
     p.close()
+
+
+PREDICT_CASES = [
+    ("one-channel-one-source", Cadence(6, 1, 1, 1, seed=231)),
+    ("64-channels-32", Cadence(7, 64, 9, 32, seed=232)),                     # QH = 2, a warp's second strip
+    ("65-channels-33", Cadence(7, 65, 3, 33, seed=233)),
+    ("128-channels-64", Cadence(6, 128, 8, 64, seed=234)),                   # one full launch
+    ("129-channels-65", Cadence(6, 129, 2, 65, seed=235)),                   # two launches, a second tile of one channel
+    ("300-channels", Cadence(5, 300, 5, 100, seed=236)),
+]
+
+
+@pytest.mark.parametrize("name,cad", PREDICT_CASES, ids=[c[0] for c in PREDICT_CASES])
+def test_strip_prediction_matches_oracle(name, cad):
+    J = cad.jones().astype(np.complex64)
+    ref = oracle.predict(cad.uvw(), cad.freqs(), cad.sources(), J.astype(np.complex128))
+    p = make_peeler(cad, "mixed")
+    got = p.predict(cad.sources(), torch.from_numpy(J).cuda())
+    base = torch.ones(p.cube_shape, dtype=torch.complex64, device="cuda")
+    added = p.predict(cad.sources(), torch.from_numpy(J).cuda(), out=base, accumulate=True)
+    assert np.abs(got.cpu().numpy() - ref).max() <= TOL["mixed"] * rms_of(ref)
+    assert np.abs(added.cpu().numpy() - (ref + 1.0)).max() <= TOL["mixed"] * rms_of(ref) + 1e-6
+    p.close()
+
+
+def test_strip_prediction_takes_gains_on_an_element_boundary():
+    cad = Cadence(7, 33, 2, 3, seed=237)
+    J = torch.from_numpy(cad.jones().astype(np.complex64)).cuda()
+    odd = torch.empty(J.numel() + 1, dtype=J.dtype, device="cuda")[1:].view(J.shape).copy_(J)
+    assert odd.data_ptr() % 16 == 8
+    p = make_peeler(cad, "mixed")
+    assert torch.equal(p.predict(cad.sources(), odd), p.predict(cad.sources(), J))
+    p.close()
