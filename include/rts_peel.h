@@ -38,7 +38,8 @@
  * _predict, _rotate_average and _solve allocate nothing.  Two workspaces whose
  * size depends on how the handle is used are allocated on first use and kept:
  * the adjoint's (first rts_peel_grad or rts_peel_offsets: 88 bytes per
- * baseline for each of max_sources sources) and the pipeline's two
+ * baseline and, in RTS_PREC_MIXED, 16 bytes per antenna and time for each of
+ * max_sources sources) and the pipeline's two
  * device cubes and page-locked staging (first rts_peel_pipeline_submit); a
  * warm-up call before real-time use moves that allocation out of the loop.  Calls are asynchronous on `stream` (a cudaStream_t, NULL
  * = legacy default stream) unless an h_status pointer is given, which makes
@@ -112,10 +113,11 @@ typedef struct rts_peel_config {
                            results agree to FP32 rounding (statuses outside a band
                            around 1e-6). */
   int32_t grad_kernel;   /* RTS_PREC_MIXED adjoint (rts_peel_grad, rts_peel_offsets):
-                           RTS_GRAD_AUTO (0: phasors factorised per 16-channel group into
-                           two shared-memory tables, T1[q] T2[r], when the tables of all
-                           n_src sources fit in shared memory, about n_src <= 580 on
-                           GB300; otherwise as RTS_GRAD_DIRECT), RTS_GRAD_DIRECT (1: one
+                           RTS_GRAD_AUTO (0: a warp per baseline, time and 256 channels,
+                           phasors factorised per 16-channel tile, T1[q] T2[r], 32
+                           sources' tables at a time, when the model matrices and totals
+                           of all n_src sources fit in shared memory, about n_src <= 1000
+                           on GB300; otherwise as RTS_GRAD_DIRECT), RTS_GRAD_DIRECT (1: one
                            hardware sin/cos per source and sample).  FP32-level accuracy
                            either way; RTS_PREC_FP64 always evaluates every phasor in FP64. */
   int32_t band_n_chan;   /* channel sharding (Section 3.1: channel groups on separate

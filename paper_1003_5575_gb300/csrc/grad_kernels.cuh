@@ -26,6 +26,7 @@
 
 #include "common.cuh"
 #include "kahan.cuh"
+#include "strip_kernels.cuh"
 
 namespace rts {
 
@@ -43,6 +44,8 @@ struct GradWorkspace {
   double* gsc = nullptr;    // [K][n_bl][3] (dl, dm, dS contributions)
   double* loss_bl = nullptr;// [n_bl]
   DirQ* dir = nullptr;   // [K] (l, m, nm1, S)
+  PhaseAB* aph = nullptr;   // [n_time][n_ant][kp] antenna phases (FP32 sweep), kp = K rounded up to 32
+  float4* lmn = nullptr;    // [kp] l / n and m / n, each as a pair of floats
   double* wchan = nullptr;  // [n_chan] per-channel weight of the position derivative (offsets)
 };
 
@@ -62,12 +65,16 @@ struct GradArgs {
   double nu0_c, dnu_c;
 };
 
-__global__ void k_grad_dirs(const double* __restrict__ src, int n, DirQ* __restrict__ dir) {
+__global__ void k_grad_dirs(const double* __restrict__ src, int n, DirQ* __restrict__ dir, float4* __restrict__ lmn) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n) {
     double l = src[3 * k], m = src[3 * k + 1], S = src[3 * k + 2];
     double r2 = l * l + m * m;
-    dir[k] = DirQ{l, m, -r2 / (1.0 + sqrt(1.0 - r2)), S};
+    const double nm1 = -r2 / (1.0 + sqrt(1.0 - r2));
+    dir[k] = DirQ{l, m, nm1, S};
+    const double ln = l / (1.0 + nm1), mn = m / (1.0 + nm1);
+    const float lh = (float)ln, mh = (float)mn;
+    lmn[k] = make_float4(lh, (float)(ln - (double)lh), mh, (float)(mn - (double)mh));
   }
 }
 
@@ -261,258 +268,338 @@ __global__ void __launch_bounds__(kGradThreads) k_grad_sweep(GradArgs a) {
   if (bw && my_g == 0) grad_store<T>(a, k0 + my_k, bl, ij, G, Hl, Hm);
 }
 
-// exp(+2 pi i x) of a Q0.64 phase x rounded to Q0.32 (the hardware sin/cos,
-// as the per-sample sweep uses for every sample)
-__device__ inline float2 grad_phasor_tab(unsigned long long ph) { return phasor_f(q64_to_turns(ph)); }
+// The FP32 adjoint on strips (strip_kernels.cuh).  One CTA per baseline; a warp
+// takes one (time, tile of 256 channels) strip of it through both halves:
+//   forward   R = V - sum_k M_k conj(T1_k[q] T2_k[r]) in registers, lane = its
+//             channels, 32 sources' phasor tables at a time in shared memory;
+//   backward  lane = source, R read by broadcast from shared-memory planes:
+//             sum_c R(c) P_k(c) = sum_q T1_k[q] s_q,  s_q = sum_r x_r, x_r = R(16q + r) T2_k[r],
+//             sum_c c R(c) P_k(c) = sum_q T1_k[q] [(c0 + 16q - 1) s_q + a_q],
+//             a_q = sum_r (r + 1) x_r, the running sum of the suffix sums while r
+//             runs down from 15 (c0 the tile's first channel).
+// A (source, channel) pair costs 20 multiply-adds in the forward half and 24 in
+// the backward one, two a packed instruction; the FP32 pipe bounds it (66 % busy,
+// 56 % of the issue slots, at 100 sources, 128 antennas x 256 channels x 8 times).
+// Where a lane had stood for each (source, channel) with every phasor and sum formed
+// apart (62 instructions a pair) that size took 5.96 ms, this takes 3.27; 300
+// sources, 512 antennas x 768 channels x 8 times with the reductions: 607 and 463 ms.
+// The last group's lanes share out the tiles when 16 sources or fewer are left (100
+// sources: a quarter of the backward half was idle lanes).  The
+// position derivative is contracted with M per strip (one number instead of two
+// complex 2x2 sums a direction).  After each group of 32 sources the CTA's warps
+// meet once and their ten sums a source are added, in warp order, to compensated
+// FP32 totals (two stages, so that one barrier a group is enough).
+constexpr int kGsQh = 8;
+constexpr int kGsTile = 32 * kGsQh;       // channels of a strip
+constexpr int kGsPitch = 17;              // float4 from tile to tile: the lanes of several tiles read other banks
+constexpr int kGsMaxWarps = 12;           // of one CTA an SM: 168 registers a thread
+constexpr int kGsPairWarps = 8;           // of each of two: 128 registers
+constexpr size_t kGsPairSmem = 112 * 1024;
+// Two CTAs of 8 warps against one of 12: 463 and 470 ms at 300 sources, where the
+// totals leave shared memory to make room for the second; at 100 sources two CTAs,
+// the sharing of the last group and k_grad_jones's reduction took 4.57 ms to 3.56
+constexpr int kGsVals = 10;               // per source: G (8), l, m
 
-// The FP32 adjoint with factorised phasors.  Within a tile of kGfTile channels
-// starting at c0, channel c = c0 + 16 q + r has
-//   exp(+2 pi i phi_k(c)) = T1_k[q] T2_k[r],
-//   T1_k[q] = exp(2 pi i (A_k + (c0 + 16 q) B_k)),  T2_k[r] = exp(2 pi i r B_k)
-// (A_k, B_k the Q0.64 phase at channel 0 and its per-channel step), so both
-// halves of the sweep multiply table entries instead of evaluating sin/cos:
-//   forward   R(c) = V(c) - sum_k M_k conj(T1_k[q] T2_k[r])   (thread = channel)
-//   backward  sum_c R(c) P_k(c) = sum_q T1_k[q] s_q,  s_q = sum_r R(16q + r) T2_k[r]
-//             sum_c c R(c) P_k(c) = sum_q T1_k[q] [(c0 + 16q - 1) s_q + a_q]
-//             with a_q = sum_r (r + 1) x_r, x_r = R(16q + r) T2_k[r], built as
-//             the running sum of the suffix sums while r runs down from 15
-//             (thread = (source, group of q)).
-// Tables are [q or r][kp] with kp = 1 (mod 16): the forward's 16 distinct r of
-// a warp and the backward's consecutive sources fall on distinct banks.  The
-// per-(source, baseline) outputs are those of k_grad_sweep.
-constexpr int kGfThreads = 384;
-constexpr int kGfTile = 384;          // channels per tile: one per thread in the forward
-constexpr int kGfNq = kGfTile / 16;
-constexpr int kGfChunk = kGfThreads;  // sources per CTA in the backward
-
-__host__ __device__ inline int grad_fac_kp(int n_src) { return ((n_src + 15) / 16) * 16 + 1; }
-
-inline size_t grad_fac_smem_bytes(int n_src) {
-  const size_t kp = (size_t)grad_fac_kp(n_src);
-  return (size_t)kGfTile * 4 * sizeof(float2)           // R
-         + (size_t)n_src * 4 * sizeof(float2)            // M
-         + (size_t)kGfThreads * 16 * sizeof(float)        // backward partials
-         + (size_t)(kGfNq + 16) * kp * sizeof(float2)     // T1, T2
-         + (size_t)n_src * 2 * sizeof(unsigned long long) // A, B
-         + (size_t)kGfTile * sizeof(float);               // channel weights of the tile
+__host__ __device__ inline int grad_kp(int n_src) { return (n_src + kStGrp - 1) / kStGrp * kStGrp; }
+template <bool WEIGHTED> __host__ __device__ constexpr size_t grad_strip_warp_bytes() {
+  constexpr size_t planes = (size_t)4 * kGsQh * kGsPitch * sizeof(float4);
+  return (planes > strip_warp_bytes<kGsQh>() ? planes : strip_warp_bytes<kGsQh>()) + (WEIGHTED ? kGsTile * sizeof(float) : 0);
+}
+// sine table | model matrices [Kp][kStMRow] float4 | (tot) totals and compensations
+// [2][kGsVals][Kp] | two stages [2][warps][kGsVals][32] | a workspace per warp
+template <bool WEIGHTED> inline size_t grad_strip_smem(int n_src, int warps, bool tot) {
+  const size_t kp = grad_kp(n_src);
+  return 256 * sizeof(float2) + kp * kStMRow * sizeof(float4) + (tot ? 2 * kGsVals * kp * sizeof(float) : 0) +
+         (size_t)warps * (2 * kGsVals * kStGrp * sizeof(float) + grad_strip_warp_bytes<WEIGHTED>());
+}
+// Warps of a CTA: as few rounds over the baseline's strips as `most` gives, then
+// as few warps as those rounds need; fewer where the sources' tables leave no
+// room in `room` bytes.  0: they do not fit.
+template <bool WEIGHTED>
+inline int grad_strip_warps(int n_src, int n_chan, int n_time, int most, size_t room, bool tot) {
+  const int64_t strips = (int64_t)n_time * ((n_chan + kGsTile - 1) / kGsTile);
+  const int64_t rounds = (strips + most - 1) / most;
+  int w = (int)((strips + rounds - 1) / rounds);
+  const int least = w < 4 ? w : 4;
+  while (w >= least && grad_strip_smem<WEIGHTED>(n_src, w, tot) > room) --w;
+  return w >= least ? w : 0;
 }
 
+// the antennas' Q0.64 phases of every source, [n_time][n_ant][kp]
+__global__ void __launch_bounds__(256) k_grad_ant_phases(const DirQ* __restrict__ dir, int n_src, int kp,
+                                                        const double* __restrict__ uvw, int n_ant, int n_time,
+                                                        double nu0_c, double dnu_c, PhaseAB* __restrict__ aph) {
+  const int64_t n = (int64_t)n_time * n_ant * kp;
+  for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t ti = x / kp;
+    const int k = (int)(x - ti * kp);
+    PhaseAB p;
+    p.a = 0; p.b = 0;
+    if (k < n_src) {
+      const DirQ d = dir[k];
+      const double* u = uvw + ti * 3;
+      const double tau = u[0] * d.x + u[1] * d.y + u[2] * d.z;
+      p.a = frac_q64(tau * nu0_c);
+      p.b = frac_q64(tau * dnu_c);
+    }
+    aph[x] = p;
+  }
+}
+
+// sums of this lane's source over a strip's planes: y0 = sum R P, y1 = sum w R P with
+// w the channel number (WEIGHTED: the table wt), as (re 0, re 1), (re 2, re 3), (im ..)
 template <bool WEIGHTED>
-__global__ void __launch_bounds__(kGfThreads, 1) k_grad_sweep_fac(GradArgs a) {
-  extern __shared__ __align__(16) unsigned char g_smem[];
-  const int K = a.n_src;
-  const int kp = grad_fac_kp(K);
-  float2* sR = reinterpret_cast<float2*>(g_smem);                  // [kGfTile][4]
-  float2* sM = sR + kGfTile * 4;                                   // [K][4]
-  float* sPart = reinterpret_cast<float*>(sM + (size_t)K * 4);     // [16][threads]
-  float2* sT1 = reinterpret_cast<float2*>(sPart + (size_t)kGfThreads * 16);   // [kGfNq][kp]
-  float2* sT2 = sT1 + (size_t)kGfNq * kp;                          // [16][kp]
-  unsigned long long* sA = reinterpret_cast<unsigned long long*>(sT2 + (size_t)16 * kp);
-  unsigned long long* sB = sA + K;
-  float* sW = reinterpret_cast<float*>(sB + K);                    // [kGfTile]
-  __shared__ double s_uvw[3];
-  __shared__ double s_loss[kGfThreads / 32];
-
-  const int tid = threadIdx.x;
-  const int64_t bl = blockIdx.x;
-  const int2 ij = a.bl_ant[bl];
-  const int k0 = blockIdx.y * kGfChunk;
-  const int kc = max(1, min(kGfChunk, K - k0));            // sources of this CTA's backward phase
-  const int groups = max(1, min(kGfNq, kGfThreads / kc));
-  const int my_k = tid % kc, my_g = tid / kc;
-  const bool bw = my_g < groups && k0 + my_k < K;
-  const int kb = k0 + my_k;                                 // source of the backward item
-  const int qa = my_g * kGfNq / groups, qb = (my_g + 1) * kGfNq / groups;
-
-  for (int k = tid; k < K; k += kGfThreads) {
-    M22<double2> Ji, Jj;
-    #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float2 p = load_j<float>(a.jones, ((size_t)k * a.n_ant + ij.x) * 4 + e);
-      float2 q = load_j<float>(a.jones, ((size_t)k * a.n_ant + ij.y) * 4 + e);
-      Ji.e[e] = make_double2(p.x, p.y); Jj.e[e] = make_double2(q.x, q.y);
-    }
-    M22<double2> P = mmul_h(Ji, Jj);
-    const double S = a.dir[k].w;
-    #pragma unroll
-    for (int e = 0; e < 4; ++e) sM[(size_t)k * 4 + e] = make_float2((float)(S * P.e[e].x), (float)(S * P.e[e].y));
-  }
-  // per-(source, baseline) sums over tiles, compensated FP32 (the FP64 pipe
-  // is far slower than FP32 on this part; 2 x n_time terms per sum)
-  float G[8], Hl[8], Hm[8], Gc[8], Hlc[8], Hmc[8];
+__device__ __forceinline__ void grad_strip_average(const float4* __restrict__ pre, const float4* __restrict__ pim,
+                                                   const float* __restrict__ wt, int nq, int c0, int part,
+                                                   int parts, PhaseAB p, const float2* lut, float2 (&y0)[4], float2 (&y1)[4]) {
+  float2 t2[16];
   #pragma unroll
-  for (int e = 0; e < 8; ++e) { G[e] = Hl[e] = Hm[e] = Gc[e] = Hlc[e] = Hmc[e] = 0.f; }
-  double loss = 0.0;
-  double lk_n = 0.0, mk_n = 0.0;
-  if (bw) {
-    const DirQ d = a.dir[kb];
-    const double n = 1.0 + d.z;
-    lk_n = d.x / n; mk_n = d.y / n;
+  for (int r = 0; r < 16; ++r) t2[r] = phasor_lut((unsigned long long)r * p.b, lut);
+  #pragma unroll
+  for (int i = 0; i < 4; ++i) y0[i] = y1[i] = make_float2(0.f, 0.f);
+  const unsigned long long step = (unsigned long long)(16 * parts) * p.b;
+  unsigned long long ph = p.a + (unsigned long long)(16 * part) * p.b;
+  pre += kGsPitch * part;
+  pim += kGsPitch * part;
+  #pragma unroll 1
+  for (int q = part; q < nq; q += parts, ph += step, pre += kGsPitch * parts, pim += kGsPitch * parts) {
+    float2 s0[4], s1[4];
+    #pragma unroll
+    for (int i = 0; i < 4; ++i) s0[i] = s1[i] = make_float2(0.f, 0.f);
+    #pragma unroll
+    for (int r = 15; r >= 0; --r) {
+      const float4 a = pre[r], b = pim[r];
+      const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w);
+      const float2 b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
+      const float2 tx = make_float2(t2[r].x, t2[r].x), ty = make_float2(t2[r].y, t2[r].y);
+      const float ny = __uint_as_float(__float_as_uint(t2[r].y) ^ 0x80000000u);
+      const float2 nty = make_float2(ny, ny);
+      if (WEIGHTED) {
+        const float w = wt[16 * q + r];
+        const float2 w2 = make_float2(w, w);
+        const float2 x[4] = {ffma2(a0, tx, fmul2(b0, nty)), ffma2(a1, tx, fmul2(b1, nty)),
+                             ffma2(a0, ty, fmul2(b0, tx)), ffma2(a1, ty, fmul2(b1, tx))};
+        #pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          s0[i] = fadd2(s0[i], x[i]);
+          s1[i] = ffma2(x[i], w2, s1[i]);
+        }
+      } else {
+        s0[0] = ffma2(a0, tx, ffma2(b0, nty, s0[0]));
+        s0[1] = ffma2(a1, tx, ffma2(b1, nty, s0[1]));
+        s0[2] = ffma2(a0, ty, ffma2(b0, tx, s0[2]));
+        s0[3] = ffma2(a1, ty, ffma2(b1, tx, s0[3]));
+        #pragma unroll
+        for (int i = 0; i < 4; ++i) s1[i] = fadd2(s1[i], s0[i]);
+      }
+    }
+    if (!WEIGHTED) {
+      const float cw = (float)(c0 + 16 * q - 1);
+      const float2 c2 = make_float2(cw, cw);
+      #pragma unroll
+      for (int i = 0; i < 4; ++i) s1[i] = ffma2(s0[i], c2, s1[i]);
+    }
+    const float2 t1 = phasor_lut(ph, lut);
+    const float2 x = make_float2(t1.x, t1.x), y = make_float2(t1.y, t1.y), ny = make_float2(-t1.y, -t1.y);
+    #pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      y0[i] = ffma2(s0[i], x, ffma2(s0[2 + i], ny, y0[i]));
+      y0[2 + i] = ffma2(s0[i], y, ffma2(s0[2 + i], x, y0[2 + i]));
+      y1[i] = ffma2(s1[i], x, ffma2(s1[2 + i], ny, y1[i]));
+      y1[2 + i] = ffma2(s1[i], y, ffma2(s1[2 + i], x, y1[2 + i]));
+    }
   }
+  for (int o = 32 / parts; o < 32; o <<= 1)          // the parts of a source
+    #pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      y0[i] = fadd2(y0[i], make_float2(__shfl_xor_sync(0xffffffffu, y0[i].x, o), __shfl_xor_sync(0xffffffffu, y0[i].y, o)));
+      y1[i] = fadd2(y1[i], make_float2(__shfl_xor_sync(0xffffffffu, y1[i].x, o), __shfl_xor_sync(0xffffffffu, y1[i].y, o)));
+    }
+}
 
-  for (int t = 0; t < a.n_time; ++t) {
-    __syncthreads();                              // previous users of sA/sB/sT2/s_uvw done
-    for (int k = tid; k < K; k += kGfThreads) {
-      SrcDir d; d.l = a.dir[k].x; d.m = a.dir[k].y; d.nm1 = a.dir[k].z; d.S = a.dir[k].w;
-      const double tau = delay_m(a.uvw, a.n_ant, t, ij.x, ij.y, d);
-      sA[k] = frac_q64(tau * a.nu0_c); sB[k] = frac_q64(tau * a.dnu_c);
+template <bool WEIGHTED, int WARPS, bool TOT>
+__global__ void __launch_bounds__(WARPS * 32, WARPS == kGsPairWarps ? 2 : 1) k_grad_strip(GradArgs a, const PhaseAB* __restrict__ aph,
+                                                                   const float4* __restrict__ lmn) {
+  extern __shared__ __align__(16) unsigned char g_smem[];
+  const int K = a.n_src, kp = grad_kp(K);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthr = blockDim.x, nw = nthr >> 5;
+  const int64_t bl = blockIdx.x;
+  float2* lut = reinterpret_cast<float2*>(g_smem);
+  float4* Mt = reinterpret_cast<float4*>(lut + 256);                           // [kp][kStMRow]
+  float* tot = reinterpret_cast<float*>(Mt + (size_t)kp * kStMRow);             // [2][kGsVals][kp]
+  float* stage = tot + (TOT ? (size_t)2 * kGsVals * kp : 0);                    // [2][nw][kGsVals][32]
+  // value v's total and compensation of source k: in shared memory, or (TOT false) in
+  // the words of this baseline's own results
+  auto total = [&](int v, int k) -> float* {
+    if (TOT) return tot + v * kp + k;
+    const size_t at = (size_t)k * a.n_bl + bl;
+    return v < 8 ? reinterpret_cast<float*>(a.G + at * 4) + v : reinterpret_cast<float*>(a.gsc + at * 3) + (v - 8);
+  };
+  auto total_comp = [&](int v, int k) -> float* {
+    if (TOT) return tot + (kGsVals + v) * kp + k;
+    return total(v, k) + (v < 8 ? 8 : 2);
+  };
+  unsigned char* ws = reinterpret_cast<unsigned char*>(stage + (size_t)2 * nw * kGsVals * kStGrp) +
+                      (size_t)warp * grad_strip_warp_bytes<WEIGHTED>();
+  StripTables<kGsQh>& tb = *reinterpret_cast<StripTables<kGsQh>*>(ws);
+  float4* pre = reinterpret_cast<float4*>(ws);
+  float4* pim = pre + 2 * kGsQh * kGsPitch;
+  float* wt = reinterpret_cast<float*>(ws + grad_strip_warp_bytes<false>());         // WEIGHTED only
+  __shared__ double s_loss[WARPS];
+  const int2 ij = a.bl_ant[bl];
+  lut_fill(lut, tid, nthr);
+  for (int i = tid; i < kp * 4; i += nthr) {
+    const int k = i >> 2, e = i & 3;
+    float2 m = make_float2(0.f, 0.f);
+    if (k < K) {
+      const double S = a.dir[k].w;
+      const float Sh = (float)S, Sl = (float)(S - (double)Sh);
+      const size_t at = (size_t)k * a.n_ant;
+      m = model_entry_ff(jones_row(a.jones, 2 * (at + ij.x) + (e >> 1)), jones_row(a.jones, 2 * (at + ij.y) + (e & 1)),
+                         Sh, Sl);
     }
-    if (tid < 3)
-      s_uvw[tid] = a.uvw[((size_t)t * a.n_ant + ij.x) * 3 + tid] - a.uvw[((size_t)t * a.n_ant + ij.y) * 3 + tid];
-    __syncthreads();
-    for (int k = tid; k < K; k += kGfThreads) {
-      const unsigned long long b = sB[k];
-      #pragma unroll 4
-      for (int r = 0; r < 16; ++r) sT2[(size_t)r * kp + k] = grad_phasor_tab((unsigned long long)r * b);
-    }
-    for (int c0 = 0; c0 < a.n_chan; c0 += kGfTile) {
-      const int nc = min(kGfTile, a.n_chan - c0);
-      const int nq = (nc + 15) / 16;
-      for (int k = tid; k < K; k += kGfThreads) {
-        const unsigned long long b = sB[k], a0 = sA[k] + (unsigned long long)c0 * b;
-        #pragma unroll 4
-        for (int q = 0; q < nq; ++q) sT1[(size_t)q * kp + k] = grad_phasor_tab(a0 + (unsigned long long)(16 * q) * b);
-      }
-      if (WEIGHTED)
-        for (int i = tid; i < nc; i += kGfThreads) sW[i] = (float)a.wchan[c0 + i];
-      __syncthreads();
-      // forward: R at channel c0 + tid, all sources subtracted
-      if (tid < nc) {
-        const int q = tid >> 4, r = tid & 15;
-        const float4* v = reinterpret_cast<const float4*>(
-            static_cast<const float2*>(a.vis) + (((size_t)t * a.n_bl + bl) * a.n_chan + c0 + tid) * 4);
-        const float4 v0 = v[0], v1 = v[1];
-        float ax[4] = {v0.x, v0.z, v1.x, v1.z}, ay[4] = {v0.y, v0.w, v1.y, v1.w};
-        const float2* t1p = sT1 + (size_t)q * kp;
-        const float2* t2p = sT2 + (size_t)r * kp;
-        #pragma unroll 4
-        for (int k = 0; k < K; ++k) {
-          const float2 t1 = t1p[k], t2 = t2p[k];
-          const float px = fmaf(t1.x, t2.x, -t1.y * t2.y);
-          const float py = fmaf(t1.x, t2.y, t1.y * t2.x);
-          const float4 m01 = reinterpret_cast<const float4*>(sM)[2 * k];
-          const float4 m23 = reinterpret_cast<const float4*>(sM)[2 * k + 1];
-          const float mx[4] = {m01.x, m01.z, m23.x, m23.z}, my[4] = {m01.y, m01.w, m23.y, m23.w};
-          #pragma unroll
-          for (int e = 0; e < 4; ++e) {          // R -= M conj(P)
-            ax[e] = fmaf(-mx[e], px, fmaf(-my[e], py, ax[e]));
-            ay[e] = fmaf(-my[e], px, fmaf(mx[e], py, ay[e]));
-          }
-        }
-        float4* o = reinterpret_cast<float4*>(sR + (size_t)tid * 4);
-        o[0] = make_float4(ax[0], ay[0], ax[1], ay[1]);
-        o[1] = make_float4(ax[2], ay[2], ax[3], ay[3]);
-        float l2 = 0.f;
-        #pragma unroll
-        for (int e = 0; e < 4; ++e) l2 = fmaf(ax[e], ax[e], fmaf(ay[e], ay[e], l2));
-        loss += (double)l2;
-      }
-      __syncthreads();
-      // backward: this thread's source over its q groups
-      if (bw) {
-        float y0[8], y1[8];
-        #pragma unroll
-        for (int e = 0; e < 8; ++e) { y0[e] = 0.f; y1[e] = 0.f; }
-        for (int q = qa; q < min(qb, nq); ++q) {
-          const int rv = min(16, nc - 16 * q);
-          float s0[8], s1[8];
-          #pragma unroll
-          for (int e = 0; e < 8; ++e) { s0[e] = 0.f; s1[e] = 0.f; }
-          auto step = [&](int r) {
-            const int cl = 16 * q + r;
-            const float4 ra = reinterpret_cast<const float4*>(sR)[2 * cl];
-            const float4 rb = reinterpret_cast<const float4*>(sR)[2 * cl + 1];
-            const float rx[4] = {ra.x, ra.z, rb.x, rb.z}, ry[4] = {ra.y, ra.w, rb.y, rb.w};
-            const float2 t2 = sT2[(size_t)r * kp + kb];
-            if (WEIGHTED) {
-              const float w = sW[cl];
-              #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float xr = fmaf(rx[e], t2.x, -ry[e] * t2.y);
-                const float xi = fmaf(rx[e], t2.y, ry[e] * t2.x);
-                s0[2 * e] += xr; s0[2 * e + 1] += xi;
-                s1[2 * e] = fmaf(w, xr, s1[2 * e]); s1[2 * e + 1] = fmaf(w, xi, s1[2 * e + 1]);
-              }
-            } else {
-              #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                s0[2 * e] = fmaf(rx[e], t2.x, fmaf(-ry[e], t2.y, s0[2 * e]));
-                s0[2 * e + 1] = fmaf(rx[e], t2.y, fmaf(ry[e], t2.x, s0[2 * e + 1]));
-              }
-              #pragma unroll
-              for (int e = 0; e < 8; ++e) s1[e] += s0[e];
-            }
-          };
-          if (rv == 16) {
-            #pragma unroll
-            for (int r = 15; r >= 0; --r) step(r);
-          } else {
-            for (int r = rv - 1; r >= 0; --r) step(r);
-          }
-          const float2 t1 = sT1[(size_t)q * kp + kb];
-          const float cw = (float)(c0 + 16 * q - 1);
-          #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            y0[2 * e] = fmaf(t1.x, s0[2 * e], fmaf(-t1.y, s0[2 * e + 1], y0[2 * e]));
-            y0[2 * e + 1] = fmaf(t1.x, s0[2 * e + 1], fmaf(t1.y, s0[2 * e], y0[2 * e + 1]));
-            // unweighted: sum_r (c0 + 16q + r) x_r = (c0 + 16q - 1) s0 + sum_r (r + 1) x_r
-            const float zr = WEIGHTED ? s1[2 * e] : fmaf(cw, s0[2 * e], s1[2 * e]);
-            const float zi = WEIGHTED ? s1[2 * e + 1] : fmaf(cw, s0[2 * e + 1], s1[2 * e + 1]);
-            y1[2 * e] = fmaf(t1.x, zr, fmaf(-t1.y, zi, y1[2 * e]));
-            y1[2 * e + 1] = fmaf(t1.x, zi, fmaf(t1.y, zr, y1[2 * e + 1]));
-          }
-        }
-        #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          sPart[e * kGfThreads + tid] = y0[e];
-          sPart[(8 + e) * kGfThreads + tid] = y1[e];
-        }
-      }
-      __syncthreads();
-      if (bw && my_g == 0) {
-        float H0[8], H1[8];
-        #pragma unroll
-        for (int e = 0; e < 8; ++e) { H0[e] = 0.f; H1[e] = 0.f; }
-        for (int g = 0; g < groups; ++g) {
-          const float* part = sPart + g * kc + my_k;
-          #pragma unroll
-          for (int e = 0; e < 8; ++e) { H0[e] += part[e * kGfThreads]; H1[e] += part[(8 + e) * kGfThreads]; }
-        }
-        const float wl = (float)(s_uvw[0] - s_uvw[2] * lk_n);
-        const float wm = (float)(s_uvw[1] - s_uvw[2] * mk_n);
-        const float nu0 = (float)a.nu0_c, dnu = (float)a.dnu_c;
-        #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float hn = WEIGHTED ? H1[e] : fmaf(nu0, H0[e], dnu * H1[e]);
-          kahan_add(G[e], Gc[e], H0[e]);
-          kahan_add(Hl[e], Hlc[e], wl * hn);
-          kahan_add(Hm[e], Hmc[e], wm * hn);
-        }
-      }
-    }
-  }
-  if (blockIdx.y == 0) {
-    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-    if ((tid & 31) == 0) s_loss[tid >> 5] = loss;
+    strip_pack_model(Mt + (size_t)k * kStMRow, e, m);
   }
   __syncthreads();
-  if (blockIdx.y == 0 && tid == 0) {
-    double s = 0.0;
-    for (int w = 0; w < kGfThreads / 32; ++w) s += s_loss[w];
-    a.loss_bl[bl] = s;
-  }
-  if (bw && my_g == 0) {
-    double Gd[8], Hld[8], Hmd[8];
+  const int n_tile = (a.n_chan + kGsTile - 1) / kGsTile, n_strip = a.n_time * n_tile;
+  const float nu0 = (float)a.nu0_c, dnu = (float)a.dnu_c;
+  FF loss = {0.f, 0.f};
+  int buf = 0;
+  for (int s0 = 0; s0 < n_strip; s0 += nw) {
+    const int s = s0 + warp, n_act = min(nw, n_strip - s0);
+    const bool active = warp < n_act;
+    const int t = active ? s / n_tile : 0, c0 = active ? (s - t * n_tile) * kGsTile : 0;
+    const int nc = min(kGsTile, a.n_chan - c0), nq = (nc + 15) >> 4, np = (nq + 1) >> 1;
+    const size_t ai = ((size_t)t * a.n_ant + ij.x) * kp, aj = ((size_t)t * a.n_ant + ij.y) * kp;
+    auto phase = [&](int k) {                  // of source k at channel c0
+      const PhaseAB x = aph[ai + k], y = aph[aj + k];
+      PhaseAB p;
+      p.b = x.b - y.b;
+      p.a = x.a - y.a + (unsigned long long)c0 * p.b;
+      return p;
+    };
+    // baseline (u, v, w) at t as float pairs
+    FF u3[3];
     #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      Gd[e] = (double)G[e] - (double)Gc[e];
-      Hld[e] = (double)Hl[e] - (double)Hlc[e];
-      Hmd[e] = (double)Hm[e] - (double)Hmc[e];
+    for (int i = 0; i < 3; ++i) {
+      const double u = a.uvw[((size_t)t * a.n_ant + ij.x) * 3 + i] - a.uvw[((size_t)t * a.n_ant + ij.y) * 3 + i];
+      u3[i].hi = (float)u;
+      u3[i].lo = (float)(u - (double)u3[i].hi);
     }
-    grad_store<float>(a, kb, bl, ij, Gd, Hld, Hmd);
+    if (active) {
+      Strip<kGsQh> R;
+      strip_load(R, static_cast<const float4*>(a.vis) + (((size_t)t * a.n_bl + bl) * a.n_chan + c0) * 2, nc, lane);
+      for (int k0 = 0; k0 < K; k0 += kStGrp) {
+        const PhaseAB p = phase(k0 + lane);
+        __syncwarp();
+        strip_tables<kGsQh>(tb, p, lane, np, lut);
+        __syncwarp();
+        strip_subtract<kGsQh>(R, tb, Mt + (size_t)k0 * kStMRow, min(kStGrp, K - k0), lane);
+      }
+      __syncwarp();
+      strip_planes<kGsQh, kGsPitch>(R, pre, pim, nc, lane);
+      const int cl = 16 * (lane >> 4) * kGsQh + (lane & 15);
+      #pragma unroll
+      for (int u = 0; u < kGsQh; ++u) {
+        float re[4], im[4], l2 = 0.f;
+        strip_channel(R, u, re, im);
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) l2 = fmaf(re[e], re[e], fmaf(im[e], im[e], l2));
+        if (cl + 16 * u < nc) {
+          const FF x = ff_two_sum(loss.hi, l2);
+          loss.hi = x.hi;
+          loss.lo += x.lo;
+        }
+        if (WEIGHTED) wt[cl + 16 * u] = cl + 16 * u < nc ? (float)a.wchan[c0 + cl + 16 * u] : 0.f;
+      }
+      __syncwarp();
+    }
+    for (int k0 = 0; k0 < K; k0 += kStGrp, buf ^= 1) {
+      float* st = stage + (size_t)buf * nw * kGsVals * kStGrp;
+      if (active) {
+        float2 y0[4], y1[4];
+        // a group of 16 sources or fewer: several lanes a source, each some of the tiles
+        const int n = K - k0, parts = n > 16 ? 1 : n > 8 ? 2 : n > 4 ? 4 : 8, kl = lane & (32 / parts - 1);
+        grad_strip_average<WEIGHTED>(pre, pim, wt, nq, c0, lane / (32 / parts), parts, phase(k0 + kl), lut, y0, y1);
+        float* o = st + (size_t)warp * kGsVals * kStGrp + lane;
+        #pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          o[(2 * i) * kStGrp] = y0[i].x;
+          o[(2 * i + 1) * kStGrp] = y0[i].y;
+        }
+        // z = Im sum_e conj(h_e) M_e, h = sum R P (d phi / d shift) / a_p
+        const float4* m = Mt + (size_t)(k0 + kl) * kStMRow;      // (-re, -re, -im, -im)
+        FF z = {0.f, 0.f};
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float hr0 = e & 1 ? y0[e >> 1].y : y0[e >> 1].x, hi0 = e & 1 ? y0[2 + (e >> 1)].y : y0[2 + (e >> 1)].x;
+          const float hr1 = e & 1 ? y1[e >> 1].y : y1[e >> 1].x, hi1 = e & 1 ? y1[2 + (e >> 1)].y : y1[2 + (e >> 1)].x;
+          const float hr = WEIGHTED ? hr1 : fmaf(nu0, hr0, dnu * hr1), hi = WEIGHTED ? hi1 : fmaf(nu0, hi0, dnu * hi1);
+          const float4 me = m[e];
+          z = ff_fma(-hr, me.z, z);                    // hr Im M
+          z = ff_fma(hi, me.x, z);                     // - hi Re M
+        }
+        const float zf = z.hi + z.lo;
+        const float4 ln = lmn[k0 + kl];                // l / n, m / n as float pairs
+        auto arm = [&](FF u, float qh, float ql) {      // u - w q
+          FF v = ff_fma(-u3[2].hi, qh, u);
+          v.lo -= fmaf(u3[2].hi, ql, u3[2].lo * qh);
+          return v.hi + v.lo;
+        };
+        o[8 * kStGrp] = arm(u3[0], ln.x, ln.y) * zf;
+        o[9 * kStGrp] = arm(u3[1], ln.z, ln.w) * zf;
+      }
+      __syncthreads();
+      for (int i = tid; i < kGsVals * kStGrp; i += nthr) {
+        const int v = i / kStGrp, k = k0 + (i & (kStGrp - 1));
+        if (!TOT && k >= K) continue;
+        float *ps = total(v, k), *pc = total_comp(v, k);
+        float sum = s0 ? *ps : 0.f, comp = s0 ? *pc : 0.f;
+        for (int w = 0; w < n_act; ++w) kahan_add(sum, comp, st[(size_t)w * kGsVals * kStGrp + i]);
+        *ps = sum;
+        *pc = comp;
+      }
+    }
+  }
+  double l = (double)loss.hi + (double)loss.lo;
+  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+  if (lane == 0) s_loss[warp] = l;
+  __syncthreads();
+  if (tid == 0) {
+    double x = 0.0;
+    for (int w = 0; w < nw; ++w) x += s_loss[w];
+    a.loss_bl[bl] = x;
+  }
+  // G, and the (dl, dm, dS) contributions: -4 pi z, -2 Re tr(G^H J_i J_j^H)
+  const double four_pi = 12.566370614359172953850573533118;
+  for (int k = tid; k < K; k += nthr) {
+    // totals in plane order re 0 1 2 3 (values 0 .. 3), im 0 1 2 3 (values 4 .. 7)
+    double2* Go = a.G + ((size_t)k * a.n_bl + bl) * 4;
+    const size_t at = (size_t)k * a.n_ant;
+    float sum[kGsVals], comp[kGsVals];
+    #pragma unroll
+    for (int v = 0; v < kGsVals; ++v) { sum[v] = *total(v, k); comp[v] = *total_comp(v, k); }
+    if (!TOT) asm volatile("" ::: "memory");         // read before the same words take the results
+    FF tg = {0.f, 0.f};
+    #pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      Go[e] = make_double2((double)sum[e] - (double)comp[e], (double)sum[4 + e] - (double)comp[4 + e]);
+      const float2 pe = model_entry_ff(jones_row(a.jones, 2 * (at + ij.x) + (e >> 1)),
+                                       jones_row(a.jones, 2 * (at + ij.y) + (e & 1)), 1.f, 0.f);
+      tg = ff_fma(sum[e], pe.x, tg);
+      tg = ff_fma(sum[4 + e], pe.y, tg);
+      tg.lo -= fmaf(comp[e], pe.x, comp[4 + e] * pe.y);
+    }
+    double* o = a.gsc + ((size_t)k * a.n_bl + bl) * 3;
+    o[0] = -four_pi * ((double)sum[8] - (double)comp[8]);
+    o[1] = -four_pi * ((double)sum[9] - (double)comp[9]);
+    o[2] = -2.0 * ((double)tg.hi + (double)tg.lo);
   }
 }
 
+// Bound by FP64 arithmetic: 32 fused multiply-adds a baseline and a reduction that
+// halves the values with the lanes (9 additions a lane; a full tree a value took
+// 40, and the kernel 355 us at 128 antennas and 100 sources).
 // dL/dJ for antenna p of source k: -2 S [sum_{q>p} G(pq) J_q + sum_{q<p} G(qp)^H J_q]
 template <bool MIXED>
 __global__ void __launch_bounds__(128) k_grad_jones(const double2* __restrict__ G,
@@ -543,20 +630,19 @@ __global__ void __launch_bounds__(128) k_grad_jones(const double2* __restrict__ 
       C v = load_j<T>(jones, ((size_t)k * n_ant + q) * 4 + e);
       J[e] = make_double2(v.x, v.y);
     }
-    double2 r0 = cadd(cmul(g[0], J[0]), cmul(g[1], J[2]));
-    double2 r1 = cadd(cmul(g[0], J[1]), cmul(g[1], J[3]));
-    double2 r2 = cadd(cmul(g[2], J[0]), cmul(g[3], J[2]));
-    double2 r3 = cadd(cmul(g[2], J[1]), cmul(g[3], J[3]));
-    acc[0] += r0.x; acc[1] += r0.y; acc[2] += r1.x; acc[3] += r1.y;
-    acc[4] += r2.x; acc[5] += r2.y; acc[6] += r3.x; acc[7] += r3.y;
+    auto mac = [](double2 x, double2 y, double& re, double& im) {
+      re = fma(x.x, y.x, fma(-x.y, y.y, re));
+      im = fma(x.x, y.y, fma(x.y, y.x, im));
+    };
+    #pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      mac(g[2 * (e >> 1)], J[e & 1], acc[2 * e], acc[2 * e + 1]);
+      mac(g[2 * (e >> 1) + 1], J[2 + (e & 1)], acc[2 * e], acc[2 * e + 1]);
+    }
   }
-  #pragma unroll
-  for (int e = 0; e < 8; ++e)
-    #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
-  if ((threadIdx.x & 31) == 0)
-    #pragma unroll
-    for (int e = 0; e < 8; ++e) s_red[(threadIdx.x >> 5) * 8 + e] = acc[e];
+  const int lane = threadIdx.x & 31;
+  const double tot = warp_reduce_scatter8d(acc, lane);          // value (lane >> 2) & 7
+  if ((lane & 3) == 0) s_red[(threadIdx.x >> 5) * 8 + (lane >> 2)] = tot;
   __syncthreads();
   if (threadIdx.x == 0) {
     const double f = -2.0 * dir[k].w;
@@ -595,6 +681,8 @@ inline void grad_free(GradWorkspace& w) {
   if (w.loss_bl) cudaFree(w.loss_bl);
   if (w.dir) cudaFree(w.dir);
   if (w.wchan) cudaFree(w.wchan);
+  if (w.aph) cudaFree(w.aph);
+  if (w.lmn) cudaFree(w.lmn);
   w = GradWorkspace();
 }
 
@@ -604,22 +692,26 @@ inline int grad_fail(std::string& err, cudaError_t e, const char* what) {
 }
 
 // Allocates its workspace on first use (G and per-baseline terms for up to
-// max_src sources: (64 + 24) bytes per source and baseline) and keeps it.
-inline int grad_prepare(GradWorkspace& w, int n_src, const double* src, int64_t n_bl, int max_src,
-                        cudaStream_t s, std::string& err) {
+// max_src sources: (64 + 24) bytes per source and baseline, and for the FP32
+// sweep 16 bytes per source, antenna and time) and keeps it.
+inline int grad_prepare(GradWorkspace& w, bool mixed, int n_src, const double* src, int n_ant, int n_time,
+                        int64_t n_bl, int max_src, cudaStream_t s, std::string& err) {
   cudaError_t e;
   if (!w.loss_bl) {
     w.cap_src = max_src; w.n_bl = n_bl;
     if ((e = cudaMalloc(&w.G, (size_t)max_src * n_bl * 4 * sizeof(double2))) != cudaSuccess ||
         (e = cudaMalloc(&w.gsc, (size_t)max_src * n_bl * 3 * sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&w.loss_bl, (size_t)n_bl * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&w.dir, (size_t)max_src * sizeof(DirQ))) != cudaSuccess) {
+        (e = cudaMalloc(&w.dir, (size_t)max_src * sizeof(DirQ))) != cudaSuccess ||
+        (e = cudaMalloc(&w.lmn, (size_t)grad_kp(max_src) * sizeof(float4))) != cudaSuccess ||
+        (e = cudaMemsetAsync(w.lmn, 0, (size_t)grad_kp(max_src) * sizeof(float4), s)) != cudaSuccess ||
+        (mixed && (e = cudaMalloc(&w.aph, (size_t)n_time * n_ant * grad_kp(max_src) * sizeof(PhaseAB))) != cudaSuccess)) {
       int rc = grad_fail(err, e, "cudaMalloc(gradient workspace)");
       grad_free(w);
       return rc;
     }
   }
-  if (n_src > 0) k_grad_dirs<<<(n_src + 127) / 128, 128, 0, s>>>(src, n_src, w.dir);
+  if (n_src > 0) k_grad_dirs<<<(n_src + 127) / 128, 128, 0, s>>>(src, n_src, w.dir, w.lmn);
   return 0;
 }
 
@@ -643,11 +735,36 @@ inline int grad_sweep(GradWorkspace& w, bool mixed, const void* vis, int n_src, 
   a.G = w.G; a.gsc = w.gsc; a.loss_bl = w.loss_bl;
   a.n_src = n_src; a.n_ant = n_ant; a.n_chan = n_chan; a.n_time = n_time; a.n_bl = n_bl;
   a.nu0_c = nu0_c; a.dnu_c = dnu_c;
-  const size_t smem_fac = grad_fac_smem_bytes(n_src);
-  const bool fac = mixed && smem_fac <= kGradMaxSmem && !direct;
-  const size_t smem = fac ? smem_fac : grad_smem_bytes(mixed, n_src);
-  const int chunk = fac ? kGfChunk : kGradChunk;
-  const int chunks = n_src > 0 ? (n_src + chunk - 1) / chunk : 1;
+  if (mixed && !direct) {
+    // two CTAs an SM where they have more warps than one, with the totals in shared
+    // memory if that leaves them all of their warps
+    auto fit = [&](int most, size_t room, bool tot) {
+      return wchan ? grad_strip_warps<true>(n_src, n_chan, n_time, most, room, tot)
+                   : grad_strip_warps<false>(n_src, n_chan, n_time, most, room, tot);
+    };
+    int warps = fit(kGsMaxWarps, kGradMaxSmem - 2048, true);
+    const int two_tot = fit(kGsPairWarps, kGsPairSmem, true), two = fit(kGsPairWarps, kGsPairSmem, false);
+    const bool pair = 2 * two > warps, tot = !pair || two_tot == two;
+    if (pair) warps = two;
+    if (warps > 0) {
+      const size_t smem = wchan ? grad_strip_smem<true>(n_src, warps, tot) : grad_strip_smem<false>(n_src, warps, tot);
+      if (n_src > 0)
+        k_grad_ant_phases<<<1024, 256, 0, s>>>(w.dir, n_src, grad_kp(n_src), uvw, n_ant, n_time, nu0_c, dnu_c, w.aph);
+      auto launch = [&](auto kernel) -> cudaError_t {
+        cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradMaxSmem - 1024);
+        if (r == cudaSuccess) kernel<<<(unsigned)n_bl, 32 * warps, smem, s>>>(a, w.aph, w.lmn);
+        return r;
+      };
+      if (!pair) e = wchan ? launch(k_grad_strip<true, kGsMaxWarps, true>) : launch(k_grad_strip<false, kGsMaxWarps, true>);
+      else if (tot) e = wchan ? launch(k_grad_strip<true, kGsPairWarps, true>) : launch(k_grad_strip<false, kGsPairWarps, true>);
+      else e = wchan ? launch(k_grad_strip<true, kGsPairWarps, false>) : launch(k_grad_strip<false, kGsPairWarps, false>);
+      if (e != cudaSuccess) return grad_fail(err, e, "cudaFuncSetAttribute");
+      if ((e = cudaGetLastError()) != cudaSuccess) return grad_fail(err, e, "gradient sweep launch");
+      return 0;
+    }
+  }
+  const size_t smem = grad_smem_bytes(mixed, n_src);
+  const int chunks = n_src > 0 ? (n_src + kGradChunk - 1) / kGradChunk : 1;
   if (smem > kGradMaxSmem) {
     err = "too many sources for the gradient kernel's shared memory";
     return -1;
@@ -655,11 +772,10 @@ inline int grad_sweep(GradWorkspace& w, bool mixed, const void* vis, int n_src, 
   const dim3 grid((unsigned)n_bl, (unsigned)chunks);
   auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (r == cudaSuccess) kernel<<<grid, fac ? kGfThreads : kGradThreads, smem, s>>>(a);
+    if (r == cudaSuccess) kernel<<<grid, kGradThreads, smem, s>>>(a);
     return r;
   };
-  if (fac) e = wchan ? launch(k_grad_sweep_fac<true>) : launch(k_grad_sweep_fac<false>);
-  else if (mixed) e = wchan ? launch(k_grad_sweep<true, true>) : launch(k_grad_sweep<true, false>);
+  if (mixed) e = wchan ? launch(k_grad_sweep<true, true>) : launch(k_grad_sweep<true, false>);
   else e = wchan ? launch(k_grad_sweep<false, true>) : launch(k_grad_sweep<false, false>);
   if (e != cudaSuccess) return grad_fail(err, e, "cudaFuncSetAttribute");
   if ((e = cudaGetLastError()) != cudaSuccess) return grad_fail(err, e, "gradient sweep launch");

@@ -70,8 +70,11 @@ template <int QH> struct StripTables {
   float4 t1[kStGrp][QH + 1];
 };
 template <int QH> __host__ __device__ constexpr size_t strip_planes_bytes() { return (size_t)32 * QH * 2 * sizeof(float4); }
+// a warp's workspace: tables, planes or (6 KB at most) its sums
 template <int QH> __host__ __device__ constexpr size_t strip_warp_bytes() {
-  return sizeof(StripTables<QH>) > strip_planes_bytes<QH>() ? sizeof(StripTables<QH>) : strip_planes_bytes<QH>();
+  return sizeof(StripTables<QH>) > strip_planes_bytes<QH>()
+             ? (sizeof(StripTables<QH>) > 6144 ? sizeof(StripTables<QH>) : 6144)
+             : strip_planes_bytes<QH>();
 }
 
 // the tables of source `lane` from its phase; np pairs of tiles
@@ -216,16 +219,17 @@ __device__ __forceinline__ void strip_store(const Strip<QH>& R, float4* __restri
     }
   }
 }
-template <int QH>
+// tiles start `PITCH` float4 apart
+template <int QH, int PITCH = 16>
 __device__ __forceinline__ void strip_planes(const Strip<QH>& R, float4* pre, float4* pim, int n_chan, int lane) {
-  const int c0 = 16 * (lane >> 4) * QH + (lane & 15);
+  const int c0 = 16 * (lane >> 4) * QH + (lane & 15), at = PITCH * (lane >> 4) * QH + (lane & 15);
   #pragma unroll
   for (int u = 0; u < QH; ++u) {
     float re[4], im[4];
     strip_channel(R, u, re, im);
     const bool in = c0 + 16 * u < n_chan;          // channels past the strip hold no data
-    pre[c0 + 16 * u] = in ? make_float4(re[0], re[1], re[2], re[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
-    pim[c0 + 16 * u] = in ? make_float4(im[0], im[1], im[2], im[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    pre[at + PITCH * u] = in ? make_float4(re[0], re[1], re[2], re[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    pim[at + PITCH * u] = in ? make_float4(im[0], im[1], im[2], im[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 

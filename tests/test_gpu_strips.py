@@ -84,3 +84,37 @@ def test_strip_prediction_takes_gains_on_an_element_boundary():
     p = make_peeler(cad, "mixed")
     assert torch.equal(p.predict(cad.sources(), odd), p.predict(cad.sources(), J))
     p.close()
+
+
+GRAD_CASES = [
+    ("one-channel", Cadence(6, 1, 1, 2, pos_sigma_rad=2.909e-4, seed=241)),
+    ("255-channels-63", Cadence(5, 255, 1, 63, pos_sigma_rad=2.909e-4, seed=242)),       # one strip a baseline
+    ("256-channels-64", Cadence(5, 256, 2, 64, pos_sigma_rad=2.909e-4, seed=243)),
+    ("257-channels-65", Cadence(5, 257, 3, 65, pos_sigma_rad=2.909e-4, seed=244)),       # a strip of one channel
+    ("520-channels-13-times", Cadence(4, 520, 13, 33, pos_sigma_rad=2.909e-4, seed=245)),   # 39 strips: five rounds
+    ("12-strips", Cadence(5, 300, 6, 20, pos_sigma_rad=2.909e-4, seed=246)),               # one CTA an SM, 12 sources left
+    ("161-sources", Cadence(4, 300, 4, 161, pos_sigma_rad=2.909e-4, seed=247)),           # totals outside shared memory
+]
+
+
+@pytest.mark.parametrize("name,cad", GRAD_CASES, ids=[c[0] for c in GRAD_CASES])
+def test_strip_adjoint_matches_oracle(name, cad):
+    V = oracle.simulate(cad.with_(pos_sigma_rad=0.0)).astype(np.complex64).astype(np.complex128)
+    src = cad.perturbed_sources()
+    src[-1, 2] = 0.0                                        # a source without flux still has dL/dS
+    J = cad.jones().astype(np.complex64)
+    L_ref, gJ_ref, gl_ref, gm_ref, gS_ref = oracle.loss_grad(cad.uvw(), cad.freqs(), V, src, J.astype(np.complex128))
+    p = make_peeler(cad, "mixed")
+    args = (to_dev(V, "mixed"), torch.from_numpy(J).cuda(), torch.from_numpy(src).cuda())
+    loss, gJ, gs = p.grad(*args)
+    again = p.grad(*args)
+    torch.cuda.synchronize()
+    assert abs(loss.item() - L_ref) <= 1e-5 * L_ref
+    assert np.abs(gJ.cpu().numpy() - gJ_ref).max() <= 1e-4 * np.abs(gJ_ref).max()
+    g = gs.cpu().numpy()
+    for col, ref in ((0, gl_ref), (1, gm_ref), (2, gS_ref)):
+        assert np.abs(g[:, col] - ref).max() <= 1e-4 * np.abs(ref).max(), col
+    assert torch.equal(again[1], gJ) and torch.equal(again[2], gs)           # deterministic
+    odd = torch.empty(J.size + 1, dtype=torch.complex64, device="cuda")[1:].view(J.shape).copy_(args[1])
+    assert torch.equal(p.grad(args[0], odd, args[2])[1], gJ)                # gains on an element's boundary only
+    p.close()
