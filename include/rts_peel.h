@@ -105,8 +105,9 @@ typedef struct rts_peel_config {
                            cooperative launches and the rows of ceil(n_ant / n_SM)
                            antennas fit in shared memory, about n_ant <= 900 on GB300;
                            otherwise as RTS_SOLVE_LAUNCHES),
-                           RTS_SOLVE_LAUNCHES (1: one launch per ALS sweep, per
-                           correction and per model step).  The cluster and the
+                           RTS_SOLVE_LAUNCHES (1: one launch per correction, per model
+                           step and per solve or, above 256 antennas, per ALS sweep; a
+                           single source's solve always goes this way).  The cluster and the
                            cooperative launch solve the 2x2 systems of the sweeps before
                            the last in FP32 and the last in FP64 (from float-float or
                            FP64 sums), the per-step launches every sweep in FP64; their

@@ -135,6 +135,26 @@ __device__ __forceinline__ void cluster_wait(uint64_t* bar, uint32_t parity, vol
   }
 }
 
+__device__ __forceinline__ FF ff_shfl_xor(FF x, int o) {
+  FF r;
+  r.hi = __shfl_xor_sync(0xffffffffu, x.hi, o);
+  r.lo = __shfl_xor_sync(0xffffffffu, x.lo, o);
+  return r;
+}
+// the last three levels of the sums below
+__device__ __forceinline__ FF warp_reduce_scatter8ff(FF (&w)[8], int lane) {
+  #pragma unroll
+  for (int o = 8, n = 8; o >= 2; o >>= 1, n >>= 1) {
+    const bool upper = (lane & o) != 0;
+    #pragma unroll
+    for (int i = 0; i < n / 2; ++i) {
+      const FF send = upper ? w[i] : w[i + n / 2], keep = upper ? w[i + n / 2] : w[i];
+      w[i] = ff_add(keep, ff_shfl_xor(send, o));
+    }
+  }
+  return ff_add(w[0], ff_shfl_xor(w[0], 1));
+}
+
 // Reduce 16 floats over the 32 lanes of a warp with float-float sums (each level
 // exchanges half of the remaining values with the partner lane); afterwards
 // lane L holds the warp total of value index L >> 1.
@@ -148,22 +168,20 @@ __device__ __forceinline__ FF warp_reduce_scatter16ff(const float (&v)[16], int 
       w[i] = ff_two_sum(keep, __shfl_xor_sync(0xffffffffu, send, 16));
     }
   }
-  auto recv = [&](FF x, int o) {
-    FF r;
-    r.hi = __shfl_xor_sync(0xffffffffu, x.hi, o);
-    r.lo = __shfl_xor_sync(0xffffffffu, x.lo, o);
-    return r;
-  };
+  return warp_reduce_scatter8ff(w, lane);
+}
+// the same of 12 float-float values (and four zeros)
+__device__ __forceinline__ FF warp_reduce_scatter12ff(const FF (&v)[12], int lane) {
+  const FF zero = {0.f, 0.f};
+  FF w[8];
+  const bool upper = (lane & 16) != 0;
   #pragma unroll
-  for (int o = 8, n = 8; o >= 2; o >>= 1, n >>= 1) {
-    const bool upper = (lane & o) != 0;
-    #pragma unroll
-    for (int i = 0; i < n / 2; ++i) {
-      const FF send = upper ? w[i] : w[i + n / 2], keep = upper ? w[i + n / 2] : w[i];
-      w[i] = ff_add(keep, recv(send, o));
-    }
+  for (int i = 0; i < 8; ++i) {
+    const FF hi = i < 4 ? v[i + 8] : zero;
+    const FF send = upper ? v[i] : hi, keep = upper ? hi : v[i];
+    w[i] = ff_add(keep, ff_shfl_xor(send, 16));
   }
-  return ff_add(w[0], recv(w[0], 1));
+  return warp_reduce_scatter8ff(w, lane);
 }
 
 // A group's input from the block's tables: V_s = A_s - sum_{j<q0} M_j D_js of its
@@ -255,6 +273,29 @@ __device__ __forceinline__ void als_terms(float (&v)[16], const float4 v0, const
   v[10] = fmaf(j1.x, j1.z, v[10]); v[10] = fmaf(j1.y, j1.w, v[10]);
   v[11] = fmaf(j0.x, j0.w, v[11]); v[11] = fmaf(-j0.y, j0.z, v[11]);
   v[11] = fmaf(j1.x, j1.w, v[11]); v[11] = fmaf(-j1.y, j1.z, v[11]);
+}
+
+// one source's status and last relative change from its per-antenna norms
+// [n_ant][4] (dn, nn, non-finite), by one warp
+__device__ __forceinline__ void cluster_status(const double* norms, int n_ant, int lane, int bad, int* status,
+                                               double* rel) {
+  double dn = 0.0, nn = 0.0, nf = 0.0;
+  for (int p = lane; p < n_ant; p += 32) {
+    dn += __ldcg(norms + 4 * p);
+    nn += __ldcg(norms + 4 * p + 1);
+    nf += __ldcg(norms + 4 * p + 2);
+  }
+  #pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    dn += __shfl_xor_sync(0xffffffffu, dn, o);
+    nn += __shfl_xor_sync(0xffffffffu, nn, o);
+    nf += __shfl_xor_sync(0xffffffffu, nf, o);
+  }
+  if (lane == 0) {
+    const double r = sqrt(dn / nn);
+    *status = bad ? kSolveStatusTimeout : (nf != 0.0 || !isfinite(r)) ? -4 : (r > 1e-6 ? 1 : 0);
+    *rel = r;
+  }
 }
 
 // one launch: one cluster of gridDim.x CTAs of 32 apc threads
@@ -444,27 +485,9 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_solve(ClusterSolveArg
   if (*bad) __nanosleep(100000);
   cluster_sync();
   if (warp == 0)
-    for (int q = rank; q < a.n_grp; q += CS) {
-      double dn = 0.0, nn = 0.0, nf = 0.0;
-      for (int p = lane; p < n_ant; p += 32) {
-        const double* pt = a.part + ((size_t)(a.q0 + q) * n_ant + p) * 4;
-        dn += __ldcg(pt);
-        nn += __ldcg(pt + 1);
-        nf += __ldcg(pt + 2);
-      }
-      #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) {
-        dn += __shfl_xor_sync(0xffffffffu, dn, o);
-        nn += __shfl_xor_sync(0xffffffffu, nn, o);
-        nf += __shfl_xor_sync(0xffffffffu, nf, o);
-      }
-      if (lane == 0) {
-        const double r = sqrt(dn / nn);
-        a.status[a.s0 + a.q0 + q] = *bad ? kSolveStatusTimeout
-                                    : (nf != 0.0 || !isfinite(r)) ? -4 : (r > 1e-6 ? 1 : 0);
-        a.rel[a.s0 + a.q0 + q] = r;
-      }
-    }
+    for (int q = rank; q < a.n_grp; q += CS)
+      cluster_status(a.part + (size_t)(a.q0 + q) * n_ant * 4, n_ant, lane, *bad, a.status + a.s0 + a.q0 + q,
+                     a.rel + a.s0 + a.q0 + q);
   const int n_warp = nthr >> 5;
   const bool busy = n_warp > 1 && rank < a.n_grp;        // warp 0 is at the statuses
   if (!(busy && warp == 0))
@@ -484,6 +507,151 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_solve(ClusterSolveArg
     }
   cluster_sync();
   if (*bad && tid < a.n_grp) a.status[a.s0 + a.q0 + tid] = kSolveStatusTimeout;
+}
+
+// The solve of one source's averages with FP64 iterates (k_als_sweep's arithmetic)
+// by one cluster: 20 launches of 6.6 us and their gaps become one launch.  As
+// k_cluster_solve, but every sweep's sums over partners are float-float (a
+// partner's product and its lane's first are FP32, as a k_als_sweep thread's
+// are), and the 2x2 solve, the iterate and its averaging FP64; the sweeps' terms
+// read the FP32 rounding of the iterate.  An FP64 instruction occupies its
+// sub-partition for 64 cycles whatever its lanes, so all slots' solves run as
+// lanes of one or two warps.  Measured (128 antennas, 20 sweeps): 66 us where the
+// launches took 137; the call with its status read 185 and 110 us.  A sweep: terms
+// 1 830 cycles, reduction 870, FP64 solve 2 010, exchange 1 040.
+struct ClusterAlsArgs {
+  const float2* avg;       // [n_bl][4]
+  double S;
+  int n_ant, n_iter, apc;
+  double2* J;              // [n_ant][4] FP64 solution
+  float2* jones;           // [n_ant][4] its FP32 rounding
+  double* norms;           // [n_ant][4] dn, nn, non-finite of the last sweep
+  int* status;             // of this source
+  double* rel;
+};
+
+inline size_t cluster_als_smem(int n_ant, int apc) { return ((size_t)apc + 2) * 2 * n_ant * sizeof(float4); }
+
+__global__ void __launch_bounds__(kClThreads, 1) k_cluster_als(ClusterAlsArgs a) {
+  extern __shared__ __align__(16) unsigned char cl_smem[];
+  const int n_ant = a.n_ant;
+  float4* rows = reinterpret_cast<float4*>(cl_smem);               // [apc][2][n_ant]
+  float4* Jb = rows + (size_t)a.apc * 2 * n_ant;                    // [2][2][n_ant] iterates
+  __shared__ double s_tot64[kClMaxSlots][12];
+  __shared__ float4 s_Jn[kClMaxSlots][2];
+  __shared__ __align__(8) uint64_t s_bar[2];
+  __shared__ int s_bad;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = (int)cluster_rank(), CS = (int)cluster_size();
+  const int slot = warp, my_p = rank + slot * CS;
+  const bool live = my_p < n_ant;
+  if (tid == 0) {
+    s_bad = 0;
+    tc05::mbar_init(&s_bar[0], 1);
+    tc05::mbar_init(&s_bar[1], 1);
+  }
+  float4* row0 = rows + (size_t)slot * 2 * n_ant;
+  float4* row1 = row0 + n_ant;
+  if (live)
+    for (int qq = lane; qq < n_ant; qq += 32) {
+      float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0;
+      if (qq != my_p) {
+        const float4* P = reinterpret_cast<const float4*>(a.avg + bl_index(n_ant, min(my_p, qq), max(my_p, qq)) * 4);
+        r0 = P[0];
+        r1 = P[1];
+        if (qq < my_p) {                   // V_pq = V_qp^H
+          const float4 t0 = r0, t1 = r1;
+          r0 = make_float4(t0.x, -t0.y, t1.x, -t1.y);
+          r1 = make_float4(t0.z, -t0.w, t1.z, -t1.w);
+        }
+      }
+      row0[qq] = r0;
+      row1[qq] = r1;
+    }
+  __syncthreads();
+  cluster_sync();                          // every CTA's barriers exist before any store to them
+  volatile int* bad = &s_bad;
+  const uint32_t dst_rank = (uint32_t)(lane >> 1);
+  const bool sends = live && (int)dst_rank < CS;
+  const uint32_t my_row = tc05::smem_u32(Jb) + (uint32_t)((lane & 1) * n_ant + my_p) * 16u;
+  const uint32_t dst_row = sends ? cluster_map(my_row, dst_rank) : 0u;
+  const uint32_t dst_bar = sends ? cluster_map(tc05::smem_u32(&s_bar[0]), dst_rank) : 0u;
+  // the FP64 solver's lanes: entry e of slot s
+  const int s = tid >> 2, e = tid & 3, ps = rank + s * CS;
+  const bool solver = warp < (4 * a.apc + 31) / 32, lv = s < a.apc && ps < n_ant;
+  double2 Jd = make_double2(e == 0 || e == 3 ? 1.0 : 0.0, 0.0);    // this lane's iterate
+
+  for (int it = 1; it <= a.n_iter; ++it) {
+    const bool first = it == 1, last = it == a.n_iter;
+    const uint32_t b = (uint32_t)(it - 1) & 1u;
+    const float4* Jo = Jb + (size_t)(b ^ 1u) * 2 * n_ant;
+    if (tid == 0) mbar_expect(&s_bar[b], (uint32_t)n_ant * 32u);
+    FF sum[12];
+    #pragma unroll
+    for (int i = 0; i < 12; ++i) sum[i].hi = sum[i].lo = 0.f;
+    if (live)
+      for (int qq = lane; qq < n_ant; qq += 32) {
+        float4 j0 = first ? make_float4(1.f, 0.f, 0.f, 0.f) : Jo[qq];
+        float4 j1 = first ? make_float4(0.f, 0.f, 1.f, 0.f) : Jo[n_ant + qq];
+        if (qq == my_p) j0 = j1 = make_float4(0.f, 0.f, 0.f, 0.f);   // C excludes q = p
+        float v[16];
+        #pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = 0.f;
+        als_terms(v, row0[qq], row1[qq], j0, j1);
+        #pragma unroll
+        for (int i = 0; i < 12; ++i) {
+          const FF t = ff_two_sum(sum[i].hi, v[i]);
+          sum[i].hi = t.hi;
+          sum[i].lo += t.lo;
+        }
+      }
+    const FF wsum = warp_reduce_scatter12ff(sum, lane);
+    if ((lane & 1) == 0 && (lane >> 1) < 12) s_tot64[slot][lane >> 1] = (double)wsum.hi + (double)wsum.lo;
+    __syncthreads();
+    double2 Jp = Jd;
+    if (solver && lv) {
+      // entry (r, c) of A C^-1 / S: C^-1 = [c11 -c01; -conj(c01) c00] / det
+      const double* t = s_tot64[s];
+      const int r = e >> 1;
+      const double c00 = t[8], c11 = t[9], cx = t[10], cy = t[11];
+      const double ax = t[4 * r], ay = t[4 * r + 1], bx = t[4 * r + 2], by = t[4 * r + 3];
+      const double sc = 1.0 / (fma(c00, c11, -fma(cx, cx, cy * cy)) * a.S);
+      double2 num;
+      if (e & 1) num = make_double2(fma(bx, c00, -fma(ax, cx, -ay * cy)), fma(by, c00, -fma(ax, cy, ay * cx)));
+      else num = make_double2(fma(ax, c11, -fma(bx, cx, by * cy)), fma(ay, c11, -fma(by, cx, -bx * cy)));
+      if (it & 1) Jd = make_double2(num.x * sc, num.y * sc);
+      else Jd = make_double2(0.5 * fma(num.x, sc, Jp.x), 0.5 * fma(num.y, sc, Jp.y));
+      reinterpret_cast<float2*>(&s_Jn[s][r])[e & 1] = make_float2((float)Jd.x, (float)Jd.y);
+    }
+    __syncthreads();
+    if (sends && !*bad) cluster_send16(dst_row + b * (uint32_t)n_ant * 32u, s_Jn[slot][lane & 1], dst_bar + 8u * b);
+    if (last && solver) {
+      const double dx = Jd.x - Jp.x, dy = Jd.y - Jp.y;
+      double dn = dx * dx + dy * dy, nn = Jd.x * Jd.x + Jd.y * Jd.y;
+      int nf = lv && !(isfinite(Jd.x) && isfinite(Jd.y));
+      #pragma unroll
+      for (int o = 1; o <= 2; o <<= 1) {
+        dn += __shfl_xor_sync(0xffffffffu, dn, o);
+        nn += __shfl_xor_sync(0xffffffffu, nn, o);
+        nf |= __shfl_xor_sync(0xffffffffu, nf, o);
+      }
+      if (lv) {
+        a.J[(size_t)ps * 4 + e] = Jd;
+        a.jones[(size_t)ps * 4 + e] = make_float2((float)Jd.x, (float)Jd.y);
+        if (e == 0) {
+          a.norms[4 * ps] = dn;
+          a.norms[4 * ps + 1] = nn;
+          a.norms[4 * ps + 2] = (double)nf;
+        }
+      }
+    }
+    cluster_wait(&s_bar[b], ((uint32_t)(it - 1) >> 1) & 1u, bad);
+  }
+  if (*bad) __nanosleep(100000);
+  cluster_sync();
+  if (rank == 0 && warp == 0) cluster_status(a.norms, n_ant, lane, *bad, a.status, a.rel);
+  cluster_sync();
+  if (*bad && tid == 0) *a.status = kSolveStatusTimeout;
 }
 
 }  // namespace rts

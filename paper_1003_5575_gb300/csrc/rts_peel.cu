@@ -52,7 +52,7 @@ struct rts_peel_t {
   int tab64_q = 0, tab64_r = 0, tab64_at = 0;      // tab64_at: the last average's
   double2* d_J[2] = {nullptr, nullptr};
   float2* d_Jf[2] = {nullptr, nullptr};
-  double* d_norms = nullptr;       // [n_ant][2]
+  double* d_norms = nullptr;       // [n_ant][2] ([n_ant][4] in k_cluster_als)
   int* d_flag = nullptr;           // [1]
   int* d_status = nullptr;         // [max_sources]
   double* d_rel = nullptr;         // [max_sources]
@@ -97,6 +97,7 @@ struct rts_peel_t {
   // solve of small arrays by one cluster per group of sources (k_cluster_solve)
   int cl_size = 0, cl_apc = 0;     // CTAs (0: not used), antenna slots of each
   size_t cl_smem = 0;
+  int als_cs = 0, als_apc = 0;     // the same of k_cluster_als (launch_als, FP32 averages)
   float4* cl_V = nullptr;          // [kClGroup][n_ant][2][n_ant] a group's corrected averages
   float2* cl_D = nullptr;          // [kClPairs][n_ant][n_ant] its own D_jq
   unsigned* b_sync = nullptr;      // [2] barrier counter, abort flag
@@ -263,10 +264,67 @@ int launch_stream(rts_peel_t* h, bool sub, bool acc, bool in_peel, const StreamA
   return check_launch(h, "streaming kernel launch");
 }
 
+cudaLaunchConfig_t cluster_config(int cs, int apc, size_t smem, cudaLaunchAttribute* attr, cudaStream_t s) {
+  cudaLaunchConfig_t c;
+  std::memset(&c, 0, sizeof(c));
+  c.gridDim = dim3(cs);
+  c.blockDim = dim3(32 * apc);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = cs;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  c.attrs = attr;
+  c.numAttrs = 1;
+  return c;
+}
+
+// Cluster size and antenna slots a CTA for an n_ant-antenna solve: about kClSlots
+// antennas a CTA, at most kClMaxCta CTAs.  *cs = 0 where they do not fit (smem(apc)
+// bytes a CTA) or the device has no room for such a cluster.
+template <typename Kernel, typename Smem>
+int cluster_setup(rts_peel_t* h, Kernel kernel, Smem smem_of, int* cs_out, int* apc_out) {
+  *cs_out = 0;
+  int smem_max = 0;
+  RTS_CUDA(h, cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
+  cudaFuncAttributes fa;
+  RTS_CUDA(h, cudaFuncGetAttributes(&fa, kernel));
+  int cs = 1;
+  while (cs < kClMaxCta && (h->n_ant + cs - 1) / cs > kClSlots) cs *= 2;
+  const int apc = (h->n_ant + cs - 1) / cs;
+  const size_t smem = smem_of(h->n_ant, apc);
+  if (apc > kClMaxSlots || smem + fa.sharedSizeBytes + 1024 > (size_t)smem_max) return RTS_OK;
+  // handles of other sizes share the kernel: the attribute is the most it may take
+  RTS_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max - (int)fa.sharedSizeBytes));
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t c = cluster_config(cs, apc, smem, &attr, nullptr);
+  int n = 0;
+  if ((cs > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+      cudaOccupancyMaxActiveClusters(&n, kernel, &c) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    return RTS_OK;
+  }
+  *cs_out = cs;
+  *apc_out = apc;
+  return RTS_OK;
+}
+
 // n_iter ALS sweeps on avg; Jones to jones_out (cube precision) and the FP64
 // solution left in h->d_J[n_iter & 1]; status/rel to slot `slot`.
 int launch_als(rts_peel_t* h, const void* avg, double S, void* jones_out, int slot, cudaStream_t s) {
   Span span(h, RTS_K_SOLVE, s);
+  if (h->als_cs) {
+    ClusterAlsArgs a;
+    a.avg = static_cast<const float2*>(avg); a.S = S;
+    a.n_ant = h->n_ant; a.n_iter = h->n_iter; a.apc = h->als_apc;
+    a.J = h->d_J[h->n_iter & 1]; a.jones = static_cast<float2*>(jones_out);
+    a.norms = h->d_norms; a.status = h->d_status + slot; a.rel = h->d_rel + slot;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t c = cluster_config(h->als_cs, a.apc, cluster_als_smem(h->n_ant, a.apc), &attr, s);
+    RTS_CUDA(h, cudaLaunchKernelEx(&c, k_cluster_als, a));
+    span.end(1);
+    return check_launch(h, "cluster ALS launch");
+  }
   for (int it = 1; it <= h->n_iter; ++it) {
     AlsArgs a;
     a.avg = avg;
@@ -459,56 +517,18 @@ int setup_block_solve(rts_peel_t* h) {
   return RTS_OK;
 }
 
-cudaLaunchConfig_t cluster_config(const rts_peel_t* h, cudaLaunchAttribute* attr, cudaStream_t s) {
-  cudaLaunchConfig_t c;
-  std::memset(&c, 0, sizeof(c));
-  c.gridDim = dim3(h->cl_size);
-  c.blockDim = dim3(32 * h->cl_apc);
-  c.dynamicSmemBytes = h->cl_smem;
-  c.stream = s;
-  attr->id = cudaLaunchAttributeClusterDimension;
-  attr->val.clusterDim.x = h->cl_size;
-  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
-  c.attrs = attr;
-  c.numAttrs = 1;
-  return c;
-}
-
-// geometry of the cluster solve: about kClSlots antennas a CTA, at most kClMaxCta CTAs.
-// Leaves cl_size 0 (k_block_solve is used) when the rows do not fit or the device
-// has no room for such a cluster.
+// the cluster solve's geometry and a group's matrices (else k_block_solve is used)
 int setup_cluster_solve(rts_peel_t* h) {
   if (h->per_pass > kCorrMaxJ) return RTS_OK;
-  int smem_max = 0;
-  RTS_CUDA(h, cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
-  cudaFuncAttributes fa;
-  RTS_CUDA(h, cudaFuncGetAttributes(&fa, k_cluster_solve));
-  int cs = 1;
-  while (cs < kClMaxCta && (h->n_ant + cs - 1) / cs > kClSlots) cs *= 2;
-  const int apc = (h->n_ant + cs - 1) / cs;
-  if (apc > kClMaxSlots) return RTS_OK;
-  const size_t smem = cluster_solve_smem(h->n_ant, apc);
-  if (smem + fa.sharedSizeBytes + 1024 > (size_t)smem_max) return RTS_OK;
-  RTS_CUDA(h, cudaFuncSetAttribute(k_cluster_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max - (int)fa.sharedSizeBytes));
-  if (cs > 8 && cudaFuncSetAttribute(k_cluster_solve, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-    cudaGetLastError();
-    return RTS_OK;
-  }
-  h->cl_apc = apc;
-  h->cl_smem = smem;
-  h->cl_size = cs;
-  cudaLaunchAttribute attr;
-  const cudaLaunchConfig_t c = cluster_config(h, &attr, nullptr);
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, k_cluster_solve, &c) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    h->cl_size = 0;
-    return RTS_OK;
-  }
+  int cs = 0;
+  int rc = cluster_setup(h, k_cluster_solve, cluster_solve_smem, &cs, &h->cl_apc);
+  if (rc || !cs) return rc;
+  h->cl_smem = cluster_solve_smem(h->n_ant, h->cl_apc);
   RTS_CUDA(h, cudaMalloc((void**)&h->b_part, (size_t)h->per_pass * h->n_ant * 4 * sizeof(double)));
   const size_t nn = (size_t)h->n_ant * h->n_ant;
   RTS_CUDA(h, cudaMalloc((void**)&h->cl_V, kClGroup * 2 * nn * sizeof(float4)));
   RTS_CUDA(h, cudaMalloc((void**)&h->cl_D, kClPairs * nn * sizeof(float2)));
+  h->cl_size = cs;
   return RTS_OK;
 }
 
@@ -534,7 +554,7 @@ int launch_cluster_solve(rts_peel_t* h, int s0, int nblk, const float2* Dt, void
     }
     Span span(h, RTS_K_SOLVE, s);
     cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t c = cluster_config(h, &attr, s);
+    const cudaLaunchConfig_t c = cluster_config(h->cl_size, h->cl_apc, h->cl_smem, &attr, s);
     RTS_CUDA(h, cudaLaunchKernelEx(&c, k_cluster_solve, a));
     span.end(1);
   }
@@ -1176,7 +1196,7 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
       {(void**)&h->d_J[1], n_cplx_ant * sizeof(double2)},
       {(void**)&h->d_Jf[0], n_cplx_ant * sizeof(float2)},
       {(void**)&h->d_Jf[1], n_cplx_ant * sizeof(float2)},
-      {(void**)&h->d_norms, (size_t)h->n_ant * 2 * sizeof(double)},
+      {(void**)&h->d_norms, (size_t)h->n_ant * 4 * sizeof(double)},
       {(void**)&h->d_flag, sizeof(int)},
       {(void**)&h->d_status, (size_t)h->max_sources * sizeof(int)},
       {(void**)&h->d_rel, (size_t)h->max_sources * sizeof(double)},
@@ -1212,7 +1232,8 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
   // cadence's moments and iterates, are allocated here too (the paper's Section 5
   // advice), so a cadence allocates nothing
   int rc = RTS_OK;
-  if (h->per_pass > 1) rc = ensure_block_workspace(h);
+  if (h->precision == RTS_PREC_MIXED) rc = cluster_setup(h, k_cluster_als, cluster_als_smem, &h->als_cs, &h->als_apc);
+  if (rc == RTS_OK && h->per_pass > 1) rc = ensure_block_workspace(h);
   if (rc == RTS_OK && h->precision == RTS_PREC_MIXED) rc = taylor_setup(h);
   if (rc == RTS_OK && h->precision == RTS_PREC_MIXED) rc = predict_setup(h);
   if (rc != RTS_OK) {

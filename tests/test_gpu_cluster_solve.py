@@ -47,3 +47,27 @@ def test_cluster_solve_matches_oracle(name, cad):
     check_status(name, st, st_ref, p.rel(cad.n_src), rel_ref)
     assert torch.equal(again, resid) and torch.equal(jones2, jones)          # deterministic
     p.close()
+
+
+@pytest.mark.parametrize("n_iter", [1, 2, 5, 20])
+@pytest.mark.parametrize("n_ant", [2, 3, 17, 129, 256, 300])
+def test_single_solve_matches_oracle(n_ant, n_iter):
+    """rts_peel_solve: one cluster up to 256 antennas (k_cluster_als), sweep launches
+    past that, FP64 iterates both; tolerance 1e-5 as the other FP32 cases (the FP32
+    products of each sweep's terms carry 1e-7)."""
+    import oracle
+    cad = Cadence(n_ant, 8, 1, 1, seed=251)
+    rng = np.random.default_rng(n_ant)
+    n_bl = n_ant * (n_ant - 1) // 2
+    J = cad.jones()[0].reshape(n_ant, 2, 2)
+    i, j = np.triu_indices(n_ant, k=1)
+    S = 5.0
+    avg = S * J[i] @ J[j].conj().transpose(0, 2, 1) + 0.1 * (rng.standard_normal((n_bl, 2, 2))
+                                                             + 1j * rng.standard_normal((n_bl, 2, 2)))
+    avg = avg.reshape(n_bl, 4).astype(np.complex64)
+    J_ref, st_ref, rel_ref = oracle.als(avg.astype(np.complex128), S, n_ant, n_iter=n_iter)
+    p = make_peeler(cad, "mixed", n_iter=n_iter)
+    got, st = p.solve(torch.from_numpy(avg).cuda(), S)
+    assert np.linalg.norm(got.cpu().numpy() - J_ref) / np.linalg.norm(J_ref) <= TOL["mixed"]
+    check_status(f"solve-{n_ant}-{n_iter}", [st], [st_ref], p.rel(1), [rel_ref])
+    p.close()
