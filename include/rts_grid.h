@@ -20,8 +20,9 @@
  * visibility, as the paper's spheroidal function); visibilities outside
  * [0, n_pix) in either coordinate are not gridded.  Each visibility carries
  * n_pol complex values, each gridded into its own plane.  Sums are FP32 in a
- * fixed order (bins row by row, the sorted order inside a bin), so the grid
- * is bitwise reproducible.
+ * fixed order (bins row by row, the sorted order inside a bin, dealt 32 at a
+ * time to a few partial sums that are added in order), so the grid is bitwise
+ * reproducible.
  *
  * Ownership: the caller owns every pointer it passes ("d_" device, "h_"
  * host); the handle owns its workspace (sorted copies of up to max_vis

@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -46,11 +47,6 @@ int gcuda(rts_grid_t* g, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return gcuda((g), e_, #call);     \
   } while (0)
 
-int gather_threads(int bin) {
-  const int tpb = (bin + kGridTile - 1) / kGridTile;
-  return 32 * tpb * tpb;
-}
-
 }  // namespace
 
 extern "C" {
@@ -76,7 +72,7 @@ int rts_grid_init(const rts_grid_config* cfg, rts_grid_t** out) {
   rts_grid_t* g = new rts_grid_t();
   g->n_pix = cfg->n_pix; g->bin = cfg->bin; g->nbx = nbx; g->n_bins = nbx * nbx;
   g->n_tab = cfg->n_tab; g->n_pol = cfg->n_pol; g->max_vis = cfg->max_vis; g->r_max = cfg->r_max;
-  g->max_chunks = (cfg->max_vis + kGridChunk - 1) / kGridChunk;
+  g->max_chunks = std::min(kGridMaxChunks, (cfg->max_vis + kGridBlock - 1) / kGridBlock);
   cudaGetDevice(&g->device);
   auto bail = [&](cudaError_t e, const char* what) {
     gcuda(nullptr, e, what);
@@ -88,9 +84,9 @@ int rts_grid_init(const rts_grid_config* cfg, rts_grid_t** out) {
   if ((e = cudaMalloc(&g->d_gcf, sizeof(float) * g->n_tab)) != cudaSuccess) return bail(e, "cudaMalloc(gcf)");
   if ((e = cudaMemcpy(g->d_gcf, tab.data(), sizeof(float) * g->n_tab, cudaMemcpyHostToDevice)) != cudaSuccess)
     return bail(e, "cudaMemcpy(gcf)");
-  if ((e = cudaMalloc(&g->d_counts, sizeof(int) * (size_t)g->n_bins * g->max_chunks)) != cudaSuccess)
+  if ((e = cudaMalloc(&g->d_counts, sizeof(int) * (size_t)g->n_bins * (g->max_chunks + kGridSegs))) != cudaSuccess)
     return bail(e, "cudaMalloc(counts)");
-  if ((e = cudaMalloc(&g->d_bin_start, sizeof(int) * (size_t)(g->n_bins + 1))) != cudaSuccess)
+  if ((e = cudaMalloc(&g->d_bin_start, sizeof(int) * (size_t)(2 * g->n_bins + 2 + kGridMaxDense))) != cudaSuccess)
     return bail(e, "cudaMalloc(bin_start)");
   if ((e = cudaMalloc(&g->d_sxy, sizeof(float2) * (size_t)g->max_vis)) != cudaSuccess) return bail(e, "cudaMalloc(sxy)");
   if ((e = cudaMalloc(&g->d_svis, sizeof(float2) * (size_t)g->max_vis * g->n_pol)) != cudaSuccess)
@@ -103,6 +99,14 @@ int rts_grid_init(const rts_grid_config* cfg, rts_grid_t** out) {
       (e = cudaFuncSetAttribute(k_grid_sort_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sort_smem)) != cudaSuccess)
     return bail(e, "cudaFuncSetAttribute(sort)");
+  const int gsm = (int)grid_gather_smem(g->n_tab, g->bin, g->n_pol);
+  const void* gather[] = {(const void*)k_grid_gather<1>, (const void*)k_grid_gather<2>, (const void*)k_grid_gather<3>,
+                          (const void*)k_grid_gather<4>};
+  // all handles set the same value: the largest any configuration needs
+  if (gsm > kGridGatherMaxSmem) return bail(cudaErrorInvalidValue, "gather shared memory");
+  if ((e = cudaFuncSetAttribute(gather[g->n_pol - 1], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kGridGatherMaxSmem)) != cudaSuccess)
+    return bail(e, "cudaFuncSetAttribute(gather)");
   *out = g;
   return RTS_OK;
 }
@@ -117,34 +121,41 @@ int rts_grid_run(rts_grid_t* g, const void* d_xy, const void* d_vis, int32_t n_v
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int nbx = g->nbx;
   GRID_CUDA(g, cudaEventRecord(g->ev[0], s));
-  const int n_chunks = (n_vis + kGridChunk - 1) / kGridChunk;
+  const int64_t per = (int64_t)kGridBlock * kGridMaxChunks;
+  const int chunk = kGridBlock * (int)std::max<int64_t>(1, (n_vis + per - 1) / per);
+  const int n_chunks = (int)(((int64_t)n_vis + chunk - 1) / chunk);
   GridSortArgs a;
   a.xy = static_cast<const float2*>(d_xy); a.vis = static_cast<const float2*>(d_vis);
   a.n_vis = n_vis; a.n_pol = g->n_pol; a.n_pix = g->n_pix; a.bin = g->bin; a.nbx = nbx;
-  a.n_bins = g->n_bins; a.n_chunks = n_chunks;
+  a.n_bins = g->n_bins; a.n_chunks = n_chunks; a.chunk = chunk;
+  a.segs = g->d_counts + (size_t)g->n_bins * n_chunks;
   a.counts = g->d_counts; a.bin_start = g->d_bin_start; a.sxy = g->d_sxy; a.svis = g->d_svis;
+  a.dense = g->d_bin_start + g->n_bins + 1;
+  a.dense_min = std::max(kGridDenseMin, (int)((9 * (int64_t)n_vis + kGridMaxDense - 1) / kGridMaxDense));
   if (n_vis == 0) {
-    GRID_CUDA(g, cudaMemsetAsync(g->d_bin_start, 0, sizeof(int) * (size_t)(g->n_bins + 1), s));
+    GRID_CUDA(g, cudaMemsetAsync(g->d_bin_start, 0, sizeof(int) * (size_t)(2 * g->n_bins + 2 + kGridMaxDense), s));
   } else {
     const size_t sort_smem = sizeof(int) * (size_t)kGridWarps * g->n_bins;
     const unsigned sort_grid = (unsigned)((n_chunks + kGridWarps - 1) / kGridWarps);
     k_grid_sort_pass<false><<<sort_grid, kGridWarps * 32, sort_smem, s>>>(a);
-    const unsigned bins_grid = (unsigned)((g->n_bins + 255) / 256);
-    k_grid_bin_totals<<<bins_grid, 256, 0, s>>>(a);
+    const unsigned bins_grid = (unsigned)((g->n_bins + 31) / 32);
+    k_grid_bin_totals<<<bins_grid, kGridSegs * 32, 0, s>>>(a);
     k_grid_scan_bins<<<1, 1024, 0, s>>>(a);
-    k_grid_offsets<<<bins_grid, 256, 0, s>>>(a);
+    k_grid_offsets<<<bins_grid, kGridSegs * 32, 0, s>>>(a);
     k_grid_sort_pass<true><<<sort_grid, kGridWarps * 32, sort_smem, s>>>(a);
   }
   GRID_CUDA(g, cudaGetLastError());
   GRID_CUDA(g, cudaEventRecord(g->ev[1], s));
   GridGatherArgs b;
   b.sxy = g->d_sxy; b.svis = g->d_svis; b.bin_start = g->d_bin_start; b.gcf = g->d_gcf;
+  b.dense = a.dense;
   b.n_tab = g->n_tab; b.n_pol = g->n_pol; b.n_pix = g->n_pix; b.bin = g->bin; b.nbx = nbx; b.nby = nbx;
   b.r_max = (float)g->r_max; b.r2max = (float)(g->r_max * g->r_max);
   b.tab_scale = (float)((g->n_tab - 1) / g->r_max);
   b.grid = static_cast<float2*>(d_grid);
-  const size_t gsm = sizeof(float) * (size_t)(g->n_tab + 1);
-  const dim3 gg((unsigned)g->n_bins), gb((unsigned)gather_threads(g->bin));
+  const size_t gsm = grid_gather_smem(g->n_tab, g->bin, g->n_pol);
+  const unsigned tiles = grid_tiles(g->bin);
+  const dim3 gg((unsigned)g->n_bins + kGridMaxDense * tiles), gb(32u * tiles * grid_split(g->bin));
   switch (g->n_pol) {
     case 1: k_grid_gather<1><<<gg, gb, gsm, s>>>(b); break;
     case 2: k_grid_gather<2><<<gg, gb, gsm, s>>>(b); break;

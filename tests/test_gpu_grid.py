@@ -128,3 +128,34 @@ def test_grid_full_size_matches_oracle():
     G = run_gpu(1125, 12.0, gcf, 24, xy, vis)
     R = oracle.grid(1125, 12.0, gcf, xy.astype(np.float64), vis.astype(np.complex128))
     assert np.abs(G - R).max() <= 1e-5 * np.abs(R).max()
+
+
+EDGE_CASES = [
+    # (n_pix, r_max, bin, n_pol, n_vis, n_tab)
+    (64, 4.0, 4, 1, 500, 2),          # one tile a bin, four warps a tile
+    (50, 7.5, 13, 3, 31, 65),         # fewer visibilities than a step
+    (70, 6.0, 16, 2, 3000, 129),      # four tiles, four warps each
+    (100, 12.0, 33, 4, 2000, 1025),   # 25 tiles: one warp a tile
+    (90, 12.0, 24, 4, 140001, 257),   # two blocks of visibilities a counting warp, a ragged last chunk
+]
+
+
+@pytest.mark.parametrize("n_pix,r_max,bin,n_pol,n_vis,n_tab", EDGE_CASES)
+def test_gridder_geometry_edges_match_oracle(n_pix, r_max, bin, n_pol, n_vis, n_tab):
+    """Bin and table sizes at the edges of the sort's chunks and the gather's tiles,
+    dense points, some outside the grid and some exactly on pixels; 1e-5 x max |grid|."""
+    from paper_1003_5575_gb300 import Gridder
+    rng = np.random.default_rng(n_vis)
+    xy = (n_pix / 2 + n_pix / 3 * rng.standard_normal((n_vis, 2))).astype(np.float32)
+    xy[::7] = np.round(xy[::7])
+    vis = (rng.standard_normal((n_vis, n_pol)) + 1j * rng.standard_normal((n_vis, n_pol))).astype(np.complex64)
+    gcf = np.cos(0.5 * np.pi * np.linspace(0.0, 1.0, n_tab)) ** 2
+    ref = oracle.grid(n_pix, r_max, gcf, xy.astype(np.float64), vis.astype(np.complex128))
+    g = Gridder(n_pix, r_max, gcf, bin=bin, n_pol=n_pol, max_vis=n_vis)
+    d_xy, d_vis = torch.from_numpy(xy).cuda(), torch.from_numpy(vis).cuda()
+    got = g.run(d_xy, d_vis)
+    again = g.run(d_xy, d_vis)
+    torch.cuda.synchronize()
+    g.close()
+    assert torch.equal(got, again)
+    assert np.abs(got.cpu().numpy() - ref).max() <= 1e-5 * np.abs(ref).max()
