@@ -15,6 +15,7 @@
 #include "block_tc05_kernels.cuh"
 #include "block_tc_kernels.cuh"
 #include "cluster_solve_kernels.cuh"
+#include "cluster_taylor_kernels.cuh"
 #include "common.cuh"
 #include "grad_kernels.cuh"
 #include "offset_kernels.cuh"
@@ -98,6 +99,7 @@ struct rts_peel_t {
   int cl_size = 0, cl_apc = 0;     // CTAs (0: not used), antenna slots of each
   size_t cl_smem = 0;
   int als_cs = 0, als_apc = 0;     // the same of k_cluster_als (launch_als, FP32 averages)
+  int tay_cs = 0, tay_apc = 0;     // and of k_cluster_taylor
   float4* cl_V = nullptr;          // [kClGroup][n_ant][2][n_ant] a group's corrected averages
   float2* cl_D = nullptr;          // [kClPairs][n_ant][n_ant] its own D_jq
   unsigned* b_sync = nullptr;      // [2] barrier counter, abort flag
@@ -862,6 +864,20 @@ int launch_als_taylor(rts_peel_t* h, double S, float2* gain_out, float2* slope_o
   double mu[5];
   taylor_axis(h, &x0, &dx, mu);
   Span span(h, RTS_K_SOLVE, s);
+  if (h->tay_cs) {
+    ClusterTaylorArgs a;
+    a.mom = h->t_mom; a.S = S; a.mu0 = mu[0]; a.mu2 = mu[2]; a.mu4 = mu[4];
+    a.rotate = h->n_chan >= 3;
+    a.n_ant = h->n_ant; a.n_iter = h->n_iter; a.apc = h->tay_apc; a.n_bl = h->n_bl;
+    a.X = h->t_X[h->n_iter & 1]; a.Xf = h->t_Xf[h->n_iter & 1];
+    a.gain = gain_out; a.slope = slope_out;
+    a.norms = h->d_norms; a.status = h->d_status + slot; a.rel = h->d_rel + slot;
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t c = cluster_config(h->tay_cs, a.apc, cluster_taylor_smem(h->n_ant, a.apc), &attr, s);
+    RTS_CUDA(h, cudaLaunchKernelEx(&c, k_cluster_taylor, a));
+    span.end(1);
+    return check_launch(h, "cluster Taylor launch");
+  }
   for (int it = 1; it <= h->n_iter; ++it) {
     TaylorAlsArgs a;
     a.mom = h->t_mom;
@@ -1233,6 +1249,8 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
   // advice), so a cadence allocates nothing
   int rc = RTS_OK;
   if (h->precision == RTS_PREC_MIXED) rc = cluster_setup(h, k_cluster_als, cluster_als_smem, &h->als_cs, &h->als_apc);
+  if (rc == RTS_OK && h->precision == RTS_PREC_MIXED)
+    rc = cluster_setup(h, k_cluster_taylor, cluster_taylor_smem, &h->tay_cs, &h->tay_apc);
   if (rc == RTS_OK && h->per_pass > 1) rc = ensure_block_workspace(h);
   if (rc == RTS_OK && h->precision == RTS_PREC_MIXED) rc = taylor_setup(h);
   if (rc == RTS_OK && h->precision == RTS_PREC_MIXED) rc = predict_setup(h);
