@@ -26,6 +26,7 @@
 #include "strip_kernels.cuh"
 #include "taylor_kernels.cuh"
 #include "taylor_block_kernels.cuh"
+#include "taylor_strip_kernels.cuh"
 
 using namespace rts;
 
@@ -34,7 +35,8 @@ struct rts_peel_t {
   int per_pass = 1;                // sources per streaming pass (1 or RTS_BLOCK)
   bool block_tc = false;           // blocked passes as TF32 mma.sync (k_block_pass_tc)
   bool block_tc05 = false;           // blocked passes as tcgen05 MMAs (k_block_pass_tc05)
-  bool tay_tc05 = false;             // and the Taylor cadence's
+  bool tay_tc05 = false;             // the Taylor cadence in blocks: its passes as tcgen05 MMAs,
+  bool tay_strip = false;            // or by k_taylor_pass_strip
   int strip_qh = 0;                  // FP32 passes by k_block_pass_strip<strip_qh> (0: k_block_pass)
   int* d_perr = nullptr;           // [1] set by a tcgen05 pass whose mbarrier wait ran out
   int64_t n_bl = 0;
@@ -413,6 +415,14 @@ int set_strip_smem(rts_peel_t* h) {
   return RTS_OK;
 }
 
+template <int QH>
+int set_taylor_strip_smem(rts_peel_t* h) {
+  RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_strip<QH, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripMaxSmem));
+  RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_strip<QH, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripMaxSmem));
+  RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_strip<QH, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripMaxSmem));
+  return RTS_OK;
+}
+
 int setup_block_solve(rts_peel_t* h);
 
 // the tcgen05 pass holds all 512 TMEM columns: at least 116 KB of shared memory
@@ -454,7 +464,10 @@ int ensure_block_workspace(rts_peel_t* h) {
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
   }
-  if (h->tay_tc05) {
+  if (h->tay_strip) {
+    rc = h->n_chan <= 64 ? set_taylor_strip_smem<2>(h) : h->n_chan <= 128 ? set_taylor_strip_smem<4>(h) : set_taylor_strip_smem<8>(h);
+    if (rc) return rc;
+  } else if (h->tay_tc05) {
     const int tay = (int)tc05_tay_launch_smem(h);
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
     RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
@@ -983,8 +996,25 @@ void launch_taylor_geometry(rts_peel_t* h, int b, int n_src, cudaStream_t ps) {
   h->launches[RTS_K_BLOCK_FIX] += nblk > 1 ? 3 : 2;
 }
 
+template <int QH>
+void taylor_strip_t(const rts_peel_t* h, bool sub, bool acc, const BlockPassArgs& a, cudaStream_t s) {
+  const StripGrid g = strip_grid(h->n_time);
+  const size_t smem = taylor_strip_smem<QH>(g, h->n_time);
+  const unsigned grid = (unsigned)((h->n_bl + g.bpc - 1) / g.bpc), nthr = 32u * g.wpb * g.bpc;
+  if (sub && acc) k_taylor_pass_strip<QH, true, true><<<grid, nthr, smem, s>>>(a, 32, g);
+  else if (sub) k_taylor_pass_strip<QH, true, false><<<grid, nthr, smem, s>>>(a, 32, g);
+  else k_taylor_pass_strip<QH, false, true><<<grid, nthr, smem, s>>>(a, 32, g);
+}
+
 int launch_taylor_pass(rts_peel_t* h, bool sub, bool acc, const BlockPassArgs& a, cudaStream_t s) {
   Span span(h, RTS_K_BLOCK_PASS, s);
+  if (h->tay_strip) {
+    if (h->n_chan <= 64) taylor_strip_t<2>(h, sub, acc, a, s);
+    else if (h->n_chan <= 128) taylor_strip_t<4>(h, sub, acc, a, s);
+    else taylor_strip_t<8>(h, sub, acc, a, s);
+    span.end(1);
+    return check_launch(h, "Taylor block pass launch");
+  }
   const unsigned grid = (unsigned)h->n_bl;
   const size_t tsm = tc05_tay_launch_smem(h);
   if (sub && acc) k_block_pass_tc05<true, true, true><<<grid, kTc5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
@@ -1042,7 +1072,7 @@ int peel_taylor_blocked(rts_peel_t* h, const void* d_vis, void* d_resid, int32_t
       const int k = s0 + q;
       {
         Span span(h, RTS_K_BLOCK_FIX, s);
-        k_taylor_correct<<<bl_grid, 256, 0, s>>>(h->b_avg, q, h->b_model, Dt, h->n_bl, h->t_mom);
+        k_taylor_correct<<<dim3((unsigned)((h->n_bl + 127) / 128), 3), 128, 0, s>>>(h->b_avg, q, h->b_model, Dt, h->n_bl, h->t_mom);
         span.end(1);
       }
       rc = launch_als_taylor(h, src[3 * k + 2], static_cast<float2*>(d_gain) + k * jstride,
@@ -1171,6 +1201,7 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
   {
     int bk = cfg->block_kernel;
     h->tay_tc05 = per_pass > 1 && (bk == RTS_BLOCK_TCGEN05 || (bk == RTS_BLOCK_AUTO && cfg->n_chan <= kTc5MaxChan));
+    h->tay_strip = per_pass > 1 && bk == RTS_BLOCK_AUTO && cfg->n_chan <= kStAutoChan;
     if (bk == RTS_BLOCK_AUTO && cfg->n_chan <= kStAutoChan) bk = RTS_BLOCK_FMA;
     if (bk == RTS_BLOCK_AUTO)
       bk = cfg->n_chan <= kTc5MaxChan ? RTS_BLOCK_TCGEN05 : (cfg->n_chan <= kTcMaxChan ? RTS_BLOCK_TENSOR : RTS_BLOCK_FMA);
