@@ -27,6 +27,7 @@
 #include "taylor_kernels.cuh"
 #include "taylor_block_kernels.cuh"
 #include "taylor_strip_kernels.cuh"
+#include "taylor_tc05_kernels.cuh"
 
 using namespace rts;
 
@@ -423,13 +424,23 @@ int set_taylor_strip_smem(rts_peel_t* h) {
   return RTS_OK;
 }
 
+// the tcgen05 pass holds all 512 TMEM columns: at least 116 KB of shared memory each
+template <int NQ>
+int set_tc05_smem(rts_peel_t* h) {
+  constexpr int smem = std::max(Tc05Smem(NQ).total, 116 * 1024);
+  RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<NQ, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<NQ, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<NQ, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  return RTS_OK;
+}
+
 int setup_block_solve(rts_peel_t* h);
 
 // the tcgen05 pass holds all 512 TMEM columns: at least 116 KB of shared memory
 // keeps it at one CTA per SM (a second CTA would wait in its TMEM allocation)
 size_t tc05_launch_smem(const rts_peel_t* h) { return std::max<size_t>(tc05_pass_smem(h->n_chan), 116 * 1024); }
 size_t tc05_tay_launch_smem(const rts_peel_t* h) {
-  return std::max<size_t>(tc05_pass_smem(h->n_chan, true), 116 * 1024);
+  return std::max<size_t>(tc05_tay_pass_smem(h->n_chan, true), 116 * 1024);
 }
 
 int ensure_block_workspace(rts_peel_t* h) {
@@ -459,19 +470,17 @@ int ensure_block_workspace(rts_peel_t* h) {
   RTS_CUDA(h, cudaMalloc((void**)&h->d_perr, sizeof(int)));
   RTS_CUDA(h, cudaMemset(h->d_perr, 0, sizeof(int)));
   if (h->block_tc05) {
-    const int tsm = (int)tc05_launch_smem(h);
-    RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
-    RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
-    RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tsm));
+    rc = tc05_nq(h->n_chan) == 16 ? set_tc05_smem<16>(h) : tc05_nq(h->n_chan) == 32 ? set_tc05_smem<32>(h) : set_tc05_smem<48>(h);
+    if (rc) return rc;
   }
   if (h->tay_strip) {
     rc = h->n_chan <= 64 ? set_taylor_strip_smem<2>(h) : h->n_chan <= 128 ? set_taylor_strip_smem<4>(h) : set_taylor_strip_smem<8>(h);
     if (rc) return rc;
   } else if (h->tay_tc05) {
-    const int tay = (int)tc05_tay_launch_smem(h);
-    RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
-    RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
-    RTS_CUDA(h, cudaFuncSetAttribute(k_block_pass_tc05<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
+    const int tay = (int)tc05_tay_pass_smem(kTc5MaxChan, true);
+    RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_tc05<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
+    RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_tc05<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
+    RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_tc05<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
   }
   if (h->block_tc05) return RTS_OK;
   if (h->block_tc) {
@@ -598,6 +607,13 @@ int launch_block_solve(rts_peel_t* h, int s0, int nblk, const float2* Dt, void* 
   return check_launch(h, "block solve launch");
 }
 
+template <int NQ>
+void tc05_pass_t(bool sub, bool acc, const BlockPassArgs& a, int bk, int nb, unsigned grid, size_t smem, int* err, cudaStream_t s) {
+  if (sub && acc) k_block_pass_tc05<NQ, true, true><<<grid, kTc5Threads, smem, s>>>(a, bk, nb, err);
+  else if (sub) k_block_pass_tc05<NQ, true, false><<<grid, kTc5Threads, smem, s>>>(a, bk, nb, err);
+  else k_block_pass_tc05<NQ, false, true><<<grid, kTc5Threads, smem, s>>>(a, bk, nb, err);
+}
+
 template <int QH>
 void strip_pass_t(const rts_peel_t* h, bool sub, bool acc, const BlockPassArgs& a, cudaStream_t s) {
   const StripGrid g = strip_grid(h->n_time);
@@ -623,9 +639,11 @@ int launch_block_pass(rts_peel_t* h, bool sub, bool acc, const BlockPassArgs& a,
     // up to kTc5BaselinesPerCta baselines a CTA, keeping at least 8 waves of CTAs
     const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(kTc5BaselinesPerCta, h->n_bl / (8 * h->n_sm)));
     const unsigned g5 = (unsigned)((h->n_bl + nb - 1) / nb);
-    if (sub && acc) k_block_pass_tc05<true, true><<<g5, kTc5Threads, tsm, s>>>(a, h->per_pass, nb, h->d_perr);
-    else if (sub) k_block_pass_tc05<true, false><<<g5, kTc5Threads, tsm, s>>>(a, h->per_pass, nb, h->d_perr);
-    else k_block_pass_tc05<false, true><<<g5, kTc5Threads, tsm, s>>>(a, h->per_pass, nb, h->d_perr);
+    switch (tc05_nq(h->n_chan)) {
+      case 16: tc05_pass_t<16>(sub, acc, a, h->per_pass, nb, g5, tsm, h->d_perr, s); break;
+      case 32: tc05_pass_t<32>(sub, acc, a, h->per_pass, nb, g5, tsm, h->d_perr, s); break;
+      default: tc05_pass_t<48>(sub, acc, a, h->per_pass, nb, g5, tsm, h->d_perr, s); break;
+    }
     span.end(1);
     return check_launch(h, "block pass launch");
   }
@@ -1017,9 +1035,9 @@ int launch_taylor_pass(rts_peel_t* h, bool sub, bool acc, const BlockPassArgs& a
   }
   const unsigned grid = (unsigned)h->n_bl;
   const size_t tsm = tc05_tay_launch_smem(h);
-  if (sub && acc) k_block_pass_tc05<true, true, true><<<grid, kTc5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
-  else if (sub) k_block_pass_tc05<true, false, true><<<grid, kTc5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
-  else k_block_pass_tc05<false, true, true><<<grid, kTc5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
+  if (sub && acc) k_taylor_pass_tc05<true, true, true><<<grid, kTt5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
+  else if (sub) k_taylor_pass_tc05<true, false, true><<<grid, kTt5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
+  else k_taylor_pass_tc05<false, true, true><<<grid, kTt5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
   span.end(1);
   return check_launch(h, "Taylor block pass launch");
 }

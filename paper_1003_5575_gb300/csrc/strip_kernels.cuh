@@ -26,11 +26,14 @@ namespace rts {
 constexpr int kStWarps = 8;                // warps of a CTA
 constexpr int kStGrp = 32;                 // sources whose tables a warp holds at once
 constexpr int kStMaxQh = 8;                // tiles per half warp, at most: 256 channels
-// Strips up to here take this pass by default: at 128 antennas, 8 times and 128
-// sources the passes of a cadence take 1.02 / 1.29 / 1.99 / 3.19 / 3.49 ms for 16 / 64 /
-// 128 / 203 / 256 channels, the tcgen05 form's 3.75 ms for each of them; at 384
-// channels, where a strip no longer fits a warp's registers, the form of
-// block_kernels.cuh takes 7.7 ms and tcgen05 4.3.
+// Strips up to here take this pass, and the Taylor cadence's, by default.  At 128
+// antennas, 8 times and 128 sources the passes take 1.02 / 1.29 / 1.99 / 3.19 / 3.49 ms
+// for 16 / 64 / 128 / 203 / 256 channels, the tcgen05 form's 2.8 to 3.2 ms whatever the
+// length; with 4 times or 65 antennas this form is ahead up to 256 as well (0.25 and
+// 0.30 ms at 65 antennas x 4 times x 256 channels).  Past 256 channels a strip no longer
+// fits a warp's registers: the form of block_kernels.cuh takes 7.7 ms at 384,
+// tcgen05 3.2.  Taylor, 42 sources: 0.84 / 1.02 / 1.60 / 2.51 / 2.79 ms for 32 / 64 / 128 /
+// 203 / 256 channels, tcgen05 5.0 ms.
 constexpr int kStAutoChan = 256;
 constexpr int kStMRow = 4;                 // float4 of a source's packed model matrix
 

@@ -31,6 +31,9 @@
 
 namespace rts {
 
+constexpr int kTayBlk = 21;                  // Taylor sources per block: 3 slots each
+constexpr int kTayOut = 6 * kTayBlk;         // v_r-weighted T2 sums per block (6 per source)
+
 constexpr int kTayPairs = kTayBlk * (kTayBlk - 1) / 2;   // pairs j < k of one Taylor block
 constexpr int kTayMu = 22;                              // mu_0 .. mu_21
 constexpr int kTaySeriesM = 17;                         // highest power of 2z in the series
