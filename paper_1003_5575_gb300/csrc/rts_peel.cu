@@ -440,7 +440,7 @@ int setup_block_solve(rts_peel_t* h);
 // keeps it at one CTA per SM (a second CTA would wait in its TMEM allocation)
 size_t tc05_launch_smem(const rts_peel_t* h) { return std::max<size_t>(tc05_pass_smem(h->n_chan), 116 * 1024); }
 size_t tc05_tay_launch_smem(const rts_peel_t* h) {
-  return std::max<size_t>(tc05_tay_pass_smem(h->n_chan, true), 116 * 1024);
+  return std::max<size_t>(tc05_tay_pass_smem(h->n_chan), 116 * 1024);
 }
 
 int ensure_block_workspace(rts_peel_t* h) {
@@ -477,10 +477,10 @@ int ensure_block_workspace(rts_peel_t* h) {
     rc = h->n_chan <= 64 ? set_taylor_strip_smem<2>(h) : h->n_chan <= 128 ? set_taylor_strip_smem<4>(h) : set_taylor_strip_smem<8>(h);
     if (rc) return rc;
   } else if (h->tay_tc05) {
-    const int tay = (int)tc05_tay_pass_smem(kTc5MaxChan, true);
-    RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_tc05<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
-    RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_tc05<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
-    RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_tc05<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
+    const int tay = (int)tc05_tay_pass_smem(kTc5MaxChan);
+    RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_tc05<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
+    RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_tc05<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
+    RTS_CUDA(h, cudaFuncSetAttribute(k_taylor_pass_tc05<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tay));
   }
   if (h->block_tc05) return RTS_OK;
   if (h->block_tc) {
@@ -1035,9 +1035,9 @@ int launch_taylor_pass(rts_peel_t* h, bool sub, bool acc, const BlockPassArgs& a
   }
   const unsigned grid = (unsigned)h->n_bl;
   const size_t tsm = tc05_tay_launch_smem(h);
-  if (sub && acc) k_taylor_pass_tc05<true, true, true><<<grid, kTt5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
-  else if (sub) k_taylor_pass_tc05<true, false, true><<<grid, kTt5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
-  else k_taylor_pass_tc05<false, true, true><<<grid, kTt5Threads, tsm, s>>>(a, 32, 1, h->d_perr);
+  if (sub && acc) k_taylor_pass_tc05<true, true><<<grid, kTt5Threads, tsm, s>>>(a, 32, h->d_perr);
+  else if (sub) k_taylor_pass_tc05<true, false><<<grid, kTt5Threads, tsm, s>>>(a, 32, h->d_perr);
+  else k_taylor_pass_tc05<false, true><<<grid, kTt5Threads, tsm, s>>>(a, 32, h->d_perr);
   span.end(1);
   return check_launch(h, "Taylor block pass launch");
 }

@@ -49,7 +49,7 @@
 // reports, after the copies in flight have been waited for and TMEM is freed).
 // Limits: at most 64 sources per role, n_chan <= kTc5MaxChan.
 //
-// Gains Taylor-expanded in frequency (TAY): a source's model on a baseline is
+// Gains Taylor-expanded in frequency: a source's model on a baseline is
 // (P0 + x_c P1 + x_c^2 P2) e^{-2 pi i phi} and its averages are the three
 // moments mean x_c^n R e^{+2 pi i phi}.  With x_c = u_q + v_r (u_q = x_0 + 16 q dx,
 // v_r = r dx) the same two GEMMs carry them when each source takes three of
@@ -85,7 +85,7 @@ constexpr uint32_t kTt5Cols = 512;
 
 struct TayTc05Smem {
   int strip, bs_hi, bs_lo, ba_hi, ba_lo, t2s, t2a, mtab, ph, bar, cf, total;
-  __host__ __device__ explicit TayTc05Smem(int NQ, bool tay = false) {
+  __host__ __device__ explicit TayTc05Smem(int NQ) {
     int o = 0;
     strip = o; o += 2 * 16 * NQ * 32;            // two strips [16 NQ channels][4 pol][re, im]
     bs_hi = o; o += NQ * 128 * 4;                // B_s [NQ rows][128 K], K-major
@@ -99,15 +99,15 @@ struct TayTc05Smem {
     bar = o;   o += 80;                          // mbarriers (sub done, avg done, strip 0, strip 1, sub
                                                  // operands ready, avg operands ready, phases 0, phases 1),
                                                  // TMEM address
-    cf = o;    o += tay ? kTc5Src * 16 * 4 * 8 : 0;  // Taylor A_s coefficients [64 slots][16 r][4 e] float2
+    cf = o;    o += kTc5Src * 16 * 4 * 8;  // A_s coefficients [64 slots][16 r][4 e] float2
     total = o;
   }
 };
 
-inline size_t tc05_tay_pass_smem(int n_chan, bool tay = false) { return (size_t)TayTc05Smem(tc05_nq(n_chan), tay).total; }
+inline size_t tc05_tay_pass_smem(int n_chan) { return (size_t)TayTc05Smem(tc05_nq(n_chan)).total; }
 
-template <bool SUB, bool ACC, bool TAY = false>
-__global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassArgs a, int bk, int nb, int* err) {
+template <bool SUB, bool ACC>
+__global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassArgs a, int bk, int* err) {
   using namespace tc05;
   const int nq = (a.n_chan + 15) >> 4;
   const int NQ = (nq + 15) & ~15;           // 16, 32 or 48
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
   const int nmain_a = NQ >> 4;              // the average's hi*hi accumulators: 1, 2 or 3
   const int n16 = 16 * NQ;
   const uint32_t strip_bytes = (uint32_t)a.n_chan * 32u;
-  const TayTc05Smem L(NQ, TAY);
+  const TayTc05Smem L(NQ);
   extern __shared__ __align__(1024) unsigned char tc05_smem[];
   float* strip0 = reinterpret_cast<float*>(tc05_smem + L.strip);
   unsigned char* bs_hi = tc05_smem + L.bs_hi;
@@ -130,22 +130,19 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
   uint32_t* tslot = reinterpret_cast<uint32_t*>(tc05_smem + L.bar + 64);
   float2* cf = reinterpret_cast<float2*>(tc05_smem + L.cf);             // Taylor only
   // [4 cg][64 slots][8] (Taylor: [4 cg][128 sums][8], B_a hi and lo): B_a is free in P4
-  constexpr int kPartRows = TAY ? 2 * kTc5Src : kTc5Src;
+  constexpr int kPartRows = 2 * kTc5Src;
   float* part = reinterpret_cast<float*>(ba_hi);
   // slot -> source, and the slot's power m of u_q (Taylor: slot 3 k + m)
-  auto src_of = [](int s) { return TAY ? s / 3 : s; };
-  auto pow_of = [](int s) { return TAY ? s % 3 : 0; };
+  auto src_of = [](int s) { return s / 3; };
+  auto pow_of = [](int s) { return s % 3; };
   // u_q^m, u_q = x_0 + 16 q dx the offset of tile q's channel 0 from the band centre
   auto upow = [&](int q, int m) {
     const float u = fmaf((float)(16 * q), a.tdx, a.tx0);
     return m == 0 ? 1.f : (m == 1 ? u : u * u);
   };
 
-  // baselines bl0 .. bl0 + nbl - 1, their time steps one after another: step g
-  // is time g % n_time of baseline bl0 + g / n_time
-  const int64_t bl0 = (int64_t)blockIdx.x * nb;
-  const int nbl = TAY ? 1 : (int)min((int64_t)nb, a.n_bl - bl0), n_steps = TAY ? a.n_time : nbl * a.n_time;
-  auto bl_of = [&](int g) { return bl0 + g / a.n_time; };
+  const int64_t bl0 = blockIdx.x;            // the CTA's baseline; step g is time g
+  const int n_steps = a.n_time;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, qtr = warp & 3, cg = warp >> 2;
   const uint32_t lane_base = (uint32_t)(32 * qtr) << 16;
 
@@ -161,13 +158,13 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
     strip0[a.n_chan * 8 + i] = 0.f;
     strip0[(n16 + a.n_chan) * 8 + i] = 0.f;
   }
-  const int n_sub_slots = TAY ? 3 * a.n_sub : a.n_sub;
+  const int n_sub_slots = 3 * a.n_sub;
   if (SUB)
     for (int i = tid; compute && i < kTc5Src * 4; i += kTt5Compute) {
       const int s = i >> 2, e = i & 3;
       mtab[i] = s < n_sub_slots ? a.M_sub[((size_t)s * a.n_bl + bl0) * 4 + e] : make_float2(0.f, 0.f);
     }
-  if (SUB && TAY) {
+  if (SUB) {
     // the Taylor subtraction's A_s coefficients, slot (k, m), channel offset r:
     // sum_{n >= m} C(n, m) v_r^{n-m} P_n, v_r = r dx (from the model table mtab)
     __syncthreads();
@@ -209,9 +206,9 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
 
   // strip of step g -> buffer g & 1 (thread 0)
   auto issue_load = [&](int g) {
-    const int b = g & 1, t = g % a.n_time;
+    const int b = g & 1;
     mbar_expect_tx(&mbar[2 + b], strip_bytes);
-    bulk_load(strip0 + (size_t)b * n16 * 8, a.src + ((size_t)t * a.n_bl + bl_of(g)) * a.n_chan * 2, strip_bytes,
+    bulk_load(strip0 + (size_t)b * n16 * 8, a.src + ((size_t)g * a.n_bl + bl0) * a.n_chan * 2, strip_bytes,
               &mbar[2 + b]);
   };
   // the phases of both roles at step g -> ring slot g & 1 (thread 0): one bulk
@@ -220,7 +217,7 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
     const int b = g & 1;
     const uint32_t bytes = (uint32_t)bk * sizeof(PhaseAB);
     mbar_expect_tx(&mbar[6 + b], (SUB ? bytes : 0u) + (ACC ? bytes : 0u));
-    const size_t at = ((size_t)bl_of(g) * a.n_time + g % a.n_time) * bk;
+    const size_t at = ((size_t)bl0 * a.n_time + g) * bk;
     if (SUB) bulk_load(ph + 2 * kTc5Src * b, a.ph_sub + at, bytes, &mbar[6 + b]);
     if (ACC) bulk_load(ph + 2 * kTc5Src * b + kTc5Src, a.ph_acc + at, bytes, &mbar[6 + b]);
   };
@@ -241,10 +238,8 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
     unsigned long long x = p.a + (unsigned long long)(16 * ql) * p.b;
     for (int q = ql; q < NQ; q += 8, x += step) {
       float2 z = phasor_hw(x);
-      if (TAY) {
-        const float w = upow(q, m);
-        z = make_float2(z.x * w, z.y * w);
-      }
+      const float w = upow(q, m);
+      z = make_float2(z.x * w, z.y * w);
       const float hr = __uint_as_float(tc05_tf32(z.x)), hi = __uint_as_float(tc05_tf32(-z.y));
       const int o = kmaj_byte(q, 2 * k, 128);
       *reinterpret_cast<float2*>(bs_hi + o) = make_float2(hr, hi);
@@ -263,7 +258,7 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
       #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int k = 16 * cg + 8 * h + j;
-        const float2 m = TAY ? cf[(k * 16 + r) * 4 + e] : mtab[4 * k + e], z = t2s[k * kTt5T2Row + r];
+        const float2 m = cf[(k * 16 + r) * 4 + e], z = t2s[k * kTt5T2Row + r];
         const float ar = fmaf(m.x, z.x, m.y * z.y), ai = fmaf(m.y, z.x, -m.x * z.y);   // m conj(z)
         const float v0 = o ? ai : ar, v1 = o ? ar : -ai;
         const uint32_t h0 = tc05_tf32(v0), h1 = tc05_tf32(v1);
@@ -297,10 +292,8 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
       float2 mine = make_float2(0.f, 0.f);
       if (2 * jj < QW) {
         mine = phasor_hw(x);
-        if (TAY) {
-          const float w = upow(q0 + 2 * jj + o, m);
-          mine = make_float2(mine.x * w, mine.y * w);
-        }
+        const float w = upow(q0 + 2 * jj + o, m);
+        mine = make_float2(mine.x * w, mine.y * w);
         x += step;
       }
       const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, mine.x, 1), __shfl_xor_sync(0xffffffffu, mine.y, 1));
@@ -383,37 +376,12 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
       ba_put4(n, q0 + j, o, x);
     }
   };
-  // the T2 contraction of one step's H (rows m' = 2 k + o of lane, columns
-  // n = 4 r + e of r = 4 cg .. 4 cg + 3): o = 0 holds Re H (A += T2 Re H), o = 1
-  // Im H (A += i T2 Im H); the lane pair's sums meet by a shuffle and the four
-  // column groups' in part[cg][k]
-  auto avg_contract_plain = [&](const float (&H)[16]) {
-    const int k = 16 * qtr + (lane >> 1), o = lane & 1;
-    float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f};
-    #pragma unroll
-    for (int rr = 0; rr < 4; ++rr) {
-      const float2 z = t2a[k * kTt5T2Row + 4 * cg + rr];
-      const float wr = o ? -z.y : z.x, wi = o ? z.x : z.y;
-      #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        pr[e] = fmaf(wr, H[4 * rr + e], pr[e]);
-        pi[e] = fmaf(wi, H[4 * rr + e], pi[e]);
-      }
-    }
-    #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      pr[e] += __shfl_xor_sync(0xffffffffu, pr[e], 1);
-      pi[e] += __shfl_xor_sync(0xffffffffu, pi[e], 1);
-    }
-    if (o == 0) {
-      float4* dst = reinterpret_cast<float4*>(part + (cg * kPartRows + k) * 8);
-      dst[0] = make_float4(pr[0], pi[0], pr[1], pi[1]);
-      dst[1] = make_float4(pr[2], pi[2], pr[3], pi[3]);
-    }
-  };
-  // Taylor: slot s = 3 k + m gives Q_{k,m,d}(e) = sum_r v_r^d T2_k[r] H_km(r, e) for
+  // the T2 contraction of one step's H (rows m' = 2 s + o of lane, columns n = 4 r + e of
+  // r = 4 cg .. 4 cg + 3): o = 0 holds Re H (A += T2 Re H), o = 1 Im H (A += i T2 Im H); the
+  // lane pair's sums meet by a shuffle and the four column groups' in part[cg]
+  // Slot s = 3 k + m gives Q_{k,m,d}(e) = sum_r v_r^d T2_k[r] H_km(r, e) for
   // d = 0 .. 2 - m, sum index 6 k + {0, 3, 5}[m] + d (the moments combine them at the end)
-  auto avg_contract_tay = [&](const float (&H)[16]) {
+  auto avg_contract = [&](const float (&H)[16]) {
     const int s = 16 * qtr + (lane >> 1), o = lane & 1, k = s / 3, m = s - 3 * k;
     float pr[3][4], pi[3][4];
     #pragma unroll
@@ -455,19 +423,15 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
       }
     }
   };
-  auto avg_contract = [&](const float (&H)[16]) {
-    if (TAY) avg_contract_tay(H);
-    else avg_contract_plain(H);
-  };
   // compensated accumulation of the four column groups' sums (fixed order):
   // compute thread tid owns value i = tid & 7 of row k = tid >> 3 (Taylor: and
   // of row k + 64)
   float ks[2] = {0.f, 0.f}, kc[2] = {0.f, 0.f};
   auto avg_accumulate = [&]() {
     #pragma unroll
-    for (int u = 0; u < (TAY ? 2 : 1); ++u) {
+    for (int u = 0; u < 2; ++u) {
       const int k = (tid >> 3) + 64 * u, i = tid & 7;
-      if (TAY && k >= kTayOut) continue;
+      if (k >= kTayOut) continue;
       float x = part[k * 8 + i];
       #pragma unroll
       for (int c = 1; c < 4; ++c) x += part[(c * kPartRows + k) * 8 + i];
@@ -477,17 +441,6 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
       ks[u] = tt;
     }
   };
-  // a baseline's averages out, the sums reset for the next (not Taylor: one
-  // baseline per CTA there)
-  auto flush_avg = [&](int64_t blf) {
-    const int k = tid >> 3, i = tid & 7;     // value i = (re, im) of pol i / 2
-    if (k < a.n_acc)
-      reinterpret_cast<float*>(a.avg)[((size_t)k * a.n_bl + blf) * 8 + i] =
-          (float)(((double)ks[0] - (double)kc[0]) * a.inv_n);
-    ks[0] = 0.f;
-    kc[0] = 0.f;
-  };
-
   // the 16 compute warps' own barrier (the MMA-issuing warp is not in it)
   auto csync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(kTt5Compute) : "memory"); };
   // a bounded mbarrier wait that also gives up once another thread has raised s_bad
@@ -567,14 +520,8 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
       if (tid == 0 && !s_bad) mbar_arrive(&mbar[4]);
     }
 
-    int tt_run = 0;                          // the time step of step t
-    int64_t bl_run = bl0;                    // and its baseline (Taylor: step t is time t of bl0)
-    for (int t = 0; t < n_steps && !s_bad;
-         ++t, tt_run = (TAY || tt_run + 1 == a.n_time) ? 0 : tt_run + 1, bl_run += (!TAY && tt_run == 0)) {
-      const int tt = TAY ? t : tt_run;
-      const int64_t bl = TAY ? bl0 : bl_run;
+    for (int t = 0; t < n_steps && !s_bad; ++t) {
       const int buf = t & 1;
-      const bool bl_last = !TAY && tt == a.n_time - 1 && t + 1 < n_steps;   // another baseline follows
       float* strip = strip0 + (size_t)buf * n16 * 8;
       // ---- C1 (beside the subtraction MMAs): the next step's strip and
       // phases, the previous step's T2 contraction, T1 and T2 of the averaged
@@ -586,22 +533,12 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
         if ((t + 1) & 1) ++issued1;
         else ++issued0;
       }
-      // the next baseline's model matrices into mtab (free since the previous
-      // step formed this step's A_s) by asynchronous copies, before this step
-      // forms the next step's A_s in C3
-      if (SUB && bl_last && tid < kTc5Src * 4 && (tid >> 2) < n_sub_slots) {
-        const unsigned sa = (unsigned)__cvta_generic_to_shared(mtab + tid);
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa),
-                     "l"(a.M_sub + ((size_t)(tid >> 2) * a.n_bl + bl + 1) * 4 + (tid & 3)) : "memory");
-        asm volatile("cp.async.commit_group;" ::: "memory");
-      }
       float2 t1v[12];
       if (ACC) {
         if (t > 0) avg_contract(H);          // the previous step's H with its T2 (still in t2a)
         if (!wait_ph(t)) s_bad = 1;
         csync();                             // parts written; t2a free
         if (t > 0) avg_accumulate();
-        if (!TAY && tt == 0 && t > 0) flush_avg(bl - 1);   // the previous baseline is complete
         aa_compute(t1v, ph_slot(t) + kTc5Src);
         t2_fill(t2a, ph_slot(t) + kTc5Src);
       }
@@ -631,7 +568,7 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
       csync();
       if (ACC && tid == 0) mbar_arrive(&mbar[5]);
       if (SUB && tid == 0) {
-        bulk_store(a.dst + ((size_t)tt * a.n_bl + bl) * a.n_chan * 2, strip, strip_bytes);
+        bulk_store(a.dst + ((size_t)t * a.n_bl + bl0) * a.n_chan * 2, strip, strip_bytes);
         bulk_commit();
       }
       // ---- C3 (beside the average MMAs): the next step's subtraction tables
@@ -641,7 +578,6 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
         if (!wait_ph(t + 1)) s_bad = 1;
         bs_fill(ph_slot(t + 1));
         t2_fill(t2s, ph_slot(t + 1));
-        if (bl_last) asm volatile("cp.async.wait_all;" ::: "memory");   // this thread's model copy
         csync();
         as_store_hi(as_lo);
       }
@@ -680,8 +616,7 @@ __global__ void __launch_bounds__(kTt5Threads, 1) k_taylor_pass_tc05(BlockPassAr
       csync();
       avg_accumulate();
     }
-    if (ACC && !s_bad && !TAY) flush_avg(bl0 + nbl - 1);
-    if (ACC && !s_bad && TAY) {
+    if (ACC && !s_bad) {
       // the moments M_kn = sum_{m <= n} C(n, m) Q_{k,m,n-m} from the compensated sums
       // (the coefficient table is no longer read: its words hold them)
       float* qs = reinterpret_cast<float*>(cf);  // [128][8][2]: sum, compensation
