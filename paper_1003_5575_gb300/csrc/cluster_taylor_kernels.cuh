@@ -28,11 +28,12 @@
 // iterate) in float-float arithmetic (about 47 bits).  The 4x4 systems of the
 // sweep and of the step are solved in FP32 and refined once from a float-float
 // residual; where a pivot is below 1e-3 of its scale they are solved in FP64.
-// Measured (128 antennas, 20 sweeps): 184 us a source where the launches took 630
+// Measured (128 antennas, 20 sweeps): 176 us a source where the launches took 630
 // (20 sweeps of 12.8 us, 19 row sums of 12.0 and 19 steps of 5.4, and their gaps);
 // error of a 50-source cadence against 64 bits 3.7e-6 with the launches, 6e-7
 // here.  In cycles an iteration: row sums 4 200, Gram sums 1 300, the step's sums
-// 3 100, the step 3 800, normal matrix 1 250, solve 2 000, exchange 1 600.
+// 3 100, the step 3 000 (one lane an entry of its matrix, the CTAs' sums pairwise; every
+// lane doing all of it took 3 800), normal matrix 1 250, solve 2 000, exchange 1 600.
 // The rows of all antennas have to fit the cluster's shared memory, up to about
 // 175 antennas; larger arrays keep the launches (k_als_taylor_sweep).
 #pragma once
@@ -176,26 +177,29 @@ __device__ inline bool ct_schur4f(const float2 (&C)[4][4], const float2 (&b)[4],
 // The rotation step k = -h^-1 g from the 18 sums (float-float): h in 2x2 blocks,
 // solved in FP32 and refined once, or in FP64 where a pivot is below 1e-3 of
 // the largest diagonal entry.  Returns whether the step is taken.
-__device__ inline bool ct_step(const FF (&s)[kCtRot], double S, double mu4, FF (&k)[4]) {
-  const FF c4 = ff_of(2.0 * S * S * mu4), c2 = ff_of(2.0 * S);
-  const FF zero = {0.f, 0.f};
-  FF h[10], g[4];                          // (0,0) (0,1) (0,2) (0,3) (1,1) (1,2) (1,3) (2,2) (2,3) (3,3); -g
-  auto two = [](FF a) { a.hi *= 2.f; a.lo *= 2.f; return a; };
-  const FF r01 = ff_add(s[0], s[1]);
-  const FF sub[10] = {two(s[0]), zero, s[2], s[3], two(s[1]), s[2], s[3], two(r01), zero, two(r01)};
+__device__ inline bool ct_step(FF t, int lane, FF c4, FF c2, FF (&k)[4]) {
+  auto from = [](FF v, int src) { return FF{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)}; };
+  // lanes 0 .. 9: entry (0,0) (0,1) (0,2) (0,3) (1,1) (1,2) (1,3) (2,2) (2,3) (3,3) of the matrix,
+  // c4 s[8 + lane] - c2 sub; lanes 10 .. 13: c2 s[4 ..], minus the gradient
+  const int i = lane < 14 ? lane : 13;
+  const bool is_h = i < 10;
+  const FF first = from(t, is_h ? 8 + i : i - 6);
+  const FF b1 = from(t, (int)((0x0003213200ull >> (4 * i)) & 15u)), b2 = from(t, 1);
+  const float f1 = is_h ? (float)((0x2021121102ull >> (4 * i)) & 15u) : 0.f, f2 = i == 7 || i == 9 ? 2.f : 0.f;
+  const FF sub = ff_add(FF{f1 * b1.hi, f1 * b1.lo}, FF{f2 * b2.hi, f2 * b2.lo});
+  const FF mine = ff_norm(ff_add(ff_mul(is_h ? c4 : c2, first), ff_neg(ff_mul(c2, sub))));
+  float h[14];
   #pragma unroll
-  for (int i = 0; i < 10; ++i) h[i] = ff_norm(ff_add(ff_mul(c4, s[8 + i]), ff_neg(ff_mul(c2, sub[i]))));
-  #pragma unroll
-  for (int b = 0; b < 4; ++b) g[b] = ff_norm(ff_mul(c2, s[4 + b]));
-  const float dmax = fmaxf(fmaxf(h[0].hi, h[4].hi), fmaxf(h[7].hi, h[9].hi));
+  for (int j = 0; j < 14; ++j) h[j] = __shfl_sync(0xffffffffu, mine.hi, j);
+  const float dmax = fmaxf(fmaxf(h[0], h[4]), fmaxf(h[7], h[9]));
   if (!(dmax > 0.f)) return false;
-  const float h00 = h[0].hi, h01 = h[1].hi, h02 = h[2].hi, h03 = h[3].hi, h11 = h[4].hi, h12 = h[5].hi, h13 = h[6].hi;
+  const float h00 = h[0], h01 = h[1], h02 = h[2], h03 = h[3], h11 = h[4], h12 = h[5], h13 = h[6];
   const float detA = h00 * h11 - h01 * h01, idA = __frcp_rn(detA);
   const float A00 = h11 * idA, A01 = -h01 * idA, A11 = h00 * idA;
   const float T00 = A00 * h02 + A01 * h12, T01 = A00 * h03 + A01 * h13;
   const float T10 = A01 * h02 + A11 * h12, T11 = A01 * h03 + A11 * h13;
-  const float S00 = h[7].hi - (h02 * T00 + h12 * T10), S01 = h[8].hi - (h02 * T01 + h12 * T11);
-  const float S11 = h[9].hi - (h03 * T01 + h13 * T11);
+  const float S00 = h[7] - (h02 * T00 + h12 * T10), S01 = h[8] - (h02 * T01 + h12 * T11);
+  const float S11 = h[9] - (h03 * T01 + h13 * T11);
   const float detS = S00 * S11 - S01 * S01, idS = __frcp_rn(detS), tol = 1e-3f * dmax;
   if (h00 > tol && detA > tol * h00 && S00 > tol && detS > tol * S00) {
     auto solve = [&](const float (&r)[4], float (&x)[4]) {
@@ -206,27 +210,27 @@ __device__ inline bool ct_step(const FF (&s)[kCtRot], double S, double mu4, FF (
       x[0] = A00 * w0 + A01 * w1;
       x[1] = A01 * w0 + A11 * w1;
     };
-    float r[4] = {g[0].hi, g[1].hi, g[2].hi, g[3].hi}, x[4], d[4];
+    float r[4] = {h[10], h[11], h[12], h[13]}, x[4], d[4];
     solve(r, x);
-    const int at[4][4] = {{0, 1, 2, 3}, {1, 4, 5, 6}, {2, 5, 7, 8}, {3, 6, 8, 9}};
+    // lane u & 3: the residual of row u, whose entries sit on lanes 0 1 2 3 | 1 4 5 6 | 2 5 7 8 | 3 6 8 9
+    const unsigned row = lane & 2 ? (lane & 1 ? 0x9863u : 0x8752u) : (lane & 1 ? 0x6541u : 0x3210u);
+    FF res = from(mine, 10 + (lane & 3));
     #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      FF t = g[i];
-      #pragma unroll
-      for (int j = 0; j < 4; ++j) t = ff_mac(-x[j], h[at[i][j]], t);
-      r[i] = ff_f(t);
-    }
+    for (int j = 0; j < 4; ++j) res = ff_mac(-x[j], from(mine, (int)((row >> (4 * j)) & 15u)), res);
+    const float rf = ff_f(res);
+    #pragma unroll
+    for (int j = 0; j < 4; ++j) r[j] = __shfl_sync(0xffffffffu, rf, j);
     solve(r, d);
     #pragma unroll
-    for (int i = 0; i < 4; ++i) k[i] = ff_two_sum(x[i], d[i]);
+    for (int j = 0; j < 4; ++j) k[j] = ff_two_sum(x[j], d[j]);
     return true;
   }
   // FP64 (the pivot test itself at 1e-6 of the largest diagonal entry)
   double H[10], r[4];
   #pragma unroll
-  for (int i = 0; i < 10; ++i) H[i] = ff_d(h[i]);
+  for (int j = 0; j < 10; ++j) H[j] = ff_d(from(mine, j));
   #pragma unroll
-  for (int i = 0; i < 4; ++i) r[i] = ff_d(g[i]);
+  for (int j = 0; j < 4; ++j) r[j] = ff_d(from(mine, 10 + j));
   const double dm = fmax(fmax(H[0], H[4]), fmax(H[7], H[9])), tol64 = 1e-6 * dm;
   const double dA = H[0] * H[4] - H[1] * H[1], iA = 1.0 / dA;
   const double a00 = H[4] * iA, a01 = -H[1] * iA, a11 = H[0] * iA;
@@ -305,6 +309,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_taylor(ClusterTaylorA
   const uint32_t dst_bar = sends ? cluster_map(tc05::smem_u32(&s_bar[0]), dst_rank) : 0u;
   const float mu2 = (float)a.mu2, mu4 = (float)a.mu4;
   const FF fS = ff_of(a.S), fmu0S = ff_of(a.mu0 * a.S), fmu2S = ff_of(a.mu2 * a.S), fmu4S = ff_of(a.mu4 * a.S);
+  const FF c4 = ff_of(2.0 * a.S * a.S * a.mu4), c2 = ff_of(2.0 * a.S);
   // lanes 0 .. 7: entry e of X_p = [G H] (row er, column ec of 4), the rotated iterate
   const int e = lane & 7, er = (e & 3) >> 1, ec = (e < 4 ? 0 : 2) + (e & 1);
   FFC X = ffc_zero(), Xprev = X;
@@ -471,11 +476,14 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_taylor(ClusterTaylorA
         for (int i = 0; i < kCtRot; ++i) s_r[slot][i] = live ? 0.5f * val[i] : 0.f;
       __syncthreads();
       if (tid < kCtRot) {
-        FF t = {s_r[0][tid], 0.f};
-        for (int s = 1; s < a.apc; ++s) {
-          const FF x = {s_r[s][tid], 0.f};
-          t = ff_add(t, x);
-        }
+        FF v[kClMaxSlots];
+        #pragma unroll
+        for (int q = 0; q < kClMaxSlots; ++q) v[q] = FF{q < a.apc ? s_r[q][tid] : 0.f, 0.f};
+        #pragma unroll
+        for (int o = kClMaxSlots / 2; o >= 1; o >>= 1)
+          #pragma unroll
+          for (int q = 0; q < o; ++q) v[q] = ff_add(v[q], v[q + o]);
+        const FF t = v[0];
         s_rsum[tid] = ff_norm(t);
       }
       __syncthreads();
@@ -490,20 +498,19 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_taylor(ClusterTaylorA
       }
       cluster_wait(&s_rbar[rb], (uint32_t)(n_red >> 1) & 1u, bad);
       ++n_red;
-      FF sum[kCtRot];
-      {
-        FF t = {0.f, 0.f};
-        if (lane < kCtRot) {
-          t = s_red[rb][0][lane];
-          for (int r = 1; r < CS; ++r) t = ff_add(t, s_red[rb][r][lane]);
-        }
+      FF t = {0.f, 0.f};
+      if (lane < kCtRot) {                             // the CTAs' sums, pairwise
+        FF v[kClMaxCta];
         #pragma unroll
-        for (int i = 0; i < kCtRot; ++i) {
-          sum[i].hi = __shfl_sync(0xffffffffu, t.hi, i);
-          sum[i].lo = __shfl_sync(0xffffffffu, t.lo, i);
-        }
+        for (int r = 0; r < kClMaxCta; ++r) v[r] = r < CS ? s_red[rb][r][lane] : t;
+        #pragma unroll
+        for (int o = kClMaxCta / 2; o >= 1; o >>= 1)
+          #pragma unroll
+          for (int r = 0; r < o; ++r) v[r] = ff_add(v[r], v[r + o]);
+        t = v[0];
       }
-      if (!ct_step(sum, a.S, a.mu4, k)) {
+      __syncwarp();
+      if (!ct_step(t, lane, c4, c2, k)) {
         const FF z = {0.f, 0.f};
         k[0] = k[1] = k[2] = k[3] = z;
       }
