@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -39,7 +40,8 @@ struct rts_peel_t {
   bool tay_tc05 = false;             // the Taylor cadence in blocks: its passes as tcgen05 MMAs,
   bool tay_strip = false;            // or by k_taylor_pass_strip
   int strip_qh = 0;                  // FP32 passes by k_block_pass_strip<strip_qh> (0: k_block_pass)
-  int* d_perr = nullptr;           // [1] set by a tcgen05 pass whose mbarrier wait ran out
+  int* d_perr = nullptr;           // [1] set by a tcgen05 pass whose mbarrier wait ran out; d_status follows
+  std::vector<int32_t> status_in;  // [1 + max_sources] the same on the host (read_status)
   int64_t n_bl = 0;
   double nu0 = 0, dnu = 0;
   int device = 0;
@@ -349,11 +351,11 @@ int launch_als(rts_peel_t* h, const void* avg, double S, void* jones_out, int sl
 const double2* als_solution(rts_peel_t* h) { return h->d_J[h->n_iter & 1]; }
 
 int read_status(rts_peel_t* h, int32_t n, int32_t* h_status, cudaStream_t s) {
-  RTS_CUDA(h, cudaMemcpyAsync(h_status, h->d_status, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, s));
-  int perr = 0;
-  if (h->d_perr) RTS_CUDA(h, cudaMemcpyAsync(&perr, h->d_perr, sizeof(int), cudaMemcpyDeviceToHost, s));
+  // the pass's flag sits before the statuses: one copy (a second one took 10 us)
+  RTS_CUDA(h, cudaMemcpyAsync(h->status_in.data(), h->d_perr, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost, s));
   RTS_CUDA(h, cudaStreamSynchronize(s));
-  if (perr) return fail(h, RTS_ECUDA, "a tensor-core completion wait of the blocked pass timed out");
+  std::copy(h->status_in.begin() + 1, h->status_in.begin() + 1 + n, h_status);
+  if (h->status_in[0]) return fail(h, RTS_ECUDA, "a tensor-core completion wait of the blocked pass timed out");
   for (int k = 0; k < n; ++k)
     if (h_status[k] == kSolveStatusTimeout)
       return fail(h, RTS_ECUDA, "a grid barrier of the block solve timed out at source " + std::to_string(k));
@@ -467,8 +469,6 @@ int ensure_block_workspace(rts_peel_t* h) {
   RTS_CUDA(h, cudaEventCreateWithFlags(&h->b_ev_done, cudaEventDisableTiming));
   int rc = setup_block_solve(h);
   if (rc) return rc;
-  RTS_CUDA(h, cudaMalloc((void**)&h->d_perr, sizeof(int)));
-  RTS_CUDA(h, cudaMemset(h->d_perr, 0, sizeof(int)));
   if (h->block_tc05) {
     rc = tc05_nq(h->n_chan) == 16 ? set_tc05_smem<16>(h) : tc05_nq(h->n_chan) == 32 ? set_tc05_smem<32>(h) : set_tc05_smem<48>(h);
     if (rc) return rc;
@@ -1263,7 +1263,7 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
       {(void**)&h->d_Jf[1], n_cplx_ant * sizeof(float2)},
       {(void**)&h->d_norms, (size_t)h->n_ant * 4 * sizeof(double)},
       {(void**)&h->d_flag, sizeof(int)},
-      {(void**)&h->d_status, (size_t)h->max_sources * sizeof(int)},
+      {(void**)&h->d_perr, (size_t)(1 + h->max_sources) * sizeof(int)},
       {(void**)&h->d_rel, (size_t)h->max_sources * sizeof(double)},
       {(void**)&h->d_src, (size_t)h->max_sources * 3 * sizeof(double)},
       {(void**)&h->d_jones_stage, (size_t)h->max_sources * n_cplx_ant * h->elem},
@@ -1277,8 +1277,10 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
   if ((e = cudaMemcpy(h->d_freq_c, fc.data(), fc.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess)
     return bail(e, "copy frequencies");
   if ((e = cudaMemset(h->d_flag, 0, sizeof(int))) != cudaSuccess) return bail(e, "clear flag");
-  if ((e = cudaMemset(h->d_status, 0, (size_t)h->max_sources * sizeof(int))) != cudaSuccess)
+  if ((e = cudaMemset(h->d_perr, 0, (size_t)(1 + h->max_sources) * sizeof(int))) != cudaSuccess)
     return bail(e, "clear status");
+  h->d_status = h->d_perr + 1;
+  h->status_in.resize(1 + h->max_sources);
   if (h->precision == RTS_PREC_FP64) {
     // phasor tables where nu_0 + c dnu is every channel to FP64 rounding (a phase of
     // 1e3 turns then moves by less than the FP64 phase itself is rounded) and they
@@ -1809,7 +1811,7 @@ void rts_peel_destroy(rts_peel_t* h) {
   int prev = -1;
   if (cudaGetDevice(&prev) == cudaSuccess && prev != h->device) cudaSetDevice(h->device);
   void* ptrs[] = {h->d_uvw, h->d_bl_ant, h->d_freq_c, h->d_avg, h->d_J[0], h->d_J[1], h->d_Jf[0],
-                  h->d_Jf[1], h->d_norms, h->d_flag, h->d_status, h->d_rel, h->d_src, h->d_jones_stage,
+                  h->d_Jf[1], h->d_norms, h->d_flag, h->d_rel, h->d_src, h->d_jones_stage,
                   h->b_avg, h->b_aph, h->b_model, h->b_sync, h->b_part, h->cl_V, h->cl_D, h->d_perr, h->d_aph, h->d_tab64[0], h->d_tab64[1], h->t_mom, h->t_X[0],
                   h->t_X[1], h->t_Xf[0], h->t_Xf[1], h->t_rot_part, h->t_rot_count, h->t_rot_step};
   for (void* p : ptrs)
