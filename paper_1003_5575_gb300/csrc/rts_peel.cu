@@ -224,14 +224,6 @@ StreamArgs stream_args(rts_peel_t* h, const void* src, void* dst, void* avg) {
   return a;
 }
 
-template <bool TAB>
-void launch_stream_fp64(bool sub, bool acc, const StreamArgs& a, const Fp64Tables& tb, size_t smem, cudaStream_t s) {
-  const dim3 grid((unsigned)a.n_bl), block(kStreamThreads);
-  if (sub && acc) k_stream_fp64<true, true, TAB><<<grid, block, smem, s>>>(a, tb);
-  else if (sub) k_stream_fp64<true, false, TAB><<<grid, block, smem, s>>>(a, tb);
-  else k_stream_fp64<false, true, TAB><<<grid, block, smem, s>>>(a, tb);
-}
-
 // one streaming pass: sub (subtract source) and/or acc (average for source).
 // in_peel: the passes of a cadence, which own the handle's workspace (the FP64
 // phasor tables among it); rts_peel_rotate_average may run beside one
@@ -245,7 +237,7 @@ int launch_stream(rts_peel_t* h, bool sub, bool acc, bool in_peel, const StreamA
     tb.R = h->tab64_r; tb.Q = h->tab64_q;
     tb.lr = 0;
     while ((1 << tb.lr) < tb.R) ++tb.lr;
-    const size_t per_t = (size_t)2 * (tb.Q + tb.R) * sizeof(double2);
+    const size_t per_t = (size_t)2 * tb.Q * sizeof(double2);
     tb.n_t = (int)std::max<size_t>(1, std::min<size_t>(h->n_time, kFp64TableBytes / per_t));
     tb.sub = h->d_tab64[h->tab64_at];
     if (acc) {
@@ -254,7 +246,10 @@ int launch_stream(rts_peel_t* h, bool sub, bool acc, bool in_peel, const StreamA
                                                              a.nu0_c, a.dnu_c, h->d_tab64[h->tab64_at]);
     }
     tb.acc = h->d_tab64[h->tab64_at];
-    launch_stream_fp64<true>(sub, acc, a, tb, tb.n_t * per_t, s);
+    const size_t smem = tb.n_t * per_t;
+    if (sub && acc) k_stream_fp64_tab<true, true><<<grid, kFp64Threads, smem, s>>>(a, tb);
+    else if (sub) k_stream_fp64_tab<true, false><<<grid, kFp64Threads, smem, s>>>(a, tb);
+    else k_stream_fp64_tab<false, true><<<grid, kFp64Threads, smem, s>>>(a, tb);
     span.end(acc ? 2 : 1);
     return check_launch(h, "streaming kernel launch");
   }
@@ -265,7 +260,10 @@ int launch_stream(rts_peel_t* h, bool sub, bool acc, bool in_peel, const StreamA
     else if (sub) k_stream_mixed<true, false><<<grid, block, smem, s>>>(a);
     else k_stream_mixed<false, true><<<grid, block, smem, s>>>(a);
   } else {
-    launch_stream_fp64<false>(sub, acc, a, Fp64Tables(), (size_t)h->n_time * 2 * sizeof(double), s);
+    const size_t smem = (size_t)h->n_time * 2 * sizeof(double);
+    if (sub && acc) k_stream_fp64<true, true><<<grid, block, smem, s>>>(a);
+    else if (sub) k_stream_fp64<true, false><<<grid, block, smem, s>>>(a);
+    else k_stream_fp64<false, true><<<grid, block, smem, s>>>(a);
   }
   span.end(1);
   return check_launch(h, "streaming kernel launch");
@@ -1289,9 +1287,13 @@ int rts_peel_init(const rts_peel_config* cfg, rts_peel_t** out) {
     for (int c = 0; c < h->n_chan && uniform; ++c) uniform = std::fabs(f[c] - (nu0 + c * dnu)) <= 4.5e-16 * f[c];
     const int R = fp64_table_r(h->n_chan), Q = (h->n_chan + R - 1) / R;
     const size_t bytes = (size_t)h->n_time * h->n_ant * (Q + R) * sizeof(double2);
-    if (uniform && bytes <= ((size_t)128 << 20)) {
-      for (int k = 0; k < 2; ++k)
-        if ((e = cudaMalloc((void**)&h->d_tab64[k], bytes)) != cudaSuccess) return bail(e, "cudaMalloc(phasor tables)");
+    if (uniform && bytes <= ((size_t)128 << 20) && (size_t)2 * Q * sizeof(double2) <= kFp64TableBytes) {
+      // no room for them: a sincospi a sample
+      if (cudaMalloc((void**)&h->d_tab64[0], bytes) != cudaSuccess || cudaMalloc((void**)&h->d_tab64[1], bytes) != cudaSuccess) {
+        cudaGetLastError();
+        if (h->d_tab64[0]) cudaFree(h->d_tab64[0]);
+        h->d_tab64[0] = h->d_tab64[1] = nullptr;
+      }
       h->tab64_q = Q; h->tab64_r = R;
     }
   }

@@ -197,16 +197,16 @@ __global__ void __launch_bounds__(kStreamThreads, 3) k_stream_mixed(StreamArgs a
 // and, because tau_ij = tau_i - tau_j, each table of a baseline is the product
 // T_i conj(T_j) of its antennas' tables, which k_fp64_ant_tables forms once per
 // source ([n_time][n_ant][Q + R]).  At 128 antennas x 128 channels x 8 times x 50
-// sources the whole cadence, solves included, went from 111 to 48.6 ms.  Other
+// sources the whole cadence, solves included, went from 111 ms to 36.4.  Other
 // frequency lists (uniform to 1e-9 only) keep one sincospi per sample and role
-// (TAB = false).
+// (k_stream_fp64).
 
 constexpr size_t kFp64TableBytes = 32 * 1024;    // a CTA's baseline tables, at most (but one time's)
 
-// R of the tables: about sqrt(n_chan), a power of two
+// R of the tables: about sqrt(n_chan), a power of two, at most kFp64Threads
 __host__ inline int fp64_table_r(int n_chan) {
   int r = 1;
-  while (r * r < n_chan) r *= 2;
+  while (r * r < n_chan && r < 128) r *= 2;
   return r;
 }
 
@@ -232,28 +232,134 @@ struct Fp64Tables {
   int n_t;                  // times whose baseline tables a CTA holds at once
 };
 
-template <bool SUB, bool ACC, bool TAB>
-__global__ void __launch_bounds__(kStreamThreads) k_stream_fp64(StreamArgs a, Fp64Tables tb) {
-  extern __shared__ __align__(16) unsigned char s_f64[];
-  // TAB: [n_t][sub, acc][Q + R] double2; else [n_time][2] double: tau_sub, tau_acc
-  double2* s_tab = reinterpret_cast<double2*>(s_f64);
-  double* s_tau = reinterpret_cast<double*>(s_f64);
-  __shared__ double2 s_M[4];
-  __shared__ double s_red[kStreamThreads / 32][8];
-  const int64_t bl = blockIdx.x;
-  const int2 ij = a.bl_ant[bl];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (!TAB)
-    for (int t = tid; t < a.n_time; t += kStreamThreads) {
-      if (SUB) s_tau[2 * t] = delay_m(a.uvw, a.n_ant, t, ij.x, ij.y, a.sub);
-      if (ACC) s_tau[2 * t + 1] = delay_m(a.uvw, a.n_ant, t, ij.x, ij.y, a.acc);
-    }
-  if (SUB && tid < 4) {                      // -S J_i J_j^H, one entry a thread
+// -S J_i J_j^H of the subtracted source, one entry a thread
+__device__ __forceinline__ void fp64_model(const StreamArgs& a, int2 ij, int tid, double2* s_M) {
+  if (tid < 4) {
     const int r = tid >> 1, c = tid & 1;
     const double2 *Ji = a.Jsub + (size_t)ij.x * 4 + 2 * r, *Jj = a.Jsub + (size_t)ij.y * 4 + 2 * c;
     const double2 m = cadd(cmulc(Ji[0], Jj[0]), cmulc(Ji[1], Jj[1]));
     s_M[tid] = make_double2(-a.sub.S * m.x, -a.sub.S * m.y);
   }
+}
+// a CTA's averages: warp totals by halving exchanges (9 additions a lane for the 8 sums),
+// then one thread a sum adds the warps' in warp order
+template <int WARPS>
+__device__ __forceinline__ void fp64_average(const StreamArgs& a, int64_t bl, double (&acc)[8], double (*s_red)[8]) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const double v = warp_reduce_scatter8d(acc, lane);
+  if ((lane & 3) == 0) s_red[warp][lane >> 2] = v;
+  __syncthreads();
+  if (tid < 8) {
+    double t = 0.0;
+    #pragma unroll
+    for (int w = 0; w < WARPS; ++w) t += s_red[w][tid];
+    static_cast<double*>(a.avg)[bl * 8 + tid] = t * a.inv_n;
+  }
+}
+
+// The pass from phasor tables.  A thread owns channel offset r of one time and walks
+// the tiles q, so T2[r] is applied once a (time, r) on each side of the walk: to the
+// model before it and to the sums after it; a sample then takes 32 multiply-adds
+// (36 with a walk of 8 tiles), where the product of both tables for every sample
+// took 40.  Threads: groups of R offsets, each a (time, part of the tiles).
+constexpr int kFp64Threads = 128;
+template <bool SUB, bool ACC>
+__global__ void __launch_bounds__(kFp64Threads) k_stream_fp64_tab(StreamArgs a, Fp64Tables tb) {
+  extern __shared__ __align__(16) unsigned char s_f64[];
+  double2* s_tab = reinterpret_cast<double2*>(s_f64);            // [n_t][sub, acc][Q]
+  __shared__ double2 s_M[4];
+  __shared__ double s_red[kFp64Threads / 32][8];
+  const int64_t bl = blockIdx.x;
+  const int2 ij = a.bl_ant[bl];
+  const int tid = threadIdx.x, r = tid & (tb.R - 1), g = tid >> tb.lr, G = kFp64Threads >> tb.lr;
+  if (SUB) fp64_model(a, ij, tid, s_M);
+  double acc[8];
+  #pragma unroll
+  for (int k = 0; k < 8; ++k) acc[k] = 0.0;
+  const double2* src = static_cast<const double2*>(a.src);
+  double2* dst = static_cast<double2*>(a.dst);
+  const int n_e = tb.Q + tb.R;
+  for (int t0 = 0; t0 < a.n_time; t0 += tb.n_t) {
+    const int nt = min(tb.n_t, a.n_time - t0);
+    if (t0) __syncthreads();                 // the previous times' tables are read
+    for (int x = tid; x < nt * 2 * tb.Q; x += kFp64Threads) {
+      const int row = x / tb.Q, e = x - row * tb.Q;
+      if ((row & 1) ? !ACC : !SUB) continue;
+      const double2* tab = (row & 1) ? tb.acc : tb.sub;
+      const size_t at = (size_t)(t0 + (row >> 1)) * a.n_ant;
+      s_tab[x] = cmulc(tab[(at + ij.x) * n_e + e], tab[(at + ij.y) * n_e + e]);
+    }
+    __syncthreads();
+    const int parts = max(1, G / nt);
+    for (int it = g; it < nt * parts; it += G) {
+      const int t = it % nt, part = it / nt;
+      const size_t ti = ((size_t)(t0 + t) * a.n_ant + ij.x) * n_e + tb.Q + r, tj = ti + (size_t)(ij.y - ij.x) * n_e;
+      double2 A[4], s[4];
+      if (SUB) {
+        const double2 z = cmulc(tb.sub[ti], tb.sub[tj]);
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) A[e] = cmulc(s_M[e], z);
+      }
+      if (ACC) {
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) s[e] = make_double2(0.0, 0.0);
+      }
+      const double2* T = s_tab + (size_t)2 * t * tb.Q;
+      const size_t row = ((size_t)(t0 + t) * a.n_bl + bl) * a.n_chan;
+      #pragma unroll 2
+      for (int q = part; q < tb.Q; q += parts) {
+        const int c = (q << tb.lr) + r;
+        if (c >= a.n_chan) break;
+        const size_t idx = (row + c) * 4;
+        double2 x[4];
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = src[idx + e];
+        if (SUB) {
+          const double2 z = T[q];
+          #pragma unroll
+          for (int e = 0; e < 4; ++e) {       // x += A conj(z)
+            x[e].x = fma(A[e].x, z.x, fma(A[e].y, z.y, x[e].x));
+            x[e].y = fma(A[e].y, z.x, fma(-A[e].x, z.y, x[e].y));
+            dst[idx + e] = x[e];
+          }
+        }
+        if (ACC) {
+          const double2 z = T[tb.Q + q];
+          #pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            s[e].x = fma(x[e].x, z.x, fma(-x[e].y, z.y, s[e].x));
+            s[e].y = fma(x[e].x, z.y, fma(x[e].y, z.x, s[e].y));
+          }
+        }
+      }
+      if (ACC) {
+        const double2 z = cmulc(tb.acc[ti], tb.acc[tj]);
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          acc[2 * e] = fma(s[e].x, z.x, fma(-s[e].y, z.y, acc[2 * e]));
+          acc[2 * e + 1] = fma(s[e].x, z.y, fma(s[e].y, z.x, acc[2 * e + 1]));
+        }
+      }
+    }
+  }
+  if (ACC) fp64_average<kFp64Threads / 32>(a, bl, acc, s_red);
+}
+
+// The pass on any frequency list: one sincospi a sample and role.
+template <bool SUB, bool ACC>
+__global__ void __launch_bounds__(kStreamThreads) k_stream_fp64(StreamArgs a) {
+  extern __shared__ __align__(16) unsigned char s_f64[];
+  double* s_tau = reinterpret_cast<double*>(s_f64);              // [n_time][2]: tau_sub, tau_acc
+  __shared__ double2 s_M[4];
+  __shared__ double s_red[kStreamThreads / 32][8];
+  const int64_t bl = blockIdx.x;
+  const int2 ij = a.bl_ant[bl];
+  const int tid = threadIdx.x;
+  for (int t = tid; t < a.n_time; t += kStreamThreads) {
+    if (SUB) s_tau[2 * t] = delay_m(a.uvw, a.n_ant, t, ij.x, ij.y, a.sub);
+    if (ACC) s_tau[2 * t + 1] = delay_m(a.uvw, a.n_ant, t, ij.x, ij.y, a.acc);
+  }
+  if (SUB) fp64_model(a, ij, tid, s_M);
   __syncthreads();
   double2 M[4];
   if (SUB) {
@@ -265,66 +371,33 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream_fp64(StreamArgs a, Fp
   for (int k = 0; k < 8; ++k) acc[k] = 0.0;
   const double2* src = static_cast<const double2*>(a.src);
   double2* dst = static_cast<double2*>(a.dst);
-  const int n_e = tb.Q + tb.R;
-  const int t_step = TAB ? tb.n_t : a.n_time;
-  for (int t0 = 0; t0 < a.n_time; t0 += t_step) {
-    const int nt = min(t_step, a.n_time - t0);
-    if (TAB) {
-      if (t0) __syncthreads();               // the previous times' tables are read
-      for (int x = tid; x < nt * 2 * n_e; x += kStreamThreads) {
-        const int row = x / n_e, e = x - row * n_e;
-        if ((row & 1) ? !ACC : !SUB) continue;
-        const double2* g = (row & 1) ? tb.acc : tb.sub;
-        const size_t at = (size_t)(t0 + (row >> 1)) * a.n_ant;
-        s_tab[x] = cmulc(g[(at + ij.x) * n_e + e], g[(at + ij.y) * n_e + e]);
-      }
-      __syncthreads();
-    }
-    const int n_s = nt * a.n_chan;
-    TCWalk w;
-    w.init(tid, a.n_chan);
-    for (int s = tid; s < n_s; s += kStreamThreads, w.next()) {
-      const size_t idx = (((size_t)(t0 + w.t) * a.n_bl + bl) * a.n_chan + w.c) * 4;
-      double2 x[4];
+  const int n_s = a.n_time * a.n_chan;
+  TCWalk w;
+  w.init(tid, a.n_chan);
+  for (int s = tid; s < n_s; s += kStreamThreads, w.next()) {
+    const size_t idx = (((size_t)w.t * a.n_bl + bl) * a.n_chan + w.c) * 4;
+    double2 x[4];
+    #pragma unroll
+    for (int e = 0; e < 4; ++e) x[e] = src[idx + e];
+    if (SUB) {
+      const double2 ph = phasor_d(s_tau[2 * w.t] * a.freq_c[w.c]);          // exp(+2 pi i phi)
       #pragma unroll
-      for (int e = 0; e < 4; ++e) x[e] = src[idx + e];
-      auto phasor = [&](int role) {           // exp(+2 pi i phi)
-        if (!TAB) return phasor_d(s_tau[2 * w.t + role] * a.freq_c[w.c]);
-        const double2* T = s_tab + (size_t)(2 * w.t + role) * n_e;
-        return cmul(T[w.c >> tb.lr], T[tb.Q + (w.c & (tb.R - 1))]);
-      };
-      if (SUB) {
-        const double2 ph = phasor(0);
-        #pragma unroll
-        for (int e = 0; e < 4; ++e) {         // x += (-M) conj(ph)
-          x[e].x = fma(M[e].x, ph.x, fma(M[e].y, ph.y, x[e].x));
-          x[e].y = fma(M[e].y, ph.x, fma(-M[e].x, ph.y, x[e].y));
-          dst[idx + e] = x[e];
-        }
+      for (int e = 0; e < 4; ++e) {           // x += (-M) conj(ph)
+        x[e].x = fma(M[e].x, ph.x, fma(M[e].y, ph.y, x[e].x));
+        x[e].y = fma(M[e].y, ph.x, fma(-M[e].x, ph.y, x[e].y));
+        dst[idx + e] = x[e];
       }
-      if (ACC) {
-        const double2 ph = phasor(1);
-        #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          acc[2 * e] = fma(x[e].x, ph.x, fma(-x[e].y, ph.y, acc[2 * e]));
-          acc[2 * e + 1] = fma(x[e].x, ph.y, fma(x[e].y, ph.x, acc[2 * e + 1]));
-        }
+    }
+    if (ACC) {
+      const double2 ph = phasor_d(s_tau[2 * w.t + 1] * a.freq_c[w.c]);
+      #pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        acc[2 * e] = fma(x[e].x, ph.x, fma(-x[e].y, ph.y, acc[2 * e]));
+        acc[2 * e + 1] = fma(x[e].x, ph.y, fma(x[e].y, ph.x, acc[2 * e + 1]));
       }
     }
   }
-  if (ACC) {
-    // warp totals by halving exchanges (9 additions a lane for the 8 sums), then
-    // one thread a sum adds the warps' in warp order
-    const double v = warp_reduce_scatter8d(acc, lane);
-    if ((lane & 3) == 0) s_red[warp][lane >> 2] = v;
-    __syncthreads();
-    if (tid < 8) {
-      double t = 0.0;
-      #pragma unroll
-      for (int w2 = 0; w2 < kStreamThreads / 32; ++w2) t += s_red[w2][tid];
-      static_cast<double*>(a.avg)[bl * 8 + tid] = t * a.inv_n;
-    }
-  }
+  if (ACC) fp64_average<kStreamThreads / 32>(a, bl, acc, s_red);
 }
 
 }  // namespace rts

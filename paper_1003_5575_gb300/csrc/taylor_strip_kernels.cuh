@@ -8,9 +8,8 @@
 // down give s0 = sum x_r, s1 = sum (r + 1) x_r, s2 = sum (r + 1)(r + 2)/2 x_r of
 // x_r = R(16 q + r) T2[r], and sum r x_r = s1 - s0, sum r^2 x_r = 2 s2 - 3 s1 + s0.
 // Bound by the FP32 pipe and instruction issue.  At 128 antennas x 128 channels x 8
-// times and 50 sources the four passes take 2.15 ms, the tcgen05 form's 7.3; a
-// strip no longer fits a warp's registers past 256 channels, where the tcgen05
-// form (whose cost does not depend on the length up to there) keeps the pass.
+// times and 50 sources the four passes take 2.15 ms, the tcgen05 form's 7.3; past 256
+// channels a strip no longer fits a warp's registers and the tcgen05 form keeps the pass.
 #pragma once
 #include "strip_kernels.cuh"
 #include "taylor_block_kernels.cuh"

@@ -47,3 +47,15 @@ def test_fp64_cadence_matches_oracle(name, cad):
     assert jones_rel(jones.cpu().numpy(), J_ref) <= TOL["fp64"]
     check_status(name, st, st_ref, p.rel(cad.n_src), rel_ref, "fp64")
     p.close()
+
+
+WALK_CASES = [
+    ("one-time", Cadence(6, 600, 1, 2, precision="fp64", seed=226)),               # four groups share a time's tiles
+    ("three-times", Cadence(6, 100, 3, 2, precision="fp64", seed=227)),            # two groups a time, two idle
+    ("130-times", Cadence(4, 200, 130, 2, precision="fp64", seed=228)),            # tables of 78 times, then 52
+]
+
+
+@pytest.mark.parametrize("name,cad", WALK_CASES, ids=[c[0] for c in WALK_CASES])
+def test_fp64_walk_of_tiles_matches_oracle(name, cad):
+    test_fp64_cadence_matches_oracle(name, cad)
