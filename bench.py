@@ -116,10 +116,12 @@ class Clocks:
 KERNEL_SOURCES = {"k_stream_mixed<true,true>": ("common.cuh", "stream_kernels.cuh"),
                   "k_block_pass<64,true,true>": ("common.cuh", "stream_kernels.cuh", "block_kernels.cuh"),
                   "k_block_pass_tc05<true,true>": ("common.cuh", "stream_kernels.cuh", "block_kernels.cuh",
-                                                   "tc05.cuh", "block_tc05_kernels.cuh"),
-                  "k_block_pass_tc05<true,true,true>": ("common.cuh", "stream_kernels.cuh", "block_kernels.cuh",
-                                                        "tc05.cuh", "block_tc05_kernels.cuh"),
-                  "k_grad_sweep_fac<false>": ("common.cuh", "kahan.cuh", "grad_kernels.cuh"),
+                                                   "kahan.cuh", "strip_kernels.cuh", "tc05.cuh",
+                                                   "block_tc05_kernels.cuh"),
+                  "k_taylor_pass_tc05<true,true>": ("common.cuh", "stream_kernels.cuh", "block_kernels.cuh",
+                                                    "tc05.cuh", "block_tc05_kernels.cuh",
+                                                    "taylor_block_kernels.cuh", "taylor_tc05_kernels.cuh"),
+                  "k_grad_strip<false>": ("common.cuh", "kahan.cuh", "strip_kernels.cuh", "grad_kernels.cuh"),
                   "k_stream_taylor<true,true>": ("common.cuh", "stream_kernels.cuh", "als_kernels.cuh",
                                                  "taylor_kernels.cuh"),
                   "k_integrate": ("rts_integrate.cu",)}
@@ -361,7 +363,8 @@ def main():
         flops = 2 * K * cad.n_vis * FLOPS_PER_UPDATE * args.steps        # every source subtracted and averaged once
         achieved = flops / (ms_bp / 1e3) / 1e12
         sm_mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
-        name = {1: "k_block_pass<64,SUB,ACC> (FP32 FMA)", 2: "k_block_pass_tc<SUB,ACC> (TF32 mma.sync)",
+        name = {1: ("k_block_pass_strip<QH,SUB,ACC> (FP32 FMA)" if cad.n_chan <= 256 else
+                    "k_block_pass<64,SUB,ACC> (FP32 FMA)"), 2: "k_block_pass_tc<SUB,ACC> (TF32 mma.sync)",
                 3: "k_block_pass_tc05<SUB,ACC> (tcgen05.mma kind::tf32, TMEM accumulators)"}[block_kernel]
         if block_kernel == 1:
             peak = fp32_peak_tflops(sm_mhz)
@@ -377,7 +380,7 @@ def main():
                            "(of measured)")
         roofline = {"bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak,
-                    "traffic": (ncu_traffic("k_block_pass<64,true,true>") if block_kernel == 1 else
+                    "traffic": (ncu_traffic("k_block_pass<64,true,true>") if block_kernel == 1 and cad.n_chan > 256 else
                                 ncu_traffic("k_block_pass_tc05<true,true>") if block_kernel == 3 else None),
                     "kernel": name + ": subtract 64 solved sources + average the next 64",
                     "algorithmic_flops_per_update": FLOPS_PER_UPDATE,
@@ -807,9 +810,9 @@ def extra_legs(args, p, cad, d_vis, d_resid, src, rank, mixed_rate, sm_mhz):
         "sweeps_60": {"ms": a60.elapsed_time(b60), "not_converged": int(np.sum(st_60 == 1)),
                       "last_relative_change_median": float(np.median(rel_60)),
                       "last_relative_change_max": float(np.max(rel_60))},
-        "roofline": {"bound": "tensor", "kernel": "k_block_pass_tc05<SUB,ACC,TAY> (tcgen05.mma kind::tf32)",
+        "roofline": {"bound": "tensor", "kernel": "k_taylor_pass_tc05<SUB,ACC> (tcgen05.mma kind::tf32)",
                      "achieved": tay_tflops, "peak": tf32_peak, "unit": "TFLOP/s", "frac": tay_tflops / tf32_peak,
-                     "traffic": ncu_traffic("k_block_pass_tc05<true,true,true>"),
+                     "traffic": ncu_traffic("k_taylor_pass_tc05<true,true>"),
                      "algorithmic_flops_per_update": 3 * FLOPS_PER_UPDATE,
                      "algorithmic_bytes_per_launch": cad.n_vis * BYTES_PER_UPDATE,
                      "avg_launch_ms": ms_bp / n_bp,
@@ -903,10 +906,10 @@ def extra_legs(args, p, cad, d_vis, d_resid, src, rank, mixed_rate, sm_mhz):
     out["adjoint"] = {
         "workload": "512 ant x 768 ch x 8 t, 300 sources, positions perturbed N(0, 1 arcmin^2); loss + dL/d(J,l,m,S)",
         "ms_per_step": ms_adj, "loss": float(loss.item()),
-        "roofline": {"bound": "alu", "kernel": "k_grad_sweep_fac<false> (factorised phasor tables; + reductions, in the step time)",
+        "roofline": {"bound": "alu", "kernel": "k_grad_strip<false> (strips in registers, factorised phasor tables; + reductions, in the step time)",
                      "achieved": adj_tflops, "peak": adj_peak, "unit": "TFLOP/s", "frac": adj_tflops / adj_peak,
                      "algorithmic_flops_per_update": ADJ_FLOPS_PER_UPDATE,
-                     "traffic": ncu_traffic("k_grad_sweep_fac<false>"),
+                     "traffic": ncu_traffic("k_grad_strip<false>"),
                      "algorithmic_bytes_per_launch": c5.n_vis * 32 + c5.n_src * c5.n_bl * (64 + 24)},
         "fp64_ms_per_step_at_300_sources_extrapolated": per_upd_64 * c5.n_src * c5.n_vis,
         "fp64_sources_timed": k_adj64, "speedup_mixed_vs_fp64": per_upd_64 / per_upd_mixed,
