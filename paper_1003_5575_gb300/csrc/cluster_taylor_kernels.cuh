@@ -307,7 +307,6 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_taylor(ClusterTaylorA
   const uint32_t my_row = tc05::smem_u32(Xb) + (uint32_t)((lane & 1) * n + p) * 16u;
   const uint32_t dst_row = sends ? cluster_map(my_row, dst_rank) : 0u;
   const uint32_t dst_bar = sends ? cluster_map(tc05::smem_u32(&s_bar[0]), dst_rank) : 0u;
-  const float mu2 = (float)a.mu2, mu4 = (float)a.mu4;
   const FF fS = ff_of(a.S), fmu0S = ff_of(a.mu0 * a.S), fmu2S = ff_of(a.mu2 * a.S), fmu4S = ff_of(a.mu4 * a.S);
   const FF c4 = ff_of(2.0 * a.S * a.S * a.mu4), c2 = ff_of(2.0 * a.S);
   // lanes 0 .. 7: entry e of X_p = [G H] (row er, column ec of 4), the rotated iterate
