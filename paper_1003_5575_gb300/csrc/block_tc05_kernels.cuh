@@ -51,13 +51,14 @@
 // arrival.  Every wait is bounded (a wait that runs out sets *err and stops the
 // pass, which the status read reports, after the copies in flight have been
 // waited for and TMEM is freed).
-// Bound by the CUDA cores' phases (issue 60 % of the slots, shared-memory pipe 52 %,
-// ALU pipe 37 %, tensor pipe 28 %; without any MMA a step takes 5 % less).  A step of both
-// roles at 768 channels, 64 sources: about 7 300 cycles (the 2 x 2 form with five barriers
+// Bound by the CUDA cores' phases (issue 62 % of the slots, shared-memory pipe 57 %,
+// ALU pipe 40 %, tensor pipe 31 %; without any MMA a step takes 5 % less).  A step of both
+// roles at 768 channels, 64 sources: about 7 200 cycles (the 2 x 2 form with five barriers
 // a step: 9 700); a cadence of 512 antennas x 768 channels x 8 times x 1000 sources went
-// from 722 to 587 ms, its passes from 559 to about 430.  Steps on the way: real parts and
-// one barrier 496 ms of passes, constant offsets, polled waits and loads before stores 472,
-// A_a before the barrier 430.  Phasors by polynomials instead of the sine table: no gain.
+// from 722 to 582 ms, its passes from 559 to 418 (24.6 ms each).  Steps on the way: real
+// parts and one barrier 496 ms of passes, constant offsets, polled waits and loads before
+// stores 472, A_a before the barrier 418.  Phasors by polynomials instead of the sine
+// table: no gain.
 // Limits: at most 64 sources per role, n_chan <= kTc5MaxChan.
 #pragma once
 #include "block_kernels.cuh"

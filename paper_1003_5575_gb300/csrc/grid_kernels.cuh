@@ -30,7 +30,7 @@
 // Measured (512 antennas, 1125^2 pixels, radius 12, 4 values): 591 us before the
 // warps of a tile shared its list, values were fetched 32 together, the two
 // pixels of a lane became packed operands and the sort's warps were more than 128;
-// 233 us now.  The gather is bound by instruction issue (68 % of the slots),
+// 233 us now.  The gather is bound by instruction issue and latency (189 us, 61 % of the slots, ALU 42 %),
 // the sort by the latency of its five short launches.
 #pragma once
 #include <cuda_runtime.h>

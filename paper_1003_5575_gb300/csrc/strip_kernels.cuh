@@ -257,8 +257,8 @@ template <int QH> size_t strip_pass_smem(const StripGrid& g, int n_time) {
 // The pass of the blocked peel (see block_kernels.cuh) on strips of at most 32 QH
 // channels.  Bound by instruction issue and the FP32 pipe together: (20 + 17)
 // multiply-adds per source and channel of both roles, two a packed instruction, and
-// 41 instructions a phasor of the tables; 58 % of the FP32 pipe, 55 % of the issue
-// slots and 72 % of the shared-memory pipe measured (128 channels).  Two CTAs an SM
+// 41 instructions a phasor of the tables; 59 % of the FP32 pipe, 56 % of the issue
+// slots and 65 % of the shared-memory pipe measured (128 channels).  Two CTAs an SM
 // (<= 128 registers a thread): the loads and tables of one warp hide behind the
 // multiply-adds of others.  Against the kernel it replaces on short strips
 // (k_block_pass, FP32, one CTA a baseline): 3.9 / 4.2 / 4.6 / 5.9 / 6.2 ms.
