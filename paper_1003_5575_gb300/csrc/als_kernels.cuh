@@ -15,7 +15,8 @@
 // memory), and the 2x2 solve is FP64.  The FP64 path does all of it in FP64: an FP64
 // instruction occupies its sub-partition for 64 cycles, so a thread skips the terms past
 // the last antenna (at 128 antennas three of every four) and adds by fused
-// multiply-adds: 16.5 us a sweep before, 8 now.
+// multiply-adds (16.5 us a sweep before, 8 after), and a sweep starts while the one
+// before it ends (5.6).
 #pragma once
 #include "common.cuh"
 
@@ -85,6 +86,14 @@ __device__ __forceinline__ float warp_reduce_scatter16f(float (&v)[16], int lane
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
+// Launches of a source's sweeps after the first are programmatic dependents: a sweep's
+// CTAs start and fetch their averages while the sweep before it ends, and wait for it
+// here before they touch an iterate.  (In any other launch both are no-ops.)
+__device__ __forceinline__ void als_previous_sweep_done() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <typename T>   // T = float (mixed) or double (FP64)
 __global__ void __launch_bounds__(kAlsThreads) k_als_sweep(AlsArgs a) {
   using C = typename cplx_of<T>::type;
@@ -106,6 +115,16 @@ __global__ void __launch_bounds__(kAlsThreads) k_als_sweep(AlsArgs a) {
       const int q = q0 + u * kAlsThreads;
       if (q < a.n_ant && q != p) {
         load_vpq<C>(avg, a.n_ant, p, q, V[u]);
+      } else {
+        #pragma unroll
+        for (int e = 0; e < 4; ++e) V[u][e] = cmk<C>(0, 0);
+      }
+    }
+    if (q0 == threadIdx.x) als_previous_sweep_done();
+    #pragma unroll
+    for (int u = 0; u < kAlsPerThread; ++u) {
+      const int q = q0 + u * kAlsThreads;
+      if (q < a.n_ant && q != p) {
         if (a.first) {
           J[u][0] = cmk<C>(1, 0); J[u][1] = cmk<C>(0, 0); J[u][2] = cmk<C>(0, 0); J[u][3] = cmk<C>(1, 0);
         } else if constexpr (sizeof(T) == 4) {
@@ -117,7 +136,7 @@ __global__ void __launch_bounds__(kAlsThreads) k_als_sweep(AlsArgs a) {
         }
       } else {
         #pragma unroll
-        for (int e = 0; e < 4; ++e) { V[u][e] = cmk<C>(0, 0); J[u][e] = cmk<C>(0, 0); }
+        for (int e = 0; e < 4; ++e) J[u][e] = cmk<C>(0, 0);
       }
     }
     #pragma unroll
@@ -145,6 +164,7 @@ __global__ void __launch_bounds__(kAlsThreads) k_als_sweep(AlsArgs a) {
       }
     }
   }
+  if (threadIdx.x >= a.n_ant) als_previous_sweep_done();         // threads without a term
   double v[16];
   #pragma unroll
   for (int k = 0; k < 8; ++k) v[k] = (double)A[k];

@@ -338,8 +338,18 @@ int launch_als(rts_peel_t* h, const void* avg, double S, void* jones_out, int sl
     a.norms = h->d_norms; a.flag = h->d_flag;
     a.jones_out = it == h->n_iter ? jones_out : nullptr;
     a.n_ant = h->n_ant; a.S = S; a.first = it == 1; a.average = (it % 2) == 0;
-    if (h->precision == RTS_PREC_MIXED) k_als_sweep<float><<<als_grid(h->n_ant), kAlsThreads, 0, s>>>(a);
-    else k_als_sweep<double><<<als_grid(h->n_ant), kAlsThreads, 0, s>>>(a);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = it > 1;      // the first waits for the averages
+    cudaLaunchConfig_t c;
+    std::memset(&c, 0, sizeof(c));
+    c.gridDim = dim3(als_grid(h->n_ant));
+    c.blockDim = dim3(kAlsThreads);
+    c.stream = s;
+    c.attrs = &attr;
+    c.numAttrs = 1;
+    if (h->precision == RTS_PREC_MIXED) RTS_CUDA(h, cudaLaunchKernelEx(&c, k_als_sweep<float>, a));
+    else RTS_CUDA(h, cudaLaunchKernelEx(&c, k_als_sweep<double>, a));
   }
   k_als_finalize<<<1, 256, 0, s>>>(h->d_norms, h->n_ant, h->d_flag, h->d_status + slot, h->d_rel + slot);
   span.end(h->n_iter + 1);

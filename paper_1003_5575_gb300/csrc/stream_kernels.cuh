@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kStreamThreads, 3) k_stream_mixed(StreamArgs a
 // and, because tau_ij = tau_i - tau_j, each table of a baseline is the product
 // T_i conj(T_j) of its antennas' tables, which k_fp64_ant_tables forms once per
 // source ([n_time][n_ant][Q + R]).  At 128 antennas x 128 channels x 8 times x 50
-// sources the whole cadence, solves included, went from 111 ms to 36.4.  Other
+// sources the whole cadence, solves included, went from 111 ms to 33.8.  Other
 // frequency lists (uniform to 1e-9 only) keep one sincospi per sample and role
 // (k_stream_fp64).
 
