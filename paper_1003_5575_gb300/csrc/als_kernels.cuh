@@ -90,8 +90,8 @@ __device__ __forceinline__ float warp_reduce_scatter16f(float (&v)[16], int lane
 // CTAs start and fetch their averages while the sweep before it ends, and wait for it
 // here before they touch an iterate.  (In any other launch both are no-ops.)
 __device__ __forceinline__ void als_previous_sweep_done() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_previous_done();
+  grid_next_may_start();
 }
 
 template <typename T>   // T = float (mixed) or double (FP64)

@@ -196,13 +196,18 @@ __global__ void __launch_bounds__(128) k_cluster_prep(const float2* __restrict__
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t bl = idx >> 2;
   const int g0 = 2 * (int)(idx & 3);
-  if (bl >= n_bl || g0 >= n_grp) return;
+  if (bl >= n_bl || g0 >= n_grp) {
+    grid_next_may_start();
+    return;
+  }
   const bool two = g0 + 1 < n_grp;
   const int ka = q0 + g0, kb = two ? ka + 1 : ka;
   const float2* Da = Dtab + dir_index(n_bl, bl, 0, ka);
   const float2* Db = Dtab + dir_index(n_bl, bl, 0, kb);
   const float4* M4 = reinterpret_cast<const float4*>(Mblk) + 2 * bl;
   const int2 ij = bl_ant[bl];
+  grid_previous_done();                      // the group before it has written its models
+  grid_next_may_start();
   const int64_t up = (int64_t)ij.x * n_ant + ij.y, lo = (int64_t)ij.y * n_ant + ij.x, nn = (int64_t)n_ant * n_ant;
   float2 va[4], vb[4];
   #pragma unroll
@@ -322,6 +327,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_solve(ClusterSolveArg
   if (tid < a.n_grp) s_S[tid] = (float)a.src[3 * (a.s0 + a.q0 + tid) + 2];
   __syncthreads();
   cluster_sync();                          // every CTA's barriers exist before any store to them
+  grid_previous_done();                    // V and D are written
   volatile int* bad = &s_bad;
   // this lane's destination: row (lane & 1) of the warp's antenna in CTA lane >> 1
   const uint32_t dst_rank = (uint32_t)(lane >> 1);
@@ -482,6 +488,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_solve(ClusterSolveArg
   // ---- every CTA's norms are written and no store is in flight past this barrier;
   // warp 0 of CTA q % CS takes source q's status, the others form the group's
   // model matrices from the rows p < q of their antennas
+  grid_next_may_start();
   if (*bad) __nanosleep(100000);
   cluster_sync();
   if (warp == 0)

@@ -66,6 +66,11 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
   return make_float2(__uint_as_float((unsigned)rd), __uint_as_float((unsigned)(rd >> 32)));
 }
 
+// programmatic dependent launches: wait until the launch before this one has ended and
+// its writes are visible; let the next one start (no-ops in other launches)
+__device__ __forceinline__ void grid_previous_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---- 2x2 complex matrices [0 1; 2 3] -------------------------------------------
 template <typename C> struct M22 { C e[4]; };
 
