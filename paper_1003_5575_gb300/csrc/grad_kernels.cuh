@@ -699,6 +699,14 @@ inline int grad_prepare(GradWorkspace& w, bool mixed, int n_src, const double* s
   cudaError_t e;
   if (!w.loss_bl) {
     w.cap_src = max_src; w.n_bl = n_bl;
+    // the most any call may take, once a handle (every handle sets the same)
+    auto room = [&](auto kernel) {
+      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradMaxSmem - 1024) != cudaSuccess;
+    };
+    if (mixed && (room(k_grad_strip<false, kGsPairWarps, true>) || room(k_grad_strip<false, kGsPairWarps, false>) ||
+                  room(k_grad_strip<false, kGsMaxWarps, true>) || room(k_grad_strip<true, kGsPairWarps, true>) ||
+                  room(k_grad_strip<true, kGsPairWarps, false>) || room(k_grad_strip<true, kGsMaxWarps, true>)))
+      return grad_fail(err, cudaGetLastError(), "cudaFuncSetAttribute");
     if ((e = cudaMalloc(&w.G, (size_t)max_src * n_bl * 4 * sizeof(double2))) != cudaSuccess ||
         (e = cudaMalloc(&w.gsc, (size_t)max_src * n_bl * 3 * sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&w.loss_bl, (size_t)n_bl * sizeof(double))) != cudaSuccess ||
@@ -751,9 +759,8 @@ inline int grad_sweep(GradWorkspace& w, bool mixed, const void* vis, int n_src, 
       if (n_src > 0)
         k_grad_ant_phases<<<1024, 256, 0, s>>>(w.dir, n_src, grad_kp(n_src), uvw, n_ant, n_time, nu0_c, dnu_c, w.aph);
       auto launch = [&](auto kernel) -> cudaError_t {
-        cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradMaxSmem - 1024);
-        if (r == cudaSuccess) kernel<<<(unsigned)n_bl, 32 * warps, smem, s>>>(a, w.aph, w.lmn);
-        return r;
+        kernel<<<(unsigned)n_bl, 32 * warps, smem, s>>>(a, w.aph, w.lmn);
+        return cudaSuccess;
       };
       if (!pair) e = wchan ? launch(k_grad_strip<true, kGsMaxWarps, true>) : launch(k_grad_strip<false, kGsMaxWarps, true>);
       else if (tot) e = wchan ? launch(k_grad_strip<true, kGsPairWarps, true>) : launch(k_grad_strip<false, kGsPairWarps, true>);
