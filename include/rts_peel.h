@@ -288,8 +288,8 @@ int rts_peel_rel(rts_peel_t* h, int32_t n_src, double* h_rel, void* stream);
  * integer arithmetic).  form = 0 returns that Q0.64 phase (the streaming,
  * predict and adjoint kernels); form = 1 the FP32 value the kernels hand to the
  * hardware sin/cos (rounded to Q0.32 first); form = 2 the Q0.64 phase as the
- * blocked schedule forms it, from the two antennas' delays
- * tau_i = u_i l + v_i m + w_i (n - 1) (the same geometry: uvw_ij = uvw_i - uvw_j)
+ * blocked schedule forms it, from the two antennas' delays about antenna 0
+ * (u, v, w of uvw_i - uvw_0; the same geometry: uvw_ij = uvw_i - uvw_j)
  * as the difference of their Q0.64 phases modulo one turn.  A pair with t or
  * bl out of range gets NaN.  Asynchronous on `stream`.  RTS_EINVAL for a NULL
  * handle or pointer, n_pair < 0, form not 0, 1 or 2, or a direction with

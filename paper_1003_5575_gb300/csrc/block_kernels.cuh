@@ -235,8 +235,9 @@ __device__ inline unsigned long long pair_mid_phase(unsigned long long dA, long 
 // geometry of one block (no visibility data): Q0.64 phases of its sources,
 //   ph[bl][t][k] = (frac(tau nu_0 / c), frac(tau dnu / c)).
 // The array's baselines are antenna pairs with (u, v, w)_ij = uvw_i - uvw_j, so
-// tau_ij = tau_i - tau_j with the antenna delay tau_i = u_i l + v_i m + w_i (n - 1),
-// and the Q0.64 phases of a baseline are the differences of its antennas'
+// tau_ij = tau_i - tau_j with the antenna delay tau_i = u l + v m + w (n - 1) of
+// uvw_i - uvw_0 (about antenna 0: the coordinates' own origin means nothing and may
+// be far away), and the Q0.64 phases of a baseline are the differences of its antennas'
 // phases modulo one turn (2^64: exact integer arithmetic).  The FP64 work is
 // per (time, antenna, source) instead of per (time, baseline, source); the
 // result differs from the per-baseline FP64 evaluation by the rounding of the
@@ -254,11 +255,13 @@ __global__ void __launch_bounds__(256) k_block_ant_phases(const double* __restri
     PhaseAB p;
     p.a = 0; p.b = 0;
     if (k < n_blk) {
-      const double l = src[3 * k], m = src[3 * k + 1];
-      const double r2 = l * l + m * m;
-      const double nm1 = -r2 / (1.0 + sqrt(1.0 - r2));
-      const double* x = uvw + ti * 3;
-      const double tau = x[0] * l + x[1] * m + x[2] * nm1;
+      SrcDir d;
+      d.l = src[3 * k];
+      d.m = src[3 * k + 1];
+      const double r2 = d.l * d.l + d.m * d.m;
+      d.nm1 = -r2 / (1.0 + sqrt(1.0 - r2));
+      const int t = (int)(ti / n_ant);
+      const double tau = delay_m(uvw, n_ant, t, (int)(ti - (int64_t)t * n_ant), 0, d);
       p.a = frac_q64(tau * nu0_c);
       p.b = frac_q64(tau * dnu_c);
     }

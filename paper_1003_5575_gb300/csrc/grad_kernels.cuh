@@ -325,7 +325,7 @@ inline int grad_strip_warps(int n_src, int n_chan, int n_time, int most, size_t 
   return w >= least ? w : 0;
 }
 
-// the antennas' Q0.64 phases of every source, [n_time][n_ant][kp]
+// the antennas' Q0.64 phases of every source (of u_i - u_0: see k_block_ant_phases), [n_time][n_ant][kp]
 __global__ void __launch_bounds__(256) k_grad_ant_phases(const DirQ* __restrict__ dir, int n_src, int kp,
                                                         const double* __restrict__ uvw, int n_ant, int n_time,
                                                         double nu0_c, double dnu_c, PhaseAB* __restrict__ aph) {
@@ -336,9 +336,10 @@ __global__ void __launch_bounds__(256) k_grad_ant_phases(const DirQ* __restrict_
     PhaseAB p;
     p.a = 0; p.b = 0;
     if (k < n_src) {
-      const DirQ d = dir[k];
-      const double* u = uvw + ti * 3;
-      const double tau = u[0] * d.x + u[1] * d.y + u[2] * d.z;
+      SrcDir d;
+      d.l = dir[k].x; d.m = dir[k].y; d.nm1 = dir[k].z;
+      const int t = (int)(ti / n_ant);
+      const double tau = delay_m(uvw, n_ant, t, (int)(ti - (int64_t)t * n_ant), 0, d);
       p.a = frac_q64(tau * nu0_c);
       p.b = frac_q64(tau * dnu_c);
     }

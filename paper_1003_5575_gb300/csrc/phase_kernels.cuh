@@ -13,8 +13,8 @@ namespace rts {
 // FP64 delay (the streaming, predict and adjoint kernels); form 1, that phase
 // as the FP32 value the kernels pass to the hardware sin/cos (rounded to Q0.32,
 // then converted); form 2, the Q0.64 phase as the blocked schedule forms it,
-// the difference of the two antennas' Q0.64 phases (their FP64 delays
-// tau_i = u_i l + v_i m + w_i (n - 1)).  Pairs whose time or baseline index is
+// the difference of the two antennas' Q0.64 phases (their FP64 delays about
+// antenna 0, from uvw_i - uvw_0).  Pairs whose time or baseline index is
 // out of range get NaN in every channel.
 __global__ void __launch_bounds__(256) k_phase_table(const double* __restrict__ uvw, const int2* __restrict__ bl_ant,
                                                      int n_ant, int n_chan, int n_time, int64_t n_bl, SrcDir d,
@@ -33,9 +33,7 @@ __global__ void __launch_bounds__(256) k_phase_table(const double* __restrict__ 
     const int2 ij = bl_ant[bl];
     unsigned long long A, B;
     if (form == 2) {
-      const double* ui = uvw + ((size_t)t * n_ant + ij.x) * 3;
-      const double* uj = uvw + ((size_t)t * n_ant + ij.y) * 3;
-      const double ti = ui[0] * d.l + ui[1] * d.m + ui[2] * d.nm1, tj = uj[0] * d.l + uj[1] * d.m + uj[2] * d.nm1;
+      const double ti = delay_m(uvw, n_ant, t, ij.x, 0, d), tj = delay_m(uvw, n_ant, t, ij.y, 0, d);
       A = frac_q64(ti * nu0_c) - frac_q64(tj * nu0_c);
       B = frac_q64(ti * dnu_c) - frac_q64(tj * dnu_c);
     } else {

@@ -242,8 +242,10 @@ int launch_stream(rts_peel_t* h, bool sub, bool acc, bool in_peel, const StreamA
     tb.sub = h->d_tab64[h->tab64_at];
     if (acc) {
       h->tab64_at ^= 1;
-      k_fp64_ant_tables<<<2 * (unsigned)h->n_sm, 256, 0, s>>>(h->d_uvw, a.acc, h->n_ant, h->n_time, tb.Q, tb.R,
-                                                             a.nu0_c, a.dnu_c, h->d_tab64[h->tab64_at]);
+      const Fp64Freq f = {a.nu0_c, -std::fma(a.nu0_c, kCLight, -h->nu0) / kCLight,
+                          a.dnu_c, -std::fma(a.dnu_c, kCLight, -h->dnu) / kCLight};
+      k_fp64_ant_tables<<<2 * (unsigned)h->n_sm, 256, 0, s>>>(h->d_uvw, a.acc, h->n_ant, h->n_time, tb.Q, tb.R, f,
+                                                             h->d_tab64[h->tab64_at]);
     }
     tb.acc = h->d_tab64[h->tab64_at];
     const size_t smem = tb.n_t * per_t;

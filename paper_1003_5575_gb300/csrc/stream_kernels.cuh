@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kStreamThreads, 3) k_stream_mixed(StreamArgs a
 // and, because tau_ij = tau_i - tau_j, each table of a baseline is the product
 // T_i conj(T_j) of its antennas' tables, which k_fp64_ant_tables forms once per
 // source ([n_time][n_ant][Q + R]).  At 128 antennas x 128 channels x 8 times x 50
-// sources the whole cadence, solves included, went from 111 ms to 33.8.  Other
+// sources the whole cadence, solves included, went from 111 ms to 34.1.  Other
 // frequency lists (uniform to 1e-9 only) keep one sincospi per sample and role
 // (k_stream_fp64).
 
@@ -210,18 +210,46 @@ __host__ inline int fp64_table_r(int n_chan) {
   return r;
 }
 
-// [n_time][n_ant][Q + R]: T1 then T2 of one source direction
+// [n_time][n_ant][Q + R]: T1 then T2 of one source direction.  The delays are those of
+// u_i - u_0: only differences of coordinates mean anything, so their origin may be far
+// from the array, and from a geocentric one (6.4e6 m) the phases of u_i itself are off by
+// up to 8.6e-10 radian.  Differences, delay, frequency and their product are pairs of
+// doubles: an antenna's error is common to all of its baselines and so goes whole into
+// its gains, where a baseline's own rounding averages out.  *_lo: what nu0 / c and
+// dnu / c leave after their rounding.
+struct Fp64Freq { double nu0, nu0_lo, dnu, dnu_lo; };
 __global__ void __launch_bounds__(256) k_fp64_ant_tables(const double* __restrict__ uvw, SrcDir d, int n_ant,
-                                                        int n_time, int Q, int R, double nu0_c, double dnu_c,
+                                                        int n_time, int Q, int R, Fp64Freq f,
                                                         double2* __restrict__ tab) {
   const int n_e = Q + R;
   const int64_t n = (int64_t)n_time * n_ant * n_e;
+  // hi + lo = a + b
+  auto two_sum = [](double a, double b, double& lo) {
+    const double s = a + b, bb = s - a;
+    lo += (a - (s - bb)) + (b - bb);
+    return s;
+  };
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
     const int64_t ta = x / n_e;
     const int e = (int)(x - ta * n_e);
-    const double* u = uvw + ta * 3;
-    const double tau = u[0] * d.l + u[1] * d.m + u[2] * d.nm1;
-    tab[x] = phasor_d(tau * (e < Q ? nu0_c + (double)(R * e) * dnu_c : (double)(e - Q) * dnu_c));
+    const double *u = uvw + ta * 3, *u0 = uvw + ta / n_ant * n_ant * 3;
+    double tl = 0.0, th = 0.0;
+    const double dir[3] = {d.l, d.m, d.nm1};
+    #pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      double dl = 0.0;
+      const double dh = two_sum(u[i], -u0[i], dl), p = __dmul_rn(dh, dir[i]);
+      tl += fma(dh, dir[i], -p) + dl * dir[i];
+      th = two_sum(th, p, tl);
+    }
+    const double k = (double)(e < Q ? R * e : e - Q), s = __dmul_rn(k, f.dnu);
+    double fl = fma(k, f.dnu, -s) + k * f.dnu_lo, fh = s;
+    if (e < Q) {
+      fl += f.nu0_lo;
+      fh = two_sum(f.nu0, s, fl);
+    }
+    const double p = __dmul_rn(th, fh);
+    tab[x] = phasor_d((p - rint(p)) + (fma(th, fh, -p) + fma(th, fl, tl * fh)));
   }
 }
 
