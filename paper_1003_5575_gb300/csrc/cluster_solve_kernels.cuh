@@ -29,7 +29,10 @@
 //     it has received every matrix of sweep g, which every CTA sends after its
 //     last read of the buffer that sweep g + 1 overwrites, and after its wait for
 //     sweep g - 1, so no store can reach a buffer still read or a barrier phase
-//     still open.
+//     still open.  That holds for warps that send; a warp whose slot has no antenna
+//     sends nothing, so nobody would wait for it and the phase it waits for could be two
+//     behind: it reads no iterate and waits for none of the sweeps' barriers (it meets the
+//     others at the last sweep's CTA barriers and at the cluster barrier).
 //   last sweep: the lane partials added in float-float arithmetic (about 47
 //     bits; an FP64 tree cost 5 us a source here), the 2x2 solve, the averaging
 //     and the relative change in FP64 against the FP32 previous iterate.
@@ -481,7 +484,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_solve(ClusterSolveArg
         const uint32_t off = last ? (uint32_t)(4 + 2 * q) * (uint32_t)n_ant * 16u : b * (uint32_t)n_ant * 32u;
         cluster_send16(dst_row + off, Jn, dst_bar + 8u * b);
       }
-      cluster_wait(&s_bar[b], (g >> 1) & 1u, bad);
+      if (live) cluster_wait(&s_bar[b], (g >> 1) & 1u, bad);
     }
   }
 
