@@ -192,10 +192,13 @@ __device__ __forceinline__ FF warp_reduce_scatter12ff(const FF (&v)[12], int lan
 // antenna matrices.  Four threads a baseline, two targets each: M_j is read once
 // for both, and the four threads' reads of it meet in the same 32 bytes.  Bound
 // by L2 (M_j and D_jk once each, the matrices' stores).
+// It is resident while the launch before it writes M, so M is read from L2 and through
+// no pointer that promises read-only data (D_jk, the averages and the antenna pairs
+// are older than both launches).
 __global__ void __launch_bounds__(128) k_cluster_prep(const float2* __restrict__ Ablk, int q0, int n_grp,
-                                                     const float2* __restrict__ Mblk, const float2* __restrict__ Dtab,
+                                                     const float2* Mblk, const float2* __restrict__ Dtab,
                                                      const int2* __restrict__ bl_ant, int n_ant, int64_t n_bl,
-                                                     float4* __restrict__ V, float2* __restrict__ D) {
+                                                     float4* V, float2* D) {
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t bl = idx >> 2;
   const int g0 = 2 * (int)(idx & 3);
@@ -222,7 +225,7 @@ __global__ void __launch_bounds__(128) k_cluster_prep(const float2* __restrict__
   };
   #pragma unroll 8
   for (int j = 0; j < q0; ++j) {
-    const float4 m0 = __ldg(M4 + (size_t)j * n_bl * 2), m1 = __ldg(M4 + (size_t)j * n_bl * 2 + 1);
+    const float4 m0 = __ldcg(M4 + (size_t)j * n_bl * 2), m1 = __ldcg(M4 + (size_t)j * n_bl * 2 + 1);
     const float2 m[4] = {make_float2(m0.x, m0.y), make_float2(m0.z, m0.w), make_float2(m1.x, m1.y),
                          make_float2(m1.z, m1.w)};
     const float2 da = __ldg(Da + j), db = __ldg(Db + j);

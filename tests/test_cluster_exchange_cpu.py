@@ -61,3 +61,10 @@ def test_no_wait_of_the_kernel_can_be_overtaken():
     body = open(SRC).read().split("k_cluster_solve(ClusterSolveArgs a)")[1].split("struct ClusterAlsArgs")[0]
     guards = re.findall(r"(if \(live\) )?cluster_wait\(", body)
     assert guards and lost_waits(WARPS, 5, idle_waits=not all(guards)) == set()
+
+
+def test_models_written_beside_the_prep_launch_are_not_read_as_constants():
+    """k_cluster_prep is resident while the launch before it writes the model matrices:
+    neither a read-only pointer nor the non-coherent load may be used for them."""
+    body = open(SRC).read().split("k_cluster_prep(")[1].split("\n}\n")[0]
+    assert re.search(r"const float2\* Mblk,", body) and not re.search(r"__ldg\(M4", body)
