@@ -18,10 +18,12 @@
 // A CTA owns the antennas p = rank + slot CS.  Per source q of the group:
 //   rows: V_pq of its antennas in shared memory, with the terms
 //     S_j D_jq J_p J_q^H of the group's solved sources j < q taken out.
-//   sweeps: W warps a slot, each lane the partners lane + 32 w (+ 32 W u);
-//     lane partials and a warp's shuffle tree in FP32, the slot's warps added
-//     exactly (two-sums) and rounded once, as their FP64 sum would be.  The slot's first
-//     warp solves the 2x2 system (each lane the row it sends) and lane (rank,
+//   sweeps: one warp a slot, each lane the partners lane + 32 u, up to kClChain terms
+//     added in FP32 one after another; of the warp's shuffle tree the first level in
+//     FP32, the others float-float, the total rounded once.  (k_block_solve: trees of 32
+//     FP32 terms, their totals in FP64, rounded once; in units of a term's rounding
+//     157 there and 146 here at 128 antennas, 287 and 282 at 256.)  The warp solves the
+//     2x2 system (each lane the row it sends) and lane (rank,
 //     row) stores one 16-byte row of J_p into CTA `rank` with st.async, which
 //     completes 16 bytes of that CTA's mbarrier transaction count; a CTA starts
 //     the next sweep when all n_ant matrices have arrived.  Iterates alternate
@@ -33,13 +35,16 @@
 //     sends nothing, so nobody would wait for it and the phase it waits for could be two
 //     behind: it reads no iterate and waits for none of the sweeps' barriers (it meets the
 //     others at the last sweep's CTA barriers and at the cluster barrier).
-//   last sweep: the lane partials added in float-float arithmetic (about 47
+//   last sweep: a partner's terms in FP32, everything after that in float-float (about 47
 //     bits; an FP64 tree cost 5 us a source here), the 2x2 solve, the averaging
 //     and the relative change in FP64 against the FP32 previous iterate.
-// Measured (GB300, 20 sweeps): 36 us a source at 128 antennas where k_block_solve
-// took 87 (its barriers alone 54), 27 against 83 at 65, 23 against 80 at 32.  At 128
-// antennas a sweep is about 2 900 cycles: 1 000 of FP32 terms, 250 of shuffles,
-// 300 of the 2x2 solve and 1 000 of the exchange.
+// Measured (GB300, 20 sweeps): 35 us a source at 128 antennas where k_block_solve
+// took 87 (its barriers alone 54), 27 against 83 at 65, 22 against 80 at 32.  At 128
+// antennas a sweep is about 2 700 cycles: 1 000 of FP32 terms, 400 of the tree,
+// 300 of the 2x2 solve and 1 000 of the exchange.  Error of the gains against 64 bits,
+// 61 sources on 65 antennas x 203 channels x 3 times / 50 on 128 x 128 x 8 (8 seeds):
+// 2.4e-7 / 1.9e-7, with k_block_solve's schedule 3.3e-7 / 2.6e-7; with the corrections
+// of a group summed in FP32 3.8e-7 / 2.7e-7.
 // Every wait is bounded (kSolveWaitNs).  A CTA whose wait ran out keeps its
 // control flow, but waits and sends no more and marks the group's statuses
 // kSolveStatusTimeout; no CTA exits before the last cluster barrier, so no store
@@ -54,6 +59,7 @@ namespace rts {
 constexpr int kClThreads = 512;            // at most (a warp per slot)
 constexpr int kClGroup = 8;                // sources per launch
 constexpr int kClMaxCta = 16;
+constexpr int kClChain = 4;                // partners whose terms a lane adds one after another
 constexpr int kClMaxSlots = 16;            // antennas per CTA, at most
 constexpr int kClSlots = 8;                // and as many where more CTAs can be had: two warps a
                                            // sub-partition; the exchange costs the same whatever the CTAs
@@ -144,7 +150,7 @@ __device__ __forceinline__ FF ff_shfl_xor(FF x, int o) {
   r.lo = __shfl_xor_sync(0xffffffffu, x.lo, o);
   return r;
 }
-// the last three levels of the sums below
+// the last four levels of the sums below
 __device__ __forceinline__ FF warp_reduce_scatter8ff(FF (&w)[8], int lane) {
   #pragma unroll
   for (int o = 8, n = 8; o >= 2; o >>= 1, n >>= 1) {
@@ -158,9 +164,41 @@ __device__ __forceinline__ FF warp_reduce_scatter8ff(FF (&w)[8], int lane) {
   return ff_add(w[0], ff_shfl_xor(w[0], 1));
 }
 
-// Reduce 16 floats over the 32 lanes of a warp with float-float sums (each level
-// exchanges half of the remaining values with the partner lane); afterwards
-// lane L holds the warp total of value index L >> 1.
+// Reduce 16 floats over the 32 lanes of a warp (each level exchanges half of the
+// remaining values with the partner lane) with the last four levels, whose sums are
+// the large ones, in float-float; afterwards lane L holds the warp total of value
+// index L >> 1, rounded once
+__device__ __forceinline__ float warp_reduce_scatter16c(float (&v)[16], int lane) {
+  {
+    const bool upper = (lane & 16) != 0;
+    #pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float send = upper ? v[i] : v[i + 8], keep = upper ? v[i + 8] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+  }
+  FF w[4];
+  {
+    const bool upper = (lane & 8) != 0;
+    #pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float send = upper ? v[i] : v[i + 4], keep = upper ? v[i + 4] : v[i];
+      w[i] = ff_two_sum(keep, __shfl_xor_sync(0xffffffffu, send, 8));
+    }
+  }
+  #pragma unroll
+  for (int o = 4, n = 4; o >= 2; o >>= 1, n >>= 1) {
+    const bool upper = (lane & o) != 0;
+    #pragma unroll
+    for (int i = 0; i < n / 2; ++i) {
+      const FF send = upper ? w[i] : w[i + n / 2], keep = upper ? w[i + n / 2] : w[i];
+      w[i] = ff_add(keep, ff_shfl_xor(send, o));
+    }
+  }
+  const FF t = ff_add(w[0], ff_shfl_xor(w[0], 1));
+  return t.hi + t.lo;
+}
+// the same of 16 floats, all levels in float-float
 __device__ __forceinline__ FF warp_reduce_scatter16ff(const float (&v)[16], int lane) {
   FF w[8];
   {
@@ -215,31 +253,53 @@ __global__ void __launch_bounds__(128) k_cluster_prep(const float2* __restrict__
   grid_previous_done();                      // the group before it has written its models
   grid_next_may_start();
   const int64_t up = (int64_t)ij.x * n_ant + ij.y, lo = (int64_t)ij.y * n_ant + ij.x, nn = (int64_t)n_ant * n_ant;
-  float2 va[4], vb[4];
-  #pragma unroll
-  for (int e = 0; e < 4; ++e) va[e] = vb[e] = make_float2(0.f, 0.f);
+  // sums of eight terms in FP32, added to A - (those before) in float-float: near the
+  // phase centre and on short baselines the terms add up to many times the difference
+  FF va[8], vb[8];
+  auto load = [&](int s, FF (&v)[8]) {
+    const float4* A = reinterpret_cast<const float4*>(Ablk + ((size_t)(q0 + s) * n_bl + bl) * 4);
+    const float4 a0 = A[0], a1 = A[1];
+    const float x[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+    #pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = FF{x[e], 0.f};
+  };
+  load(g0, va);
+  load(two ? g0 + 1 : g0, vb);
   auto cfma = [](float2 acc, float2 m, float2 d) {
     acc.x = fmaf(m.x, d.x, fmaf(-m.y, d.y, acc.x));
     acc.y = fmaf(m.x, d.y, fmaf(m.y, d.x, acc.y));
     return acc;
   };
-  #pragma unroll 8
-  for (int j = 0; j < q0; ++j) {
-    const float4 m0 = __ldcg(M4 + (size_t)j * n_bl * 2), m1 = __ldcg(M4 + (size_t)j * n_bl * 2 + 1);
-    const float2 m[4] = {make_float2(m0.x, m0.y), make_float2(m0.z, m0.w), make_float2(m1.x, m1.y),
-                         make_float2(m1.z, m1.w)};
-    const float2 da = __ldg(Da + j), db = __ldg(Db + j);
+  auto less = [](FF (&v)[8], const float2 (&t)[4]) {
     #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      va[e] = cfma(va[e], m[e], da);
-      vb[e] = cfma(vb[e], m[e], db);
+      const FF x = ff_two_sum(v[2 * e].hi, -t[e].x), y = ff_two_sum(v[2 * e + 1].hi, -t[e].y);
+      v[2 * e] = FF{x.hi, v[2 * e].lo + x.lo};
+      v[2 * e + 1] = FF{y.hi, v[2 * e + 1].lo + y.lo};
     }
+  };
+  for (int j0 = 0; j0 < q0; j0 += kClGroup) {              // q0: a multiple of kClGroup
+    float2 ta[4], tb[4];
+    #pragma unroll
+    for (int e = 0; e < 4; ++e) ta[e] = tb[e] = make_float2(0.f, 0.f);
+    #pragma unroll
+    for (int j = j0; j < j0 + kClGroup; ++j) {
+      const float4 m0 = __ldcg(M4 + (size_t)j * n_bl * 2), m1 = __ldcg(M4 + (size_t)j * n_bl * 2 + 1);
+      const float2 m[4] = {make_float2(m0.x, m0.y), make_float2(m0.z, m0.w), make_float2(m1.x, m1.y),
+                           make_float2(m1.z, m1.w)};
+      const float2 da = __ldg(Da + j), db = __ldg(Db + j);
+      #pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        ta[e] = cfma(ta[e], m[e], da);
+        tb[e] = cfma(tb[e], m[e], db);
+      }
+    }
+    less(va, ta);
+    less(vb, tb);
   }
-  auto put = [&](int s, const float2 (&v)[4], const float2* Dk) {
-    const float4* A = reinterpret_cast<const float4*>(Ablk + ((size_t)(q0 + s) * n_bl + bl) * 4);
-    float4 a0 = A[0], a1 = A[1];
-    a0 = make_float4(a0.x - v[0].x, a0.y - v[0].y, a0.z - v[1].x, a0.w - v[1].y);
-    a1 = make_float4(a1.x - v[2].x, a1.y - v[2].y, a1.z - v[3].x, a1.w - v[3].y);
+  auto put = [&](int s, const FF (&v)[8], const float2* Dk) {
+    const float4 a0 = make_float4(v[0].hi + v[0].lo, v[1].hi + v[1].lo, v[2].hi + v[2].lo, v[3].hi + v[3].lo);
+    const float4 a1 = make_float4(v[4].hi + v[4].lo, v[5].hi + v[5].lo, v[6].hi + v[6].lo, v[7].hi + v[7].lo);
     // [p][plane][q]: planes of entries (0, 1) and (2, 3); V_qp = V_pq^H below the diagonal
     float4* Vs = V + (size_t)s * 2 * nn;
     Vs[(int64_t)ij.x * 2 * n_ant + ij.y] = a0;
@@ -257,33 +317,38 @@ __global__ void __launch_bounds__(128) k_cluster_prep(const float2* __restrict__
 }
 
 // normal-equation terms of one partner: A += V J (8 reals), C += J^H J (c00,
-// c11, re c01, im c01), entries row-major, complex interleaved
+// c11, re c01, im c01), entries row-major, complex interleaved.  J is near the identity:
+// the products with its small entries first, so that a partner's own sum (v = 0) is
+// rounded once at its full size
 __device__ __forceinline__ void als_terms(float (&v)[16], const float4 v0, const float4 v1, const float4 j0,
                                           const float4 j1) {
-  v[0] = fmaf(v0.x, j0.x, v[0]); v[0] = fmaf(-v0.y, j0.y, v[0]);
-  v[0] = fmaf(v0.z, j1.x, v[0]); v[0] = fmaf(-v0.w, j1.y, v[0]);
-  v[1] = fmaf(v0.x, j0.y, v[1]); v[1] = fmaf(v0.y, j0.x, v[1]);
-  v[1] = fmaf(v0.z, j1.y, v[1]); v[1] = fmaf(v0.w, j1.x, v[1]);
-  v[2] = fmaf(v0.x, j0.z, v[2]); v[2] = fmaf(-v0.y, j0.w, v[2]);
-  v[2] = fmaf(v0.z, j1.z, v[2]); v[2] = fmaf(-v0.w, j1.w, v[2]);
-  v[3] = fmaf(v0.x, j0.w, v[3]); v[3] = fmaf(v0.y, j0.z, v[3]);
-  v[3] = fmaf(v0.z, j1.w, v[3]); v[3] = fmaf(v0.w, j1.z, v[3]);
-  v[4] = fmaf(v1.x, j0.x, v[4]); v[4] = fmaf(-v1.y, j0.y, v[4]);
-  v[4] = fmaf(v1.z, j1.x, v[4]); v[4] = fmaf(-v1.w, j1.y, v[4]);
-  v[5] = fmaf(v1.x, j0.y, v[5]); v[5] = fmaf(v1.y, j0.x, v[5]);
-  v[5] = fmaf(v1.z, j1.y, v[5]); v[5] = fmaf(v1.w, j1.x, v[5]);
-  v[6] = fmaf(v1.x, j0.z, v[6]); v[6] = fmaf(-v1.y, j0.w, v[6]);
-  v[6] = fmaf(v1.z, j1.z, v[6]); v[6] = fmaf(-v1.w, j1.w, v[6]);
-  v[7] = fmaf(v1.x, j0.w, v[7]); v[7] = fmaf(v1.y, j0.z, v[7]);
-  v[7] = fmaf(v1.z, j1.w, v[7]); v[7] = fmaf(v1.w, j1.z, v[7]);
-  v[8] = fmaf(j0.x, j0.x, v[8]); v[8] = fmaf(j0.y, j0.y, v[8]);
-  v[8] = fmaf(j1.x, j1.x, v[8]); v[8] = fmaf(j1.y, j1.y, v[8]);
-  v[9] = fmaf(j0.z, j0.z, v[9]); v[9] = fmaf(j0.w, j0.w, v[9]);
-  v[9] = fmaf(j1.z, j1.z, v[9]); v[9] = fmaf(j1.w, j1.w, v[9]);
-  v[10] = fmaf(j0.x, j0.z, v[10]); v[10] = fmaf(j0.y, j0.w, v[10]);
-  v[10] = fmaf(j1.x, j1.z, v[10]); v[10] = fmaf(j1.y, j1.w, v[10]);
-  v[11] = fmaf(j0.x, j0.w, v[11]); v[11] = fmaf(-j0.y, j0.z, v[11]);
-  v[11] = fmaf(j1.x, j1.w, v[11]); v[11] = fmaf(-j1.y, j1.z, v[11]);
+  auto row = [](float* a, float4 m, float4 j0, float4 j1) {
+    a[0] = fmaf(m.z, j1.x, a[0]); a[0] = fmaf(-m.w, j1.y, a[0]); a[0] = fmaf(-m.y, j0.y, a[0]); a[0] = fmaf(m.x, j0.x, a[0]);
+    a[1] = fmaf(m.z, j1.y, a[1]); a[1] = fmaf(m.w, j1.x, a[1]); a[1] = fmaf(m.x, j0.y, a[1]); a[1] = fmaf(m.y, j0.x, a[1]);
+    a[2] = fmaf(m.x, j0.z, a[2]); a[2] = fmaf(-m.y, j0.w, a[2]); a[2] = fmaf(-m.w, j1.w, a[2]); a[2] = fmaf(m.z, j1.z, a[2]);
+    a[3] = fmaf(m.x, j0.w, a[3]); a[3] = fmaf(m.y, j0.z, a[3]); a[3] = fmaf(m.z, j1.w, a[3]); a[3] = fmaf(m.w, j1.z, a[3]);
+  };
+  row(v, v0, j0, j1);
+  row(v + 4, v1, j0, j1);
+  v[8] = fmaf(j1.x, j1.x, v[8]); v[8] = fmaf(j1.y, j1.y, v[8]); v[8] = fmaf(j0.y, j0.y, v[8]); v[8] = fmaf(j0.x, j0.x, v[8]);
+  v[9] = fmaf(j0.z, j0.z, v[9]); v[9] = fmaf(j0.w, j0.w, v[9]); v[9] = fmaf(j1.w, j1.w, v[9]); v[9] = fmaf(j1.z, j1.z, v[9]);
+  v[10] = fmaf(j0.y, j0.w, v[10]); v[10] = fmaf(j1.y, j1.w, v[10]); v[10] = fmaf(j0.x, j0.z, v[10]); v[10] = fmaf(j1.x, j1.z, v[10]);
+  v[11] = fmaf(-j0.y, j0.z, v[11]); v[11] = fmaf(j1.x, j1.w, v[11]); v[11] = fmaf(j0.x, j0.w, v[11]); v[11] = fmaf(-j1.y, j1.z, v[11]);
+}
+
+// a partner's terms added to a lane's float-float sums
+__device__ __forceinline__ void als_terms_ff(FF (&sum)[12], const float4 v0, const float4 v1, const float4 j0,
+                                             const float4 j1) {
+  float v[16];
+  #pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = 0.f;
+  als_terms(v, v0, v1, j0, j1);
+  #pragma unroll
+  for (int i = 0; i < 12; ++i) {
+    const FF t = ff_two_sum(sum[i].hi, v[i]);
+    sum[i].hi = t.hi;
+    sum[i].lo += t.lo;
+  }
 }
 
 // one source's status and last relative change from its per-antenna norms
@@ -371,6 +436,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_solve(ClusterSolveArg
         for (int u = 0; u < 2; ++u) {
           const int qq = qb + 32 * u;
           if (qq >= n_ant) break;
+          float4 t0 = make_float4(0.f, 0.f, 0.f, 0.f), t1 = t0;
           #pragma unroll
           for (int j = 0; j < kClGroup - 1; ++j) {
             if (j < q) {
@@ -381,16 +447,18 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_solve(ClusterSolveArg
               const float2 sd = make_float2(S * d[u][j].x, S * d[u][j].y);
               const float2 w00 = cmul(sd, make_float2(i0.x, i0.y)), w01 = cmul(sd, make_float2(i0.z, i0.w));
               const float2 w10 = cmul(sd, make_float2(i1.x, i1.y)), w11 = cmul(sd, make_float2(i1.z, i1.w));
-              auto take = [](float& re, float& im, float2 w, float kx, float ky) {     // -= w conj(k)
-                re = fmaf(-w.x, kx, fmaf(-w.y, ky, re));
-                im = fmaf(-w.y, kx, fmaf(w.x, ky, im));
+              auto put = [](float& re, float& im, float2 w, float kx, float ky) {      // += w conj(k)
+                re = fmaf(w.x, kx, fmaf(w.y, ky, re));
+                im = fmaf(w.y, kx, fmaf(-w.x, ky, im));
               };
-              take(r0[u].x, r0[u].y, w00, k0.x, k0.y); take(r0[u].x, r0[u].y, w01, k0.z, k0.w);
-              take(r0[u].z, r0[u].w, w00, k1.x, k1.y); take(r0[u].z, r0[u].w, w01, k1.z, k1.w);
-              take(r1[u].x, r1[u].y, w10, k0.x, k0.y); take(r1[u].x, r1[u].y, w11, k0.z, k0.w);
-              take(r1[u].z, r1[u].w, w10, k1.x, k1.y); take(r1[u].z, r1[u].w, w11, k1.z, k1.w);
+              put(t0.x, t0.y, w00, k0.x, k0.y); put(t0.x, t0.y, w01, k0.z, k0.w);
+              put(t0.z, t0.w, w00, k1.x, k1.y); put(t0.z, t0.w, w01, k1.z, k1.w);
+              put(t1.x, t1.y, w10, k0.x, k0.y); put(t1.x, t1.y, w11, k0.z, k0.w);
+              put(t1.z, t1.w, w10, k1.x, k1.y); put(t1.z, t1.w, w11, k1.z, k1.w);
             }
           }
+          r0[u] = make_float4(r0[u].x - t0.x, r0[u].y - t0.y, r0[u].z - t0.z, r0[u].w - t0.w);
+          r1[u] = make_float4(r1[u].x - t1.x, r1[u].y - t1.y, r1[u].z - t1.z, r1[u].w - t1.w);
           const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
           row0[qq] = qq == my_p ? z : r0[u];
           row1[qq] = qq == my_p ? z : r1[u];
@@ -406,24 +474,35 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_solve(ClusterSolveArg
       const uint32_t b = g & 1u;
       const float4* Jo = Jb + (size_t)(b ^ 1u) * 2 * n_ant;       // previous iterate (not on the first sweep)
       if (tid == 0) mbar_expect(&s_bar[b], buf_bytes);
-      float v[16];
-      #pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = 0.f;
-      if (live) {
-        const float4* row0 = rows + (size_t)slot * 2 * n_ant;
-        const float4* row1 = row0 + n_ant;
-        #pragma unroll 2
-        for (int qq = lane; qq < n_ant; qq += 32) {
-          const float4 v0 = row0[qq], v1 = row1[qq];
-          float4 j0 = first ? make_float4(1.f, 0.f, 0.f, 0.f) : Jo[qq];
-          float4 j1 = first ? make_float4(0.f, 0.f, 1.f, 0.f) : Jo[n_ant + qq];
-          if (qq == my_p) j0 = j1 = make_float4(0.f, 0.f, 0.f, 0.f);   // C excludes q = p
-          als_terms(v, v0, v1, j0, j1);
-        }
-      }
+      const float4* row0 = rows + (size_t)slot * 2 * n_ant;
+      const float4* row1 = row0 + n_ant;
+      auto iterate = [&](int qq, float4& j0, float4& j1) {
+        j0 = first ? make_float4(1.f, 0.f, 0.f, 0.f) : Jo[qq];
+        j1 = first ? make_float4(0.f, 0.f, 1.f, 0.f) : Jo[n_ant + qq];
+        if (qq == my_p) j0 = j1 = make_float4(0.f, 0.f, 0.f, 0.f);     // C excludes q = p
+      };
       float4 Jn = make_float4(0.f, 0.f, 0.f, 0.f);                 // the row this lane sends
       if (!last) {
-        const float wsum = warp_reduce_scatter16f(v, lane);
+        float v[16];
+        #pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = 0.f;
+        if (live)
+          for (int q0 = lane; q0 < n_ant; q0 += 32 * kClChain) {
+            float w[16];
+            #pragma unroll
+            for (int i = 0; i < 16; ++i) w[i] = 0.f;
+            #pragma unroll
+            for (int u = 0; u < kClChain; ++u) {
+              const int qq = q0 + 32 * u;
+              if (qq >= n_ant) break;
+              float4 j0, j1;
+              iterate(qq, j0, j1);
+              als_terms(w, row0[qq], row1[qq], j0, j1);
+            }
+            #pragma unroll
+            for (int i = 0; i < 12; ++i) v[i] += w[i];
+          }
+        const float wsum = warp_reduce_scatter16c(v, lane);
         // lane L holds the total of value L >> 1: this lane's row of A, and C
         const int at = 8 * (lane & 1);
         const float2 A0 = make_float2(__shfl_sync(0xffffffffu, wsum, at), __shfl_sync(0xffffffffu, wsum, at + 2));
@@ -443,7 +522,16 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_solve(ClusterSolveArg
           }
         }
       } else {
-        const FF wsum = warp_reduce_scatter16ff(v, lane);
+        FF sum[12];
+        #pragma unroll
+        for (int i = 0; i < 12; ++i) sum[i].hi = sum[i].lo = 0.f;
+        if (live)
+          for (int qq = lane; qq < n_ant; qq += 32) {
+            float4 j0, j1;
+            iterate(qq, j0, j1);
+            als_terms_ff(sum, row0[qq], row1[qq], j0, j1);
+          }
+        const FF wsum = warp_reduce_scatter12ff(sum, lane);
         if ((lane & 1) == 0 && (lane >> 1) < 12) s_tot64[slot][lane >> 1] = (double)wsum.hi + (double)wsum.lo;
         __syncthreads();
         // the FP64 solves of all slots, one entry a lane of the first warps
@@ -607,16 +695,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster_als(ClusterAlsArgs a)
         float4 j0 = first ? make_float4(1.f, 0.f, 0.f, 0.f) : Jo[qq];
         float4 j1 = first ? make_float4(0.f, 0.f, 1.f, 0.f) : Jo[n_ant + qq];
         if (qq == my_p) j0 = j1 = make_float4(0.f, 0.f, 0.f, 0.f);   // C excludes q = p
-        float v[16];
-        #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = 0.f;
-        als_terms(v, row0[qq], row1[qq], j0, j1);
-        #pragma unroll
-        for (int i = 0; i < 12; ++i) {
-          const FF t = ff_two_sum(sum[i].hi, v[i]);
-          sum[i].hi = t.hi;
-          sum[i].lo += t.lo;
-        }
+        als_terms_ff(sum, row0[qq], row1[qq], j0, j1);
       }
     const FF wsum = warp_reduce_scatter12ff(sum, lane);
     if ((lane & 1) == 0 && (lane >> 1) < 12) s_tot64[slot][lane >> 1] = (double)wsum.hi + (double)wsum.lo;
