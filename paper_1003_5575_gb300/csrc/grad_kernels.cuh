@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kGsPairWarps ? 2 : 1) k_g
         __syncwarp();
         strip_tables<kGsQh>(tb, p, lane, np, lut);
         __syncwarp();
-        strip_subtract<kGsQh>(R, tb, Mt + (size_t)k0 * kStMRow, min(kStGrp, K - k0), lane);
+        strip_subtract<kGsQh>(R, tb, Mt + (size_t)k0 * kStMRow, 0, min(kStGrp, K - k0), lane);
       }
       __syncwarp();
       strip_planes<kGsQh, kGsPitch>(R, pre, pim, nc, lane);

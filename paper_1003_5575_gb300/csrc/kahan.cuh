@@ -1,6 +1,6 @@
 // Compensated (Kahan) FP32 summation, shared by the prediction and the adjoint.
 #pragma once
-#include <cuda_runtime.h>
+#include "common.cuh"
 
 namespace rts {
 
@@ -9,6 +9,14 @@ __device__ inline void kahan_add(float& sum, float& comp, float x) {
   const float y = x - comp;
   const float t = sum + y;
   comp = (t - sum) - y;
+  sum = t;
+}
+
+// x into sum (two of them, packed); x is left with what the sum's rounding dropped, and
+// the next x is added up on top of it
+__device__ __forceinline__ void kahan_carry2(float2& sum, float2& x) {
+  const float2 neg = make_float2(-1.f, -1.f), t = fadd2(sum, x);
+  x = ffma2(neg, ffma2(neg, sum, t), x);
   sum = t;
 }
 

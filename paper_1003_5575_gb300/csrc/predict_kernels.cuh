@@ -1,7 +1,7 @@
 // Model prediction: vis (+)= sum over a chunk of sources of
-// S_k J_i J_j^H exp(-2 pi i phi_k), one CTA per baseline.  The FP32 sums over
-// sources are Kahan-compensated, so a 1000-source prediction stays within a
-// few ulp of the exact sum.
+// S_k J_i J_j^H exp(-2 pi i phi_k).  The FP32 sums over sources are compensated (term by
+// term in k_predict_mixed, eight terms at a time in k_predict_strip), so a
+// 1000-source prediction stays within a few ulp of the exact sum.
 #pragma once
 #include "stream_kernels.cuh"
 #include "kahan.cuh"
@@ -99,16 +99,20 @@ __global__ void __launch_bounds__(kStreamThreads) k_predict_mixed(PredictArgs a)
 // (baseline, time, 32 QH channels) strip in registers, a launch takes up to
 // kPredictStripSrc sources in two groups.  Against one hardware sin/cos and a
 // compensated sum per (source, channel), about 60 instructions, it issues about
-// 15: phasors as products of table entries, packed multiply-adds, each group
-// of 32 sources summed in FP32 and the two groups and the cube added exactly
-// and rounded once.  Model matrices by float-float products (as their FP64
+// 16: phasors as products of table entries, packed multiply-adds, sums compensated
+// every kPredictSum sources: the remainder of the sum's rounding stays in the
+// registers that the next sources are added up in (three packed operations, no
+// third set of registers).  The cube is added exactly and the result rounded once.
+// Model matrices by float-float products (as their FP64
 // evaluation, rounded to FP32); phases as differences of the antennas' Q0.64
 // phases (k_block_ant_phases).  Bound by instruction issue and the FP32 pipe: 20
 // multiply-adds per source and channel, two an instruction.  100 sources into
-// 128 antennas x 256 channels x 8 times: 1.88 ms, k_predict_mixed 4.01 ms; error
-// against 64 bits 1.8e-7 and 2.0e-7.  Strips of 128 channels (QH = 4): 64 registers
-// hold a group's sum and the one before it.
+// 128 antennas x 256 channels x 8 times: 2.00 ms, k_predict_mixed 4.01 ms; error
+// against 64 bits 1.05e-7 of the rms (largest 0.9e-6) and 1.98e-7 (1.3e-6); with plain sums of
+// 32 sources 1.88 ms, 1.86e-7 and 2.6e-6, compensated every four 2.17 ms.  Strips of 128
+// channels (QH = 4): 64 registers hold the sum and its remainder.
 constexpr int kPredictStripSrc = 2 * kStGrp;
+constexpr int kPredictSum = 8;             // sources whose terms are added in plain FP32
 // Antenna phases a handle keeps for predictions, at most: 1 KB per antenna and time,
 // 4 MB for 512 antennas and 8 times.  Longer cubes (more than 131 072 antenna-times),
 // and handles whose device has no room for them, take k_predict_mixed, which needs none.
@@ -150,11 +154,11 @@ __global__ void __launch_bounds__(kStWarps * 32, 2) k_predict_strip(PredictArgs 
   for (int s = w; s < n_strip; s += g.wpb) {
     const int t = s / n_tile, c0 = (s - t * n_tile) * 32 * QH, nc = min(32 * QH, a.n_chan - c0);
     const int np = (((nc + 15) >> 4) + 1) >> 1;
-    Strip<QH> R, R0;
+    Strip<QH> S, R;                            // the sum is S + R, R what S's rounding left and the present sources
     #pragma unroll
     for (int e = 0; e < 4; ++e)
       #pragma unroll
-      for (int v = 0; v < QH / 2; ++v) R.re[e][v] = R.im[e][v] = R0.re[e][v] = R0.im[e][v] = make_float2(0.f, 0.f);
+      for (int v = 0; v < QH / 2; ++v) S.re[e][v] = S.im[e][v] = R.re[e][v] = R.im[e][v] = make_float2(0.f, 0.f);
     for (int k0 = 0; k0 < a.n_src; k0 += kStGrp) {
       PhaseAB p;
       p.a = 0; p.b = 0;
@@ -164,16 +168,21 @@ __global__ void __launch_bounds__(kStWarps * 32, 2) k_predict_strip(PredictArgs 
         p.b = pi.b - pj.b;
         p.a = pi.a - pj.a + (unsigned long long)c0 * p.b;
       }
-      if (k0) R0 = R;
-      if (k0)
-        #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          #pragma unroll
-          for (int v = 0; v < QH / 2; ++v) R.re[e][v] = R.im[e][v] = make_float2(0.f, 0.f);
       __syncwarp();
       strip_tables<QH>(tb, p, lane, np, lut);
       __syncwarp();
-      strip_subtract<QH>(R, tb, Mt + ((size_t)lb * kPredictStripSrc + k0) * kStMRow, min(kStGrp, a.n_src - k0), lane);
+      const int n_grp = min(kStGrp, a.n_src - k0);
+      #pragma unroll 1
+      for (int k1 = 0; k1 < n_grp; k1 += kPredictSum) {
+        strip_subtract<QH>(R, tb, Mt + ((size_t)lb * kPredictStripSrc + k0) * kStMRow, k1, min(k1 + kPredictSum, n_grp), lane);
+        #pragma unroll
+        for (int e = 0; e < 4; ++e)
+          #pragma unroll
+          for (int v = 0; v < QH / 2; ++v) {
+            kahan_carry2(S.re[e][v], R.re[e][v]);
+            kahan_carry2(S.im[e][v], R.im[e][v]);
+          }
+      }
     }
     float4* vis = static_cast<float4*>(a.vis) + (((size_t)t * a.n_bl + bl) * a.n_chan + c0) * 2;
     const int cl = 16 * (lane >> 4) * QH + (lane & 15);
@@ -181,19 +190,19 @@ __global__ void __launch_bounds__(kStWarps * 32, 2) k_predict_strip(PredictArgs 
     for (int u = 0; u < QH; ++u) {
       const int c = cl + 16 * u;
       if (c >= nc) continue;
-      float re[4], im[4], re0[4], im0[4];
-      strip_channel(R, u, re, im);
-      strip_channel(R0, u, re0, im0);
+      float re[4], im[4], lr[4], li[4];
+      strip_channel(S, u, re, im);
+      strip_channel(R, u, lr, li);
       float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
       if (a.accumulate) { x0 = __ldcs(vis + 2 * c); x1 = __ldcs(vis + 2 * c + 1); }
-      auto sum = [](float x, float p, float q) {           // x + p + q, rounded once
-        const FF s = ff_two_sum(p, q), o = ff_two_sum(x, s.hi);
-        return o.hi + (o.lo + s.lo);
+      auto sum = [](float x, float s, float r) {           // x + s + r, rounded once
+        const FF o = ff_two_sum(x, s);
+        return o.hi + (o.lo + r);
       };
-      __stcs(vis + 2 * c, make_float4(sum(x0.x, re0[0], re[0]), sum(x0.y, im0[0], im[0]), sum(x0.z, re0[1], re[1]),
-                                     sum(x0.w, im0[1], im[1])));
-      __stcs(vis + 2 * c + 1, make_float4(sum(x1.x, re0[2], re[2]), sum(x1.y, im0[2], im[2]),
-                                         sum(x1.z, re0[3], re[3]), sum(x1.w, im0[3], im[3])));
+      __stcs(vis + 2 * c, make_float4(sum(x0.x, re[0], lr[0]), sum(x0.y, im[0], li[0]), sum(x0.z, re[1], lr[1]),
+                                     sum(x0.w, im[1], li[1])));
+      __stcs(vis + 2 * c + 1, make_float4(sum(x1.x, re[2], lr[2]), sum(x1.y, im[2], li[2]), sum(x1.z, re[3], lr[3]),
+                                         sum(x1.w, im[3], li[3])));
     }
   }
 }

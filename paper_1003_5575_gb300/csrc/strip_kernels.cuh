@@ -118,14 +118,14 @@ __device__ __forceinline__ float2 model_entry_ff(float4 a, float4 b, float Sh, f
   return make_float2(scale(re), scale(im));
 }
 
-// R -= sum_{k < n} M_k conj(P_k), M packed [n][kStMRow]
-template <int QH>
+// R -= sum_{k0 <= k < k1} M_k conj(P_k), M packed [][kStMRow]; kUnroll: sources whose
+// loads are in flight together
+template <int QH, int kUnroll = QH < 8 ? 2 : 1>
 __device__ __forceinline__ void strip_subtract(Strip<QH>& R, const StripTables<QH>& tb, const float4* __restrict__ Mt,
-                                               int n, int lane) {
-  constexpr int kUnroll = QH < 8 ? 2 : 1;      // two sources' loads in flight where registers allow
+                                               int k0, int k1, int lane) {
   const int r = lane & 15, v0 = (lane >> 4) * (QH / 2);
   #pragma unroll kUnroll
-  for (int k = 0; k < n; ++k) {
+  for (int k = k0; k < k1; ++k) {
     float4 m4[kStMRow];
     #pragma unroll
     for (int i = 0; i < kStMRow; ++i) m4[i] = Mt[k * kStMRow + i];
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kStWarps * 32, 2) k_block_pass_strip(BlockPass
             __syncwarp();
             strip_tables<QH>(tb, p, lane, np, lut);
             __syncwarp();
-            strip_subtract<QH>(R, tb, Mt + ((size_t)lb * kBlkMax + k0) * kStMRow, min(kStGrp, a.n_sub - k0), lane);
+            strip_subtract<QH>(R, tb, Mt + ((size_t)lb * kBlkMax + k0) * kStMRow, 0, min(kStGrp, a.n_sub - k0), lane);
           }
           strip_store(R, a.dst + strip, a.n_chan, lane);
           __syncwarp();
