@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == kGsPairWarps ? 2 : 1) k_g
       }
     }
   }
-  double l = (double)loss.hi + (double)loss.lo;
+  double l = isfinite(loss.hi) ? (double)loss.hi + (double)loss.lo : (double)loss.hi;     // lo of an infinite sum is no number
   for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
   if (lane == 0) s_loss[warp] = l;
   __syncthreads();

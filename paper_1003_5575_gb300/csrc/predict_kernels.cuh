@@ -195,9 +195,9 @@ __global__ void __launch_bounds__(kStWarps * 32, 2) k_predict_strip(PredictArgs 
       strip_channel(R, u, lr, li);
       float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
       if (a.accumulate) { x0 = __ldcs(vis + 2 * c); x1 = __ldcs(vis + 2 * c + 1); }
-      auto sum = [](float x, float s, float r) {           // x + s + r, rounded once
+      auto sum = [](float x, float s, float r) {           // x + s + r, rounded once (an infinite x stays one)
         const FF o = ff_two_sum(x, s);
-        return o.hi + (o.lo + r);
+        return isfinite(o.hi) ? o.hi + (o.lo + r) : o.hi;
       };
       __stcs(vis + 2 * c, make_float4(sum(x0.x, re[0], lr[0]), sum(x0.y, im[0], li[0]), sum(x0.z, re[1], lr[1]),
                                      sum(x0.w, im[1], li[1])));
