@@ -326,8 +326,10 @@ __global__ void __launch_bounds__(1024, 1) k_grid_gather(GridGatherArgs a) {
     #pragma unroll 2
     for (int h = 0; h < n; ++h) {
       const float2 p = s_pos[h];
-      const float dx = fx - p.x, dxx = dx * dx;
-      const float2 dy = fadd2(fy, make_float2(-p.y, -p.y)), d = ffma2(dy, dy, make_float2(dxx, dxx));
+      // squared distances rounded as the box test below rounds them: a pixel inside the
+      // radius is never outside it for its tile
+      const float dx = fx - p.x;
+      const float2 dx2 = make_float2(dx, dx), dy = fadd2(fy, make_float2(-p.y, -p.y)), d = ffma2(dx2, dx2, fmul2(dy, dy));
       // table position; its integer part by a round-down addition of 2^23
       float2 at = fmul2(make_float2(grid_sqrt(d.x), grid_sqrt(d.y)), make_float2(a.tab_scale, a.tab_scale));
       at = make_float2(fminf(at.x, last), fminf(at.y, last));
