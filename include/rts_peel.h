@@ -38,8 +38,9 @@
  * _predict, _rotate_average and _solve allocate nothing.  Two workspaces whose
  * size depends on how the handle is used are allocated on first use and kept:
  * the adjoint's (first rts_peel_grad or rts_peel_offsets: 88 bytes per
- * baseline and, in RTS_PREC_MIXED, 16 bytes per antenna and time for each of
- * max_sources sources) and the pipeline's two
+ * baseline for each of max_sources sources and, for RTS_GRAD_AUTO in
+ * RTS_PREC_MIXED, 16 bytes per antenna and time for each of up to 1600 of them;
+ * where there is no room for the latter the adjoint goes as RTS_GRAD_DIRECT) and the pipeline's two
  * device cubes and page-locked staging (first rts_peel_pipeline_submit); a
  * warm-up call before real-time use moves that allocation out of the loop.  Calls are asynchronous on `stream` (a cudaStream_t, NULL
  * = legacy default stream) unless an h_status pointer is given, which makes

@@ -21,6 +21,7 @@
 // Kernels 2-4 reduce those per antenna / per source / for the loss in a fixed
 // order, so the result is deterministic (no atomics).
 #pragma once
+#include <algorithm>
 #include <string>
 #include <type_traits>
 
@@ -44,7 +45,8 @@ struct GradWorkspace {
   double* gsc = nullptr;    // [K][n_bl][3] (dl, dm, dS contributions)
   double* loss_bl = nullptr;// [n_bl]
   DirQ* dir = nullptr;   // [K] (l, m, nm1, S)
-  PhaseAB* aph = nullptr;   // [n_time][n_ant][kp] antenna phases (FP32 sweep), kp = K rounded up to 32
+  PhaseAB* aph = nullptr;   // [n_time][n_ant][kp] antenna phases (k_grad_strip), kp = K rounded up to 32
+  int aph_src = 0;          // kp, at most (0: no room for them, or never used)
   float4* lmn = nullptr;    // [kp] l / n and m / n, each as a pair of floats
   double* wchan = nullptr;  // [n_chan] per-channel weight of the position derivative (offsets)
 };
@@ -299,6 +301,9 @@ constexpr size_t kGsPairSmem = 112 * 1024;
 // totals leave shared memory to make room for the second; at 100 sources two CTAs,
 // the sharing of the last group and k_grad_jones's reduction took 4.57 ms to 3.56
 constexpr int kGsVals = 10;               // per source: G (8), l, m
+// No more sources fit (64 bytes of models a source in 112 KB for one of two CTAs, 144 with
+// the totals in 225 KB): the antenna phases are kept for no more
+constexpr int kGsMaxSrc = 1600;
 
 __host__ __device__ inline int grad_kp(int n_src) { return (n_src + kStGrp - 1) / kStGrp * kStGrp; }
 template <bool WEIGHTED> __host__ __device__ constexpr size_t grad_strip_warp_bytes() {
@@ -693,9 +698,11 @@ inline int grad_fail(std::string& err, cudaError_t e, const char* what) {
 }
 
 // Allocates its workspace on first use (G and per-baseline terms for up to
-// max_src sources: (64 + 24) bytes per source and baseline, and for the FP32
-// sweep 16 bytes per source, antenna and time) and keeps it.
-inline int grad_prepare(GradWorkspace& w, bool mixed, int n_src, const double* src, int n_ant, int n_time,
+// max_src sources: (64 + 24) bytes per source and baseline, and with strip
+// 16 bytes per antenna, time and source of up to kGsMaxSrc) and keeps it.
+// strip: the handle's sweep may be k_grad_strip; without room for its phases it is
+// k_grad_sweep, which needs none.
+inline int grad_prepare(GradWorkspace& w, bool strip, int n_src, const double* src, int n_ant, int n_time,
                         int64_t n_bl, int max_src, cudaStream_t s, std::string& err) {
   cudaError_t e;
   if (!w.loss_bl) {
@@ -704,7 +711,7 @@ inline int grad_prepare(GradWorkspace& w, bool mixed, int n_src, const double* s
     auto room = [&](auto kernel) {
       return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradMaxSmem - 1024) != cudaSuccess;
     };
-    if (mixed && (room(k_grad_strip<false, kGsPairWarps, true>) || room(k_grad_strip<false, kGsPairWarps, false>) ||
+    if (strip && (room(k_grad_strip<false, kGsPairWarps, true>) || room(k_grad_strip<false, kGsPairWarps, false>) ||
                   room(k_grad_strip<false, kGsMaxWarps, true>) || room(k_grad_strip<true, kGsPairWarps, true>) ||
                   room(k_grad_strip<true, kGsPairWarps, false>) || room(k_grad_strip<true, kGsMaxWarps, true>)))
       return grad_fail(err, cudaGetLastError(), "cudaFuncSetAttribute");
@@ -713,11 +720,18 @@ inline int grad_prepare(GradWorkspace& w, bool mixed, int n_src, const double* s
         (e = cudaMalloc(&w.loss_bl, (size_t)n_bl * sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&w.dir, (size_t)max_src * sizeof(DirQ))) != cudaSuccess ||
         (e = cudaMalloc(&w.lmn, (size_t)grad_kp(max_src) * sizeof(float4))) != cudaSuccess ||
-        (e = cudaMemsetAsync(w.lmn, 0, (size_t)grad_kp(max_src) * sizeof(float4), s)) != cudaSuccess ||
-        (mixed && (e = cudaMalloc(&w.aph, (size_t)n_time * n_ant * grad_kp(max_src) * sizeof(PhaseAB))) != cudaSuccess)) {
+        (e = cudaMemsetAsync(w.lmn, 0, (size_t)grad_kp(max_src) * sizeof(float4), s)) != cudaSuccess) {
       int rc = grad_fail(err, e, "cudaMalloc(gradient workspace)");
       grad_free(w);
       return rc;
+    }
+    if (strip) {
+      w.aph_src = std::min(grad_kp(max_src), kGsMaxSrc);
+      if (cudaMalloc(&w.aph, (size_t)n_time * n_ant * w.aph_src * sizeof(PhaseAB)) != cudaSuccess) {
+        cudaGetLastError();
+        w.aph = nullptr;
+        w.aph_src = 0;
+      }
     }
   }
   if (n_src > 0) k_grad_dirs<<<(n_src + 127) / 128, 128, 0, s>>>(src, n_src, w.dir, w.lmn);
@@ -744,7 +758,7 @@ inline int grad_sweep(GradWorkspace& w, bool mixed, const void* vis, int n_src, 
   a.G = w.G; a.gsc = w.gsc; a.loss_bl = w.loss_bl;
   a.n_src = n_src; a.n_ant = n_ant; a.n_chan = n_chan; a.n_time = n_time; a.n_bl = n_bl;
   a.nu0_c = nu0_c; a.dnu_c = dnu_c;
-  if (mixed && !direct) {
+  if (mixed && !direct && w.aph && grad_kp(n_src) <= w.aph_src) {
     // two CTAs an SM where they have more warps than one, with the totals in shared
     // memory if that leaves them all of their warps
     auto fit = [&](int most, size_t room, bool tot) {
@@ -759,14 +773,10 @@ inline int grad_sweep(GradWorkspace& w, bool mixed, const void* vis, int n_src, 
       const size_t smem = wchan ? grad_strip_smem<true>(n_src, warps, tot) : grad_strip_smem<false>(n_src, warps, tot);
       if (n_src > 0)
         k_grad_ant_phases<<<1024, 256, 0, s>>>(w.dir, n_src, grad_kp(n_src), uvw, n_ant, n_time, nu0_c, dnu_c, w.aph);
-      auto launch = [&](auto kernel) -> cudaError_t {
-        kernel<<<(unsigned)n_bl, 32 * warps, smem, s>>>(a, w.aph, w.lmn);
-        return cudaSuccess;
-      };
-      if (!pair) e = wchan ? launch(k_grad_strip<true, kGsMaxWarps, true>) : launch(k_grad_strip<false, kGsMaxWarps, true>);
-      else if (tot) e = wchan ? launch(k_grad_strip<true, kGsPairWarps, true>) : launch(k_grad_strip<false, kGsPairWarps, true>);
-      else e = wchan ? launch(k_grad_strip<true, kGsPairWarps, false>) : launch(k_grad_strip<false, kGsPairWarps, false>);
-      if (e != cudaSuccess) return grad_fail(err, e, "cudaFuncSetAttribute");
+      auto launch = [&](auto kernel) { kernel<<<(unsigned)n_bl, 32 * warps, smem, s>>>(a, w.aph, w.lmn); };
+      if (!pair) wchan ? launch(k_grad_strip<true, kGsMaxWarps, true>) : launch(k_grad_strip<false, kGsMaxWarps, true>);
+      else if (tot) wchan ? launch(k_grad_strip<true, kGsPairWarps, true>) : launch(k_grad_strip<false, kGsPairWarps, true>);
+      else wchan ? launch(k_grad_strip<true, kGsPairWarps, false>) : launch(k_grad_strip<false, kGsPairWarps, false>);
       if ((e = cudaGetLastError()) != cudaSuccess) return grad_fail(err, e, "gradient sweep launch");
       return 0;
     }

@@ -1668,7 +1668,7 @@ int rts_peel_grad(rts_peel_t* h, const void* d_vis, int32_t n_src, const void* d
   if (n_src > 0 && (!d_jones || !d_src)) return fail(h, RTS_EINVAL, "d_jones and d_src are required");
   cudaStream_t s = as_stream(stream);
   const bool mixed = h->precision == RTS_PREC_MIXED;
-  int rc = grad_prepare(h->grad, h->precision == RTS_PREC_MIXED, n_src, d_src, h->n_ant, h->n_time, h->n_bl,
+  int rc = grad_prepare(h->grad, mixed && !h->grad_direct, n_src, d_src, h->n_ant, h->n_time, h->n_bl,
                         h->max_sources, s, h->err);
   if (rc) return rc;
   {
@@ -1700,7 +1700,7 @@ int rts_peel_offsets(rts_peel_t* h, const void* d_vis, int32_t n_src, const void
   if (misaligned(d_vis)) return fail(h, RTS_EINVAL, "d_vis must start on a 16-byte boundary");
   cudaStream_t s = as_stream(stream);
   const bool mixed = h->precision == RTS_PREC_MIXED;
-  int rc = grad_prepare(h->grad, h->precision == RTS_PREC_MIXED, n_src, d_src, h->n_ant, h->n_time, h->n_bl,
+  int rc = grad_prepare(h->grad, mixed && !h->grad_direct, n_src, d_src, h->n_ant, h->n_time, h->n_bl,
                         h->max_sources, s, h->err);
   if (rc) return rc;
   const double* wtab = h->d_freq_c;              // alpha = 0: w_c = nu_c / c
