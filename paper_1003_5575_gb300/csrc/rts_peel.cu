@@ -1114,7 +1114,8 @@ int peel_taylor_blocked(rts_peel_t* h, const void* d_vis, void* d_resid, int32_t
       const int k = s0 + q;
       {
         Span span(h, RTS_K_BLOCK_FIX, s);
-        k_taylor_correct<<<dim3((unsigned)((h->n_bl + 127) / 128), 3), 128, 0, s>>>(h->b_avg, q, h->b_model, Dt, h->n_bl, h->t_mom);
+        k_taylor_correct<<<(unsigned)((2 * h->n_bl + kTayCorrThreads - 1) / kTayCorrThreads), kTayCorrThreads, 0, s>>>(
+            h->b_avg, q, h->b_model, Dt, h->n_bl, h->t_mom);
         span.end(1);
       }
       rc = launch_als_taylor(h, src[3 * k + 2], static_cast<float2*>(d_gain) + k * jstride,

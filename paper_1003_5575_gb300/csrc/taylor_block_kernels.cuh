@@ -148,37 +148,49 @@ __global__ void __launch_bounds__(256) k_block_dirichlet_taylor(const PhaseAB* _
   }
 }
 
-// corrected moments of source q of a Taylor block, one thread per (baseline, moment n):
+// corrected moments of source q of a Taylor block, two threads a baseline, each two
+// of the four entries of all three moments:
 //   mom[n][bl] = Ablk[3q + n][bl] - sum_{j<q} sum_m P[3j + m][bl] D^(n+m)_jq
-// (a thread per baseline took 21 us a source at 128 antennas, too few loads in
-// flight; this takes 13)
-__global__ void __launch_bounds__(128) k_taylor_correct(const float2* __restrict__ Ablk, int q,
+// Every model word is read once (up to 250 MB a block at 512 antennas, twice the L2), and
+// four sources' loads are in flight.  Corrections, models and geometry of 63 sources
+// at 512 / 256 / 50 at 128 antennas: 3.50 / 1.56 / 1.13 ms; with a thread a baseline 3.81 /
+// 2.05 / 1.44 (too few loads in flight), with a thread a baseline and moment, whose three
+// sweeps read the models three times, 5.49 / 1.78 / 1.14.
+constexpr int kTayCorrThreads = 128;
+__global__ void __launch_bounds__(kTayCorrThreads) k_taylor_correct(const float2* __restrict__ Ablk, int q,
                                                        const float2* __restrict__ P,
                                                        const float2* __restrict__ Dt, int64_t n_bl,
                                                        float2* __restrict__ mom) {
-  const int64_t bl = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int n = blockIdx.y;
-  if (bl >= n_bl) return;
-  const float4* A = reinterpret_cast<const float4*>(Ablk + ((size_t)(3 * q + n) * n_bl + bl) * 4);
-  const float4 a0 = A[0], a1 = A[1];
-  float2 v[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y), make_float2(a1.z, a1.w)};
-  const float2* D = Dt + ((size_t)bl * kTayPairs + q * (q - 1) / 2) * 5 + n;
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;     // (baseline, half)
+  if (idx >= 2 * n_bl) return;
+  const float4* A = reinterpret_cast<const float4*>(Ablk) + (size_t)3 * q * n_bl * 2 + idx;
+  float2 v[3][2];
+  #pragma unroll
+  for (int n = 0; n < 3; ++n) {
+    const float4 a = A[(size_t)n * n_bl * 2];
+    v[n][0] = make_float2(a.x, a.y);
+    v[n][1] = make_float2(a.z, a.w);
+  }
+  const float2* D = Dt + ((size_t)(idx >> 1) * kTayPairs + q * (q - 1) / 2) * 5;
+  const float4* P4 = reinterpret_cast<const float4*>(P) + idx;
   #pragma unroll 4
   for (int j = 0; j < q; ++j) {
+    float2 d[5];
+    #pragma unroll
+    for (int p = 0; p < 5; ++p) d[p] = __ldg(D + 5 * j + p);
     #pragma unroll
     for (int m = 0; m < 3; ++m) {
-      const float4* P4 = reinterpret_cast<const float4*>(P + ((size_t)(3 * j + m) * n_bl + bl) * 4);
-      const float4 p0 = __ldg(P4), p1 = __ldg(P4 + 1);
-      const float2 d = __ldg(D + 5 * j + m);
-      v[0] = csub(v[0], cmul(make_float2(p0.x, p0.y), d));
-      v[1] = csub(v[1], cmul(make_float2(p0.z, p0.w), d));
-      v[2] = csub(v[2], cmul(make_float2(p1.x, p1.y), d));
-      v[3] = csub(v[3], cmul(make_float2(p1.z, p1.w), d));
+      const float4 p = __ldg(P4 + (size_t)(3 * j + m) * n_bl * 2);
+      #pragma unroll
+      for (int n = 0; n < 3; ++n) {
+        v[n][0] = csub(v[n][0], cmul(make_float2(p.x, p.y), d[n + m]));
+        v[n][1] = csub(v[n][1], cmul(make_float2(p.z, p.w), d[n + m]));
+      }
     }
   }
-  float4* o = reinterpret_cast<float4*>(mom + ((size_t)n * n_bl + bl) * 4);
-  o[0] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
-  o[1] = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
+  float4* o = reinterpret_cast<float4*>(mom) + idx;
+  #pragma unroll
+  for (int n = 0; n < 3; ++n) o[(size_t)n * n_bl * 2] = make_float4(v[n][0].x, v[n][0].y, v[n][1].x, v[n][1].y);
 }
 
 // P0, P1, P2 of a solved Taylor source into slots 3q .. 3q + 2 of the block's
