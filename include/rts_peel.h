@@ -400,7 +400,8 @@ int rts_peel_timing_read(rts_peel_t* h, double* ms, int64_t* groups, int64_t* la
  * for benchmarks and tests).  *block_kernel: 0 when the handle peels one source
  * per pass, else RTS_BLOCK_FMA, RTS_BLOCK_TENSOR or RTS_BLOCK_TCGEN05 (the
  * choice RTS_BLOCK_AUTO made).  *solve_kernel: RTS_SOLVE_AUTO when the blocked
- * peel solves each block in one cooperative launch, else RTS_SOLVE_LAUNCHES.
+ * peel's solves are those of RTS_SOLVE_AUTO (clusters up to 256 antennas, one
+ * cooperative launch a block above that), else RTS_SOLVE_LAUNCHES.
  * Either pointer may be NULL.  RTS_EINVAL for a NULL handle. */
 int rts_peel_kernels(const rts_peel_t* h, int32_t* block_kernel, int32_t* solve_kernel);
 
