@@ -368,7 +368,7 @@ int read_status(rts_peel_t* h, int32_t n, int32_t* h_status, cudaStream_t s) {
   if (h->status_in[0]) return fail(h, RTS_ECUDA, "a tensor-core completion wait of the blocked pass timed out");
   for (int k = 0; k < n; ++k)
     if (h_status[k] == kSolveStatusTimeout)
-      return fail(h, RTS_ECUDA, "a grid barrier of the block solve timed out at source " + std::to_string(k));
+      return fail(h, RTS_ECUDA, "a wait between the CTAs of a solve timed out at source " + std::to_string(k));
   for (int k = 0; k < n; ++k)
     if (h_status[k] == RTS_ENONFINITE)
       return fail(h, RTS_ENONFINITE, "non-finite value in the solve of source " + std::to_string(k));
