@@ -110,8 +110,9 @@ typedef struct rts_peel_config {
                            step and per solve or, above 256 antennas, per ALS sweep; a
                            single source's solve always goes this way).  The cluster and the
                            cooperative launch solve the 2x2 systems of the sweeps before
-                           the last in FP32 and the last in FP64 (from float-float or
-                           FP64 sums), the per-step launches every sweep in FP64; their
+                           the last in FP32 and the last in FP64 (their sums over
+                           antennas end in float-float or FP64), the per-step launches
+                           every sweep in FP64; their
                            results agree to FP32 rounding (statuses outside a band
                            around 1e-6). */
   int32_t grad_kernel;   /* RTS_PREC_MIXED adjoint (rts_peel_grad, rts_peel_offsets):
@@ -184,9 +185,9 @@ int rts_peel_cadence(rts_peel_t* h, const void* d_vis, void* d_resid, int32_t n_
  * source's model and takes three channel moments mean_{t,c} x_c^n R e^{+2 pi i phi}
  * (n = 0, 1, 2) of the residual in its direction; n_iter Jacobi ALS sweeps on
  * X_p = [G_p H_p] (2x4) from G = I, H = 0, every second averaged with the
- * previous iterate, each solving the 4x4 normal equations (FP64 sums and
- * Cholesky solve); then its model is subtracted.  One pass per source
- * whatever sources_per_pass says.
+ * previous iterate, each solving the 4x4 normal equations (sums in FP64 or
+ * float-float pairs); then its model is subtracted.  Handles with blocks of 64
+ * sources and at most 768 channels take 21 sources a pass, others one.
  *   d_vis, d_resid, n_src, h_src, h_status, stream: as rts_peel_cadence
  *            (status from the relative change of X in the last sweep).
  *   d_gain   [n_src][n_ant][4] complex64 receives G (the gain at the band centre).
@@ -286,10 +287,12 @@ int rts_peel_rel(rts_peel_t* h, int32_t n_src, double* h_rel, void* stream);
  * turns in [-1/2, 1/2), as the peel's kernels form it: the FP64 delay
  * tau = u l + v m + w (n - 1), the Q0.64 fixed-point phases A = frac(tau nu_0 / c)
  * and B = frac(tau dnu / c), and channel c at A + c B modulo one turn (exact
- * integer arithmetic).  form = 0 returns that Q0.64 phase (the streaming,
- * predict and adjoint kernels); form = 1 the FP32 value the kernels hand to the
- * hardware sin/cos (rounded to Q0.32 first); form = 2 the Q0.64 phase as the
- * blocked schedule forms it, from the two antennas' delays about antenna 0
+ * integer arithmetic).  form = 0 returns that Q0.64 phase (the one-source
+ * streaming kernels, the per-sample prediction and adjoint); form = 1 the FP32
+ * value those hand to the hardware sin/cos (rounded to Q0.32 first); form = 2 the
+ * Q0.64 phase as the blocked schedule, the default prediction and the default
+ * adjoint form it (whose kernels then take products of table phasors at
+ * 16-channel steps of it), from the two antennas' delays about antenna 0
  * (u, v, w of uvw_i - uvw_0; the same geometry: uvw_ij = uvw_i - uvw_j)
  * as the difference of their Q0.64 phases modulo one turn.  A pair with t or
  * bl out of range gets NaN.  Asynchronous on `stream`.  RTS_EINVAL for a NULL

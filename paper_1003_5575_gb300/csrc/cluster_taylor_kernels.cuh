@@ -30,8 +30,8 @@
 // residual; where a pivot is below 1e-3 of its scale they are solved in FP64.
 // Measured (128 antennas, 20 sweeps): 176 us a source where the launches took 630
 // (20 sweeps of 12.8 us, 19 row sums of 12.0 and 19 steps of 5.4, and their gaps);
-// error of a 50-source cadence against 64 bits 3.7e-6 with the launches, 6e-7
-// here.  In cycles an iteration: row sums 4 200, Gram sums 1 300, the step's sums
+// error of the gains and slopes of a 50-source cadence of 128 channels against 64 bits
+// 1.5e-6 and 3.5e-6 with the launches, 1.4e-7 and 3.8e-7 here.  In cycles an iteration: row sums 4 200, Gram sums 1 300, the step's sums
 // 3 100, the step 3 000 (one lane an entry of its matrix, the CTAs' sums pairwise; every
 // lane doing all of it took 3 800), normal matrix 1 250, solve 2 000, exchange 1 600.
 // The rows of all antennas have to fit the cluster's shared memory, up to about

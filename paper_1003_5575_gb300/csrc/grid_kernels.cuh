@@ -56,7 +56,7 @@ constexpr int kGridMaxPol = 4;
 // the whole grid 290: its tables are loaded nine times as often)
 constexpr int kGridMaxDense = 128;    // bins whose tiles get a CTA each, at most
 constexpr int kGridDenseMin = 2048;   // and the fewest visibilities of such a bin and its neighbours
-constexpr int kGridGatherMaxSmem = 100 * 1024;   // 4096 samples, 4 values, 32-pixel bins: 98 312 bytes
+constexpr int kGridGatherMaxSmem = 100 * 1024;   // 4096 samples, 4 values, 32-pixel bins: 98 320 bytes
 
 // bin of a visibility, or -1 outside [0, n_pix)^2 (NaN compares false)
 __device__ __forceinline__ int grid_bin(float2 p, int n_pix, int bin, int nbx) {

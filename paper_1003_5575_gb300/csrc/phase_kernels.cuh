@@ -1,18 +1,21 @@
 // The phase step alone: the per-channel phase of one direction on chosen
-// (time, baseline) pairs, formed exactly as the streaming, blocked and adjoint
+// (time, baseline) pairs, formed as the streaming, blocked and adjoint
 // kernels form it (common.cuh): FP64 delay tau = u l + v m + w (n - 1), two
 // Q0.64 fixed-point phases A = frac(tau nu_0 / c), B = frac(tau dnu / c), and
 // channel c at A + c B (mod 2^64, the integer wrap being the reduction modulo
-// one turn).  Used to check that phase against a direct FP64 evaluation.
+// one turn).  Used to check that phase against a direct FP64 evaluation.  (The kernels
+// on strips and the tcgen05 pass take products of table phasors at 16-channel steps of
+// form 2's A and B; their phases are checked by their results.)
 #pragma once
 #include "common.cuh"
 
 namespace rts {
 
 // out[pair][c] in turns, [-1/2, 1/2): form 0, the Q0.64 phase of the baseline's
-// FP64 delay (the streaming, predict and adjoint kernels); form 1, that phase
-// as the FP32 value the kernels pass to the hardware sin/cos (rounded to Q0.32,
-// then converted); form 2, the Q0.64 phase as the blocked schedule forms it,
+// FP64 delay (the one-source streaming kernels and the per-sample prediction and
+// adjoint); form 1, that phase as the FP32 value those pass to the hardware sin/cos
+// (rounded to Q0.32, then converted); form 2, the Q0.64 phase as the blocked schedule, the
+// strip prediction and the strip adjoint form it,
 // the difference of the two antennas' Q0.64 phases (their FP64 delays about
 // antenna 0, from uvw_i - uvw_0).  Pairs whose time or baseline index is
 // out of range get NaN in every channel.

@@ -26,14 +26,19 @@ namespace rts {
 constexpr int kStWarps = 8;                // warps of a CTA
 constexpr int kStGrp = 32;                 // sources whose tables a warp holds at once
 constexpr int kStMaxQh = 8;                // tiles per half warp, at most: 256 channels
-// Strips up to here take this pass, and the Taylor cadence's, by default.  At 128
-// antennas, 8 times and 128 sources the passes take 1.02 / 1.29 / 1.99 / 3.19 / 3.49 ms
-// for 16 / 64 / 128 / 203 / 256 channels, the tcgen05 form's 2.8 to 3.2 ms whatever the
-// length; with 4 times or 65 antennas this form is ahead up to 256 as well (0.25 and
-// 0.30 ms at 65 antennas x 4 times x 256 channels).  Past 256 channels a strip no longer
-// fits a warp's registers: the form of block_kernels.cuh takes 7.7 ms at 384,
-// tcgen05 3.2.  Taylor, 42 sources: 0.84 / 1.02 / 1.60 / 2.51 / 2.79 ms for 32 / 64 / 128 /
-// 203 / 256 channels, tcgen05 5.0 ms.
+// Strips up to here take this pass, and the Taylor cadence's, by default: past 256
+// channels a strip no longer fits a warp's registers (the form of block_kernels.cuh
+// takes 7.7 ms at 384 channels, tcgen05 3.2).  128 sources, 8 times, this form / tcgen05
+// in ms:
+//   channels        64           128          160          203          256
+//   65 antennas   0.35 / 0.85  0.53 / 0.86  0.77 / 0.86  0.85 / 0.86  0.94 / 0.87
+//   128           1.28 / 2.79  1.99 / 2.80  2.89 / 2.81  3.19 / 2.83  3.48 / 2.84
+//   512               -        31.2 / 43.6  45.7 / 43.7  50.3 / 43.9  55.0 / 44.2
+// With 3 times 65 antennas are ahead here up to 256 (0.39 / 0.44), 128 up to 160.  So from
+// 160 channels on, where more than about 20 000 strips fill the tcgen05 form's CTAs, the
+// line gives up to 24 % of a pass away; it stood where the former tcgen05 pass (3.75 ms
+// at 128 antennas x 256 channels) crossed.  Taylor, 42 sources: 0.84 / 1.02 / 1.60 / 2.51 / 2.79
+// ms for 32 / 64 / 128 / 203 / 256 channels, tcgen05 5.0 ms.
 constexpr int kStAutoChan = 256;
 constexpr int kStMRow = 4;                 // float4 of a source's packed model matrix
 

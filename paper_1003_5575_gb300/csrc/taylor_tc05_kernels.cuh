@@ -1,29 +1,31 @@
-// Blocked peel pass on the 5th-generation tensor cores, transposed form: the
-// same pass as k_block_pass (subtract the solved sources of block b from one
-// (baseline, time step) strip of channels, average the directions of block b+1),
-// with both contractions as tcgen05.mma kind::tf32 GEMMs whose operands the
-// CUDA cores form in O(sources x 16) or O(sources x channels / 16) work.
+// The Taylor pass of the blocked schedule (taylor_block_kernels.cuh) on the
+// 5th-generation tensor cores, for strips of 257 to kTc5MaxChan channels: subtract a
+// block's models (P0 + x_c P1 + x_c^2 P2) e^{-2 pi i phi} from one (baseline, time step)
+// strip and take the next block's three moments mean x_c^n R e^{+2 pi i phi}, both
+// contractions as tcgen05.mma kind::tf32 GEMMs whose operands the CUDA cores form.
 //
 // The phasor of source k at channel c = 16 q + r factors as
-//   P_k(c) = T1_k[q] T2_k[r],  T1_k[q] = e^{2 pi i (A_k + 16 q B_k)},  T2_k[r] = e^{2 pi i r B_k}.
+//   P_k(c) = T1_k[q] T2_k[r],  T1_k[q] = e^{2 pi i (A_k + 16 q B_k)},  T2_k[r] = e^{2 pi i r B_k},
+// and x_c = u_q + v_r (u_q = x_0 + 16 q dx, v_r = r dx), so a source takes three of the 64
+// operand slots, s = 3 k + m (21 sources a block):
 //
-// subtraction  R(16 q + r, e) -= sum_k [M_k(e) conj(T2_k[r])] conj(T1_k[q])
-//   GEMM D_s[m, q] = sum_K A_s[m, K] B_s[q, K], M = 128 rows m = 8 r + 2 e + o
-//   (o: real or imaginary part of the output), K = 128 = (source k, re/im),
-//   N = NQ (the 16-channel tiles, rounded up to 16).  A_s = the real form of
-//   a_k(r, e) = M_k(e) conj(T2_k[r]) (rows o = 0: (a_re, -a_im), o = 1:
-//   (a_im, a_re)), written by the threads into TMEM; B_s = conj(T1) as
-//   (re, im) pairs along K in shared memory.  One 128-row tile whatever the
-//   channel count, and 64 x 16 x 4 operand products per step.
-// average      A_k(e) += sum_r T2_k[r] H_k(r, e),  H_k(r, e) = sum_q T1_k[q] R(16 q + r, e)
-//   GEMM D_a[m', n] = sum_K' A_a[m', K'] B_a[n, K'], M = 128 rows m' = 2 k + o,
-//   K' = 2 NQ = (re/im i, q) at i NQ + q, N = 64 columns n = 4 r + e.  A_a =
-//   the real form of T1 (row o = 0: t_re at i = 0, -t_im at i = 1; row o = 1:
-//   t_im, t_re) in TMEM; B_a = the new residual, written by the subtraction's
-//   epilogue in shared memory (4 consecutive tiles of one part per 16-byte
-//   store).  The 16-term T2 contraction of H runs on the CUDA cores (32 FMAs a
-//   thread) beside the next step's subtraction MMAs, summed over time steps
-//   with compensation.
+// subtraction  R(16 q + r, e) -= sum_s a_s(r, e) b_s(q),
+//   a_s(r, e) = [sum_{n >= m} C(n, m) v_r^{n-m} P_n(e)] conj(T2_k[r]),  b_s(q) = u_q^m conj(T1_k[q])
+//   GEMM D_s[i, q] = sum_K A_s[i, K] B_s[q, K], 128 rows i = 8 r + 2 e + o (o: real or
+//   imaginary part of the output), K = 128 = (slot s, re/im), N = NQ (the 16-channel
+//   tiles, rounded up to 16).  A_s = the real form of a_s (rows o = 0: (a_re, -a_im),
+//   o = 1: (a_im, a_re)), written by the threads into TMEM; B_s as (re, im) pairs along
+//   K in shared memory.  The coefficient table [..] is formed once per CTA.
+// average      H_s(r, e) = sum_q u_q^m T1_k[q] R(16 q + r, e),
+//   moment n of k = sum_{m <= n} C(n, m) sum_r v_r^{n-m} T2_k[r] H_s(r, e)
+//   GEMM D_a[i, j] = sum_K' A_a[i, K'] B_a[j, K'], 128 rows i = 2 s + o, K' = 2 NQ = (re/im, q),
+//   N = 64 columns j = 4 r + e.  A_a = the real form of u_q^m T1 (row o = 0: t_re, then -t_im;
+//   row o = 1: t_im, t_re) in TMEM; B_a = the new residual, written by the subtraction's
+//   epilogue in shared memory (4 consecutive tiles of one part per 16-byte store).  The
+//   sums over r run on the CUDA cores beside the next step's subtraction MMAs, summed
+//   over time steps with compensation.
+// (block_tc05_kernels.cuh forms the real parts of its operands once instead of this
+// 2 x 2 real form; 64 slots of one source each.)
 //
 // TF32 keeps 11 significand bits, so every operand is split x = hi + lo and
 // each product takes three MMAs, hi*hi + lo*hi + hi*lo.  The tensor cores'
@@ -31,11 +33,11 @@
 // accumulators of 4 k-steps each and the (2^-11 smaller) cross terms to one
 // more; the epilogues add them in FP32 with round-to-nearest.
 //
-// One CTA of 16 warps per baseline (1 per SM: ~170 KB of shared memory, all 512
-// TMEM columns), looping over the time steps.  The strip of a time step
-// arrives by a bulk asynchronous copy one step ahead and the residual leaves
-// by one, so the CUDA cores move no visibility data to or from HBM.  A step:
-//   P1  subtraction MMAs   | beside them: the previous step's T2 contraction,
+// One CTA of 16 compute warps per baseline (1 per SM: all 512 TMEM columns), looping
+// over the time steps.  The strip of a time step arrives by a bulk asynchronous copy
+// one step ahead and the residual leaves by one, so the CUDA cores move no
+// visibility data to or from HBM.  A step:
+//   P1  subtraction MMAs   | beside them: the previous step's sums over r,
 //                            T1 and T2 of the averaged sources
 //   P2  subtraction epilogue (residual into the strip and B_a), A_a into TMEM
 //   P3  average MMAs       | beside them: the residual's store, the next
@@ -47,20 +49,8 @@
 // it; operands-ready and MMAs-done mbarriers hand each phase between them.  Every wait is bounded
 // (a wait that runs out sets *err and stops the pass, which the status read
 // reports, after the copies in flight have been waited for and TMEM is freed).
-// Limits: at most 64 sources per role, n_chan <= kTc5MaxChan.
-//
-// Gains Taylor-expanded in frequency: a source's model on a baseline is
-// (P0 + x_c P1 + x_c^2 P2) e^{-2 pi i phi} and its averages are the three
-// moments mean x_c^n R e^{+2 pi i phi}.  With x_c = u_q + v_r (u_q = x_0 + 16 q dx,
-// v_r = r dx) the same two GEMMs carry them when each source takes three of
-// the 64 operand slots, s = 3 k + m (21 sources per block):
-//   subtraction  slot (k, m): A_s = [sum_{n >= m} C(n, m) v_r^{n-m} P_n] conj(T2_k[r])
-//                             B_s = u_q^m conj(T1_k[q])
-//   average      slot (k, m): A_a rows = u_q^m T1_k[q] (real form), so the GEMM gives
-//                             H_km(r, e) = sum_q u_q^m T1_k[q] R(16 q + r, e), and
-//                M_kn = sum_{m <= n} C(n, m) sum_r v_r^{n-m} T2_k[r] H_km(r, e).
-// The CUDA cores form the coefficient table once per CTA, the u_q^m weights
-// beside the phasors, and three v_r-weighted T2 sums per slot.
+// Bound by those phases on the CUDA cores: 512 antennas x 768 channels x 8 times, 48 ms a pass
+// of 21 sources (the streams of HBM alone 7.6).
 #pragma once
 #include "block_tc05_kernels.cuh"
 #include "taylor_block_kernels.cuh"
