@@ -28,7 +28,7 @@
 // iterate) in float-float arithmetic (about 47 bits).  The 4x4 systems of the
 // sweep and of the step are solved in FP32 and refined once from a float-float
 // residual; where a pivot is below 1e-3 of its scale they are solved in FP64.
-// Measured (128 antennas, 20 sweeps): 176 us a source where the launches took 630
+// Measured (128 antennas, 20 sweeps): 165 us a source where the launches took 606
 // (20 sweeps of 12.8 us, 19 row sums of 12.0 and 19 steps of 5.4, and their gaps);
 // error of the gains and slopes of a 50-source cadence of 128 channels against 64 bits
 // 1.5e-6 and 3.5e-6 with the launches, 1.4e-7 and 3.8e-7 here.  In cycles an iteration: row sums 4 200, Gram sums 1 300, the step's sums
